@@ -717,7 +717,8 @@ fq_status fq_autotune(int32_t op, const fq_ensemble_desc *ens, int32_t rf_dtype,
  * Volumes are channels-last [n_vol][F][Z][X][32] (X a multiple of 128, or
  * of 32 with Z a multiple of 4), BF16 activations (channels beyond the real
  * ones are 0), FP32 network output.  Convolutions run on the tcgen05 tensor cores (BF16
- * in, FP32 accumulate); weight gradients on the CUDA cores in FP32.
+ * in, FP32 accumulate), weight gradients on the warp-level tensor cores
+ * (BF16 in, FP32 accumulate).
  *
  * Parameters: one device block of fq_cnn_param_bytes() (256-byte aligned),
  * owned by the caller.  FP32 master weights W[layer] [45][32][32] (tap, in,

@@ -22,7 +22,8 @@
 //
 // The data gradient of a layer is the same convolution with the kernel
 // flipped in all three axes and its channel roles swapped; the weight
-// gradient (a reduction over voxels) runs on the CUDA cores in FP32.
+// gradient (a reduction over voxels) runs on the warp-level tensor cores
+// with FP32 accumulators held in registers (wgrad_kernel).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -61,8 +62,29 @@ __host__ __device__ constexpr int tap_dx(int t) { return t % 3 - 1; }
 
 struct ConvDims {
     int N, F, Z, X;
-    int tiles;         // N F (Z / 4) (X / 32)
+    int tiles;         // N F (Z / 4) (X / 32), the per-tap kernel's tiles
+    int zb, xb;        // depth and lateral blocks of a frame, the last one possibly ragged
+    int walk_tiles;    // N zb xb F: tile = column * F + frame
 };
+
+struct Column {
+    int n, z0, x0;
+};
+
+__device__ __forceinline__ Column column_at(const ConvDims &d, int col)
+{
+    Column c;
+    c.x0 = (col % d.xb) * TILE_X;
+    col /= d.xb;
+    c.z0 = (col % d.zb) * TILE_Z;
+    c.n = col / d.zb;
+    return c;
+}
+
+// The tiles of a CTA are a contiguous range; a segment is its part in one
+// column: output frames fa .. fb - 1.
+__device__ __forceinline__ int range_begin(int tiles) { return (int)((int64_t)tiles * blockIdx.x / gridDim.x); }
+__device__ __forceinline__ int range_end(int tiles) { return (int)((int64_t)tiles * (blockIdx.x + 1) / gridDim.x); }
 
 __device__ __forceinline__ void tile_coords(const ConvDims &d, int tile, int &n, int &f, int &z0, int &x0)
 {
@@ -612,77 +634,237 @@ __global__ void sum_parts_kernel(const double *__restrict__ part, int n, int64_t
     if (threadIdx.x == 0) *loss = (float)(s / (double)count);
 }
 
-// Weight gradient partials: dW[t][ci][co] = sum_v x[v + d_t][ci] dy[v][co]
-// over one chunk of voxels per CTA (256 threads, 4 outputs each), FP32.
-constexpr int kWgChunk = 4096;  // voxels per CTA
-constexpr int kWgSub = 64;      // voxels per shared-memory step
+// Weight gradient: dW[t][ci][co] = sum_v x[v + d_t][ci] dy[v][co], a
+// contraction over voxels with 45 x 32 x 32 results, on the warp-level
+// tensor cores (mma.sync m16n8k16, BF16 operands, FP32 accumulators).  A
+// CTA keeps the whole result in registers: warp (dt, dz) holds the three
+// taps dx = -1, 0, 1 (96 accumulators per lane) and walks the CTA's
+// contiguous range of tiles (4 depth rows x 32 pixels of a frame) column by
+// column, frame by frame.  Frames of x with their halo (6 rows x 34 pixels)
+// and tiles of dy arrive by TMA (64-byte swizzle, zero fill outside the
+// volume) in rings of 7 and 8 slots, so each is loaded once per CTA while
+// up to five frames' warps use it; operands come out of shared memory with
+// transposing ldmatrix (both are voxel-major, the K direction), conflict
+// free under the swizzle.  A CTA writes one partial (kWgVals floats); the
+// partials are summed in order by wgrad_reduce_kernel.
+//
+// Why: one thread per four results on the CUDA cores with a shared-memory
+// step of 64 voxels re-read x and dy for each of the 45 taps (3.3 ms a
+// layer), and its reduction summed db in one CTA (1.5 ms).  Four layers of a
+// training step of 4 volumes of 64 x 32 x 32 voxels: 19.1 -> 0.24 ms
+// (step 20.4 -> 1.57 ms); bound by the mma.sync rate (24 per 16 voxels and
+// warp).  tcgen05 would need 4 taps per M = 128 operand at unequal row
+// offsets, which its descriptors cannot express.
+constexpr int kHaloX = TILE_X + 2, kHaloZ = TILE_Z + 2;
+constexpr int kWgWarps = 15;                    // (dt, dz)
+constexpr int kWgThreads = 32 * (kWgWarps + 1);  // and the TMA warp
+constexpr int kWgXSlots = 7, kWgDySlots = 8;
+constexpr int kWgXBytes = kHaloX * kHaloZ * C * 2;           // 13056
+constexpr int kWgXSlotB = (kWgXBytes + 1023) & ~1023;
+constexpr int kWgDyB = TILE_M * C * 2;                        // 8192
+constexpr int kWgSmem = kWgXSlots * kWgXSlotB + kWgDySlots * kWgDyB + 1024;
+constexpr int kWgVals = NTAP * C * C + C;                     // dW, then db
+constexpr int kWgMaxParts = 152;                              // one CTA per SM
 
-__global__ void __launch_bounds__(256) wgrad_kernel(const __nv_bfloat16 *__restrict__ x,
-                                                    const __nv_bfloat16 *__restrict__ dy, ConvDims d,
-                                                    float *__restrict__ part)
+__device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4])
 {
-    __shared__ float xs[kWgSub][C + 1], gs[kWgSub][C + 1];
-    const int t = blockIdx.y;
-    const int dt = tap_dt(t), dz = tap_dz(t), dx = tap_dx(t);
-    const int64_t V = (int64_t)d.N * d.F * d.Z * d.X;
-    const int64_t v0 = (int64_t)blockIdx.x * kWgChunk;
-    const int ci = threadIdx.x >> 3, co0 = (threadIdx.x & 7) * 4;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int64_t vb = v0; vb < v0 + kWgChunk && vb < V; vb += kWgSub) {
-        for (int i = threadIdx.x; i < kWgSub * C; i += 256) {
-            const int r = i / C, c = i % C;
-            const int64_t v = vb + r;
-            float xv = 0.0f, gv = 0.0f;
-            if (v < V) {
-                gv = __bfloat162float(dy[v * C + c]);
-                const int xx = (int)(v % d.X), zz = (int)((v / d.X) % d.Z), ff = (int)((v / ((int64_t)d.X * d.Z)) % d.F);
-                const int64_t nn = v / ((int64_t)d.X * d.Z * d.F);
-                const int sx = xx + dx, sz = zz + dz, sf = ff + dt;
-                if (sx >= 0 && sx < d.X && sz >= 0 && sz < d.Z && sf >= 0 && sf < d.F)
-                    xv = __bfloat162float(x[((((int64_t)nn * d.F + sf) * d.Z + sz) * d.X + sx) * C + c]);
-            }
-            xs[r][c] = xv;
-            gs[r][c] = gv;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int r = 0; r < kWgSub; ++r) {
-            const float a = xs[r][ci];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[k] = fmaf(a, gs[r][co0 + k], acc[k]);
-        }
-        __syncthreads();
-    }
-    float *o = part + ((size_t)blockIdx.x * NTAP + t) * C * C + ci * C + co0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) o[k] = acc[k];
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
 }
 
-// Sum the chunk partials into dW [45][32][32]; block NTAP also forms
-// db[co] = sum_v dy[v][co].
-__global__ void wgrad_reduce_kernel(const float *__restrict__ part, int n_chunks, const __nv_bfloat16 *__restrict__ dy,
-                                    int64_t V, float *__restrict__ dw, float *__restrict__ db)
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
-    if (blockIdx.x < NTAP) {
-        const int t = blockIdx.x;
-        for (int i = threadIdx.x; i < C * C; i += blockDim.x) {
-            float s = 0.0f;
-            for (int c = 0; c < n_chunks; ++c) s += part[((size_t)c * NTAP + t) * C * C + i];
-            dw[(size_t)t * C * C + i] = s;
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// byte offset of 16-byte chunk c of 64-byte row q under the 64-byte swizzle
+__device__ __forceinline__ uint32_t sw64_off(int q, int c)
+{
+    return (uint32_t)(q * 64 + ((c ^ ((q >> 1) & 3)) << 4));
+}
+
+// NT: 8-channel blocks of dy that can be non-zero (1 for the last layer)
+template <int NT>
+__global__ void __launch_bounds__(kWgThreads, 1)
+    wgrad_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap dy_map,
+                 const ConvDims d, float *__restrict__ part, int *__restrict__ status)
+{
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *xs = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char *gs = xs + kWgXSlots * kWgXSlotB;
+    __shared__ __align__(8) uint64_t x_full[kWgXSlots], x_free[kWgXSlots], g_full[kWgDySlots], g_free[kWgDySlots];
+    __shared__ int s_fail;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kWgXSlots; ++s) {
+            mbar_init(&x_full[s], 1);
+            mbar_init(&x_free[s], kWgWarps);
         }
-        return;
+        for (int s = 0; s < kWgDySlots; ++s) {
+            mbar_init(&g_full[s], 1);
+            mbar_init(&g_free[s], kWgWarps);
+        }
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    __shared__ float red[8][C + 1];
-    float acc = 0.0f;
-    const int co = threadIdx.x % C, lane_v = threadIdx.x / C;  // 8 voxel lanes per channel
-    for (int64_t v = lane_v; v < V; v += blockDim.x / C) acc += __bfloat162float(dy[v * C + co]);
-    red[lane_v][co] = acc;
     __syncthreads();
-    if (threadIdx.x < C) {
-        float s = 0.0f;
-        for (int k = 0; k < (int)(blockDim.x / C); ++k) s += red[k][threadIdx.x];
-        db[threadIdx.x] = s;
+    const int t0 = range_begin(d.walk_tiles), t1 = range_end(d.walk_tiles);
+
+    if (warp == kWgWarps) {
+        if (lane == 0) {
+            int jx = 0, jg = 0;
+            bool ok = true;
+            for (int t = t0; t < t1 && ok;) {
+                const int col = t / d.F, fa = t - col * d.F, fb = min(d.F, fa + t1 - t);
+                const Column cl = column_at(d, col);
+                for (int g = fa - 2; g <= fb + 1; ++g, ++jx) {
+                    const int s = jx % kWgXSlots, use = jx / kWgXSlots;
+                    if (use > 0 && !mbar_wait(&x_free[s], (uint32_t)(use - 1) & 1u)) { ok = false; break; }
+                    mbar_expect_tx(&x_full[s], kWgXBytes);
+                    tma_load_5d(xs + s * kWgXSlotB, &x_map, &x_full[s], 0, cl.x0 - 1, cl.z0 - 1, g, cl.n);
+                    const int f = g + 2;  // the tile of dy first used with this frame
+                    if (f >= fb) continue;
+                    const int sg = jg % kWgDySlots, useg = jg / kWgDySlots;
+                    ++jg;
+                    if (useg > 0 && !mbar_wait(&g_free[sg], (uint32_t)(useg - 1) & 1u)) { ok = false; ++jx; --jg; break; }
+                    mbar_expect_tx(&g_full[sg], kWgDyB);
+                    tma_load_5d(gs + sg * kWgDyB, &dy_map, &g_full[sg], 0, cl.x0, cl.z0, f, cl.n);
+                }
+                t += fb - fa;
+            }
+            if (!ok) {
+                s_fail = 1;
+                // let the copies already issued land before the CTA can exit
+                for (int k = 1; k <= kWgXSlots && jx - k >= 0; ++k)
+                    mbar_wait(&x_full[(jx - k) % kWgXSlots], (uint32_t)((jx - k) / kWgXSlots) & 1u);
+                for (int k = 1; k <= kWgDySlots && jg - k >= 0; ++k)
+                    mbar_wait(&g_full[(jg - k) % kWgDySlots], (uint32_t)((jg - k) / kWgDySlots) & 1u);
+            }
+        }
+    } else {
+        const int dti = warp / 3, dzi = warp % 3;  // dt + 2, dz + 1
+        float acc[3][2][NT][4];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int n = 0; n < NT; ++n)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[a][m][n][k] = 0.0f;
+        float db[NT];
+#pragma unroll
+        for (int n = 0; n < NT; ++n) db[n] = 0.0f;
+        // ldmatrix rows of this lane: A (x): row = lane % 8 + 8 (lane / 16), chunk = (lane / 8) % 2;
+        // B (dy): row = lane % 8 + 8 ((lane / 8) % 2), chunk = lane / 16
+        const int a_row = (lane & 7) + ((lane >> 4) << 3), a_ch = (lane >> 3) & 1;
+        const int b_row = (lane & 7) + (((lane >> 3) & 1) << 3), b_ch = lane >> 4;
+        int jx = 0, jg0 = 0;
+        bool ok = true;
+        for (int t = t0; t < t1 && ok;) {
+            const int col = t / d.F, fa = t - col * d.F, nf = min(d.F - fa, t1 - t);
+            for (int j = 0; j < nf + 4; ++j, ++jx) {
+                const int s = jx % kWgXSlots;
+                if (!warp_wait(&x_full[s], (uint32_t)(jx / kWgXSlots) & 1u)) { ok = false; break; }
+                const int i = j - dti;  // tile of dy: frame fa + i reads x frame fa + i + dt
+                if (i >= 0 && i < nf) {
+                    const int jg = jg0 + i, sg = jg % kWgDySlots;
+                    if (!warp_wait(&g_full[sg], (uint32_t)(jg / kWgDySlots) & 1u)) { ok = false; break; }
+                    const uint32_t xb = smem_u32(xs + s * kWgXSlotB), gb = smem_u32(gs + sg * kWgDyB);
+#pragma unroll 1
+                    for (int ks = 0; ks < TILE_M / 16; ++ks) {
+                        uint32_t b[(NT + 1) / 2][4];
+#pragma unroll
+                        for (int n = 0; n < (NT + 1) / 2; ++n)
+                            ldsm4t(gb + sw64_off(16 * ks + b_row, 2 * n + b_ch), b[n]);
+                        const int q0 = ((ks >> 1) + dzi) * kHaloX + 16 * (ks & 1) + a_row;
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+                            for (int m = 0; m < 2; ++m) {
+                                uint32_t a[4];
+                                ldsm4t(xb + sw64_off(q0 + dx, 2 * m + a_ch), a);
+#pragma unroll
+                                for (int n = 0; n < NT; ++n)
+                                    mma16816(acc[dx][m][n], a, b[n / 2][2 * (n & 1)], b[n / 2][2 * (n & 1) + 1]);
+                            }
+                        }
+                        if (warp == 0) {
+#pragma unroll
+                            for (int n = 0; n < NT; ++n) {
+                                const float2 u = __bfloat1622float2(
+                                    *reinterpret_cast<const __nv_bfloat162 *>(&b[n / 2][2 * (n & 1)]));
+                                const float2 v = __bfloat1622float2(
+                                    *reinterpret_cast<const __nv_bfloat162 *>(&b[n / 2][2 * (n & 1) + 1]));
+                                db[n] += (u.x + u.y) + (v.x + v.y);
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&g_free[sg]);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&x_free[s]);
+            }
+            jg0 += nf;
+            t += nf;
+        }
+        if (!ok && lane == 0) s_fail = 1;
+        // accumulator element (row, col): rows ci = 16 m + lane / 4 (+ 8), cols co = 8 n + 2 (lane % 4) (+ 1)
+        float *o = part + (size_t)blockIdx.x * kWgVals;
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+            float *ot = o + (size_t)((dti * 3 + dzi) * 3 + dx) * C * C;
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int n = 0; n < 4; ++n) {
+                    const int ci = 16 * m + (lane >> 2), co = 8 * n + 2 * (lane & 3);
+                    float2 lo = make_float2(0.0f, 0.0f), hi = lo;
+                    if (n < NT) {
+                        lo = make_float2(acc[dx][m][n < NT ? n : 0][0], acc[dx][m][n < NT ? n : 0][1]);
+                        hi = make_float2(acc[dx][m][n < NT ? n : 0][2], acc[dx][m][n < NT ? n : 0][3]);
+                    }
+                    *reinterpret_cast<float2 *>(ot + ci * C + co) = lo;
+                    *reinterpret_cast<float2 *>(ot + (ci + 8) * C + co) = hi;
+                }
+        }
+        if (warp == 0) {  // b0 holds (k = 2 (lane % 4) .. + 1, n = lane / 4): sum the four lanes of a column
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                float v = n < NT ? db[n < NT ? n : 0] : 0.0f;
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+                v += __shfl_xor_sync(0xffffffffu, v, 2);
+                if ((lane & 3) == 0) o[NTAP * C * C + 8 * n + (lane >> 2)] = v;
+            }
+        }
     }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_fail) atomicExch(status, (int)FQ_ERR_TIMEOUT);
+}
+
+// Sum the partials, in order, into dW [45][32][32] and db [32]: one warp
+// per 32 values, the partials of a value dealt to 8 warps.
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float *__restrict__ part, int n_parts,
+                                                           float *__restrict__ dw, float *__restrict__ db)
+{
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;  // kWgVals is a multiple of 32
+    float s = 0.0f;
+    for (int c = w; c < n_parts; c += 8) s += part[(size_t)c * kWgVals + i];
+    red[w][lane] = s;
+    __syncthreads();
+    if (w) return;
+    for (int k = 1; k < 8; ++k) s += red[k][lane];
+    if (i < NTAP * C * C) dw[i] = s;
+    else db[i - NTAP * C * C] = s;
 }
 
 // Adam on a flat FP32 parameter array.
@@ -742,8 +924,13 @@ ParamLayout param_layout()
 
 struct ActLayout {
     size_t act[3], out, dy[2], part, loss_part, total;
-    int wg_chunks;
+    int wg_parts;
 };
+
+int64_t tile_count(int N, int F, int Z, int X)
+{
+    return (int64_t)N * F * ((Z + TILE_Z - 1) / TILE_Z) * ((X + TILE_X - 1) / TILE_X);
+}
 
 ActLayout act_layout(int N, int F, int Z, int X)
 {
@@ -753,8 +940,9 @@ ActLayout act_layout(int N, int F, int Z, int X)
     for (int i = 0; i < 3; ++i) { L.act[i] = o; o += (V * C * 2 + 255) & ~(size_t)255; }
     L.out = o; o += (V * C * 4 + 255) & ~(size_t)255;
     for (int i = 0; i < 2; ++i) { L.dy[i] = o; o += (V * C * 2 + 255) & ~(size_t)255; }
-    L.wg_chunks = (int)((V + kWgChunk - 1) / kWgChunk);
-    L.part = o; o += ((size_t)L.wg_chunks * NTAP * C * C * 4 + 255) & ~(size_t)255;
+    const int64_t tiles = tile_count(N, F, Z, X);
+    L.wg_parts = tiles < kWgMaxParts ? (int)tiles : kWgMaxParts;
+    L.part = o; o += ((size_t)L.wg_parts * kWgVals * 4 + 255) & ~(size_t)255;
     L.loss_part = o; o += 1024 * 8;
     L.total = o;
     return L;
@@ -776,6 +964,26 @@ fq_status encode_act_map(CUtensorMap *map, const void *p, int N, int F, int Z, i
     CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(p), dims, strides,
                      ring ? box_ring : box_tap, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                      ring ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    FQ_REQUIRE(r == CUDA_SUCCESS, FQ_ERR_CUDA, "cnn: activation tensor map (%d)", (int)r);
+    return FQ_OK;
+}
+
+// 64-byte swizzled boxes of all 32 channels: `halo` 34 pixels x 6 rows (x of
+// the weight gradient), else 32 x 4 (dy).
+fq_status encode_wg_map(CUtensorMap *map, const void *p, const ConvDims &d, bool halo)
+{
+    auto enc = (PFN_cuTensorMapEncodeTiled_v12000)fqi::tensor_map_encoder_ptr();
+    FQ_REQUIRE(enc, FQ_ERR_CUDA, "cnn: cuTensorMapEncodeTiled unavailable");
+    std::memset(map, 0, sizeof *map);
+    cuuint64_t dims[5] = {(cuuint64_t)C, (cuuint64_t)d.X, (cuuint64_t)d.Z, (cuuint64_t)d.F, (cuuint64_t)d.N};
+    cuuint64_t strides[4] = {(cuuint64_t)C * 2, (cuuint64_t)d.X * C * 2, (cuuint64_t)d.Z * d.X * C * 2,
+                             (cuuint64_t)d.F * d.Z * d.X * C * 2};
+    cuuint32_t box[5] = {(cuuint32_t)C, (cuuint32_t)(halo ? kHaloX : TILE_X), (cuuint32_t)(halo ? kHaloZ : TILE_Z), 1,
+                         1};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(p), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     FQ_REQUIRE(r == CUDA_SUCCESS, FQ_ERR_CUDA, "cnn: activation tensor map (%d)", (int)r);
     return FQ_OK;
@@ -852,12 +1060,30 @@ fq_status conv(int epi, const void *in, const void *params, int layer, bool back
     return launch(conv_tc_kernel<EPI_MASK_BF16>);
 }
 
+template <int NT>
+fq_status launch_wgrad(const void *x, const void *dy, const ConvDims &d, int n_parts, float *part, float *dw, float *db,
+                       int *status, cudaStream_t st)
+{
+    CUtensorMap x_map, dy_map;
+    fq_status r = encode_wg_map(&x_map, x, d, true);
+    if (r) return r;
+    r = encode_wg_map(&dy_map, dy, d, false);
+    if (r) return r;
+    auto kern = wgrad_kernel<NT>;
+    r = fqi::cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem),
+                        "cnn: smem attribute");
+    if (r) return r;
+    kern<<<n_parts, kWgThreads, kWgSmem, st>>>(x_map, dy_map, d, part, status);
+    wgrad_reduce_kernel<<<kWgVals / 32, 256, 0, st>>>(part, n_parts, dw, db);
+    return fqi::launch_check("fq_cnn_backward: weight gradient");
+}
+
 fq_status check_dims(int N, int F, int Z, int X, const char *who)
 {
     FQ_REQUIRE(N >= 1 && F >= 1 && Z >= 1 && X >= TILE_X, FQ_ERR_SHAPE, "%s: bad volume size", who);
     FQ_REQUIRE(X % RING_X == 0 || (Z % TILE_Z == 0 && X % TILE_X == 0), FQ_ERR_SHAPE,
                "%s: X must be a multiple of 128, or of 32 with Z a multiple of 4 (got Z %d, X %d)", who, Z, X);
-    FQ_REQUIRE((int64_t)N * F * (Z / TILE_Z) * (X / TILE_X) < ((int64_t)1 << 31), FQ_ERR_SHAPE, "%s: too many tiles",
+    FQ_REQUIRE(tile_count(N, F, Z, X) < ((int64_t)1 << 31), FQ_ERR_SHAPE, "%s: too many tiles",
                who);
     return FQ_OK;
 }
@@ -867,6 +1093,9 @@ ConvDims make_dims(int N, int F, int Z, int X)
     ConvDims d;
     d.N = N; d.F = F; d.Z = Z; d.X = X;
     d.tiles = N * F * (Z / TILE_Z) * (X / TILE_X);
+    d.zb = (Z + TILE_Z - 1) / TILE_Z;
+    d.xb = X / TILE_X;
+    d.walk_tiles = (int)tile_count(N, F, Z, X);
     return d;
 }
 
@@ -1004,11 +1233,9 @@ fq_status fq_cnn_backward(const void *params, const void *vol, const float *targ
     int cur = 0;
     for (int l = 3; l >= 0; --l) {
         // weight and bias gradients of layer l from its input and output gradient
-        dim3 g((unsigned)A.wg_chunks, NTAP);
         float *part = (float *)(ab + A.part);
-        wgrad_kernel<<<g, 256, 0, st>>>(act_in[l], dy[cur], d, part);
-        wgrad_reduce_kernel<<<NTAP + 1, 256, 0, st>>>(part, A.wg_chunks, dy[cur], V, grads + L.w[l], grads + L.b[l]);
-        s = fqi::launch_check("fq_cnn_backward: weight gradient");
+        if (l == 3) s = launch_wgrad<1>(act_in[l], dy[cur], d, A.wg_parts, part, grads + L.w[l], grads + L.b[l], status, st);
+        else s = launch_wgrad<4>(act_in[l], dy[cur], d, A.wg_parts, part, grads + L.w[l], grads + L.b[l], status, st);
         if (s) return s;
         if (l == 0) break;
         // data gradient through layer l, masked by the ReLU of layer l - 1
