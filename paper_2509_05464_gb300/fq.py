@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 import threading
 
 import numpy as np
@@ -264,6 +265,16 @@ def make_grid(g) -> Grid:
 class _FlowHolder:
     def __init__(self, segments):
         n = len(segments)
+        flat = []
+        for s in segments:
+            flat += (int(s.kind), *s.p0, *s.a1, *s.a2, *s.a3, s.length, s.radius, s.vmax, s.arc_radius, s.phi1,
+                     *s.arc_end)
+        if n and len(flat) == 20 * n:
+            # all segments in one pack: setting the structs' fields one by one
+            # took 0.25 ms for the 63 vessels of the 3D workload's tree
+            self.arr = (Segment * n).from_buffer_copy(struct.pack("=" + "i4x19d" * n, *flat))
+            self.st = Flow(n, C.cast(self.arr, C.POINTER(Segment)))
+            return
         self.arr = (Segment * max(n, 1))()
         for i, s in enumerate(segments):
             self.arr[i] = Segment(int(s.kind), (C.c_double * 3)(*s.p0), (C.c_double * 3)(*s.a1),
