@@ -66,7 +66,7 @@ struct fq_batch {
     std::vector<Wave> waves;
     int rf_tune = 3, das_threads = 128;  // RF register budget (see fq_tile_choice), DAS CTA size
     bool rf_quad = true;  // every member's rows hold whole element quads
-    int ns_max = 0, J_max = 0, M_max = 0, A_max = 0;
+    int ns_max = 0, J_max = 0, M_max = 0, A_max = 0, F_max = 0;
     size_t rf_smem = 0;  // dynamic shared memory of the RF stage kernel
     size_t off_counters = 0, off_status = 0, off_ens = 0, off_params = 0, off_queues = 0, off_scratch = 0, total = 0;
     std::vector<unsigned char> params;  // host image of the parameter blocks
@@ -133,9 +133,9 @@ void item_grids(fq_batch *b, EnsHost &h)
     h.gx[ST_DAS] = cdiv(h.d.grid.nx, b->das_threads / (das_w ? 32 : kDasThreadsPerPixel)) * h.d.grid.ny * h.d.grid.nz;
     h.gy[ST_DAS] = das_w ? cdiv(h.Fp, kDasWarpFramesB) : h.Fp / kFrameChunkB;
     h.items[ST_DAS] = h.gx[ST_DAS] * h.gy[ST_DAS];
-    const int nt = cdiv(h.F, 32);
-    h.gx[ST_GRAM] = nt * (nt + 1) / 2; h.gy[ST_GRAM] = h.n_chunks; h.items[ST_GRAM] = h.gx[ST_GRAM] * h.n_chunks;
-    h.gx[ST_GRAM_REDUCE] = cdiv((int64_t)h.F * h.F, 256); h.gy[ST_GRAM_REDUCE] = 1;
+    fqi::gram_item_counts(h.F, &h.gx[ST_GRAM], &h.gx[ST_GRAM_REDUCE]);
+    h.gy[ST_GRAM] = h.n_chunks; h.items[ST_GRAM] = h.gx[ST_GRAM] * h.n_chunks;
+    h.gy[ST_GRAM_REDUCE] = 1;
     h.items[ST_GRAM_REDUCE] = h.gx[ST_GRAM_REDUCE];
     h.gx[ST_EIG] = 1; h.gy[ST_EIG] = 1; h.items[ST_EIG] = 1;
     h.gx[ST_PROJECT] = cdiv(h.P, kItemPix); h.gy[ST_PROJECT] = 1; h.items[ST_PROJECT] = h.gx[ST_PROJECT];
@@ -289,7 +289,7 @@ fq_status launch_stage(fq_batch *b, char *arena, int w, int s, cudaStream_t st)
     case fqb::ST_RF2IQ: return fqi::batched_rf2iq(ens, q, q.total, b->rf_dtype, b->ch_dtype, b->J_max, st);
     case fqb::ST_DAS:
         return fqi::batched_das(ens, q, q.total, b->ch_dtype, b->iq_dtype, b->M_max, b->A_max, b->ns_max, b->das_threads, st);
-    case fqb::ST_GRAM: return fqi::batched_gram(ens, q, q.total, b->iq_dtype, st);
+    case fqb::ST_GRAM: return fqi::batched_gram(ens, q, q.total, b->iq_dtype, b->F_max, st);
     case fqb::ST_GRAM_REDUCE: return fqi::batched_gram_reduce(ens, q, q.total, st);
     case fqb::ST_EIG:
         return fqi::batched_eig(ens, reinterpret_cast<const int *>(arena + wv.members_off), q.n, st);
@@ -416,6 +416,7 @@ fq_status fq_batch_plan(const fq_ensemble_desc *ens, int32_t n, int32_t rf_dtype
         if (s) { delete b; return s; }
         scratch_sizes(b, h);
         b->ns_max = std::max(b->ns_max, h.ns);
+        b->F_max = std::max(b->F_max, h.F);
         b->J_max = std::max(b->J_max, h.J);
         b->M_max = std::max(b->M_max, h.M);
         b->A_max = std::max(b->A_max, h.A);

@@ -156,7 +156,8 @@ fq_status batched_rf2iq(const fqb::EnsDev *ens, const fqb::StageQueue &q, int it
                         int J_max, cudaStream_t st);
 fq_status batched_das(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int ch_dtype, int iq_dtype,
                       int M_max, int A_max, int ns_max, int threads, cudaStream_t st);
-fq_status batched_gram(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int iq_dtype, cudaStream_t st);
+fq_status batched_gram(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int iq_dtype, int F_max, cudaStream_t st);
+void gram_item_counts(int F, int *parts, int *reduce_items);  // CTAs per pixel chunk; reduction items
 fq_status batched_gram_reduce(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, cudaStream_t st);
 fq_status batched_eig(const fqb::EnsDev *ens, const int *members, int n, cudaStream_t st);
 fq_status batched_project(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int iq_dtype,

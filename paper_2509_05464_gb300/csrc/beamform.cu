@@ -196,12 +196,8 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem, int src
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
+using fqi::cp_async_commit;
+using fqi::cp_async_wait;
 
 template <typename InT>
 struct StreamShape {

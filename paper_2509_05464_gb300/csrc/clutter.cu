@@ -26,19 +26,25 @@ struct ClutterLayout {
     int64_t chunk_len;
 };
 
-constexpr int kGramTile = 32;
+constexpr int kGramThreads = 256;
+constexpr int kGramPx = 16;     // pixels per shared-memory panel of the Gram kernel
+constexpr int kGramRound = 32;  // pixel chunks are multiples of this
+
+// 4 x 4 complex blocks of the upper triangle (block rows bi <= bj)
+__host__ __device__ inline int gram_cols(int F) { return (F + 3) / 4; }
+__host__ __device__ inline int gram_blocks(int F) { return gram_cols(F) * (gram_cols(F) + 1) / 2; }
+__host__ __device__ inline int gram_parts(int F) { return (gram_blocks(F) + kGramThreads - 1) / kGramThreads; }
+size_t gram_smem(int F) { return 2 * (size_t)kGramPx * 2 * gram_cols(F) * sizeof(float4); }
 constexpr int kFastMaxK = 48;  // top-k eigenvectors by inverse iteration up to this k
 
 inline size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 int gram_chunks(int64_t P, int F)
 {
-    int nt = (F + kGramTile - 1) / kGramTile;
-    int pairs = nt * (nt + 1) / 2;
-    int want = (4 * 152 + pairs - 1) / pairs;
-    int64_t max_chunks = (P + kGramTile - 1) / kGramTile;
+    // two CTAs per SM (gram_partial_kernel), all in one wave
+    int want = 2 * 152 / gram_parts(F);
+    int64_t max_chunks = (P + kGramRound - 1) / kGramRound;
     if (want > max_chunks) want = (int)max_chunks;
-    if (want > 64) want = 64;
     if (want < 1) want = 1;
     return want;
 }
@@ -57,7 +63,7 @@ ClutterLayout layout(int64_t P, int F, int gram_mode = FQ_GRAM_F32, bool force_b
     L.G = o; o += al256(sizeof(float2) * F * F);
     L.n_chunks = gram_chunks(P, F);
     int64_t per = (P + L.n_chunks - 1) / L.n_chunks;
-    L.chunk_len = (per + kGramTile - 1) / kGramTile * kGramTile;
+    L.chunk_len = (per + kGramRound - 1) / kGramRound * kGramRound;
     L.part = o; o += esz ? 0 : al256(sizeof(float2) * (size_t)L.n_chunks * F * F);
     L.tc = o; o += esz ? fqi::gram_tc_workspace_bytes(P, F, esz) : 0;
     L.V = o; o += al256(sizeof(float2) * F * F);
@@ -84,83 +90,167 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) { return make_float2(
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 
 // ----------------------------------------------------------------- Gram --
-// Upper-triangular tiles (ti <= tj) of G over pixel chunks; each CTA: one
-// 32x32 complex tile over one chunk; 256 threads, 2x2 outputs each.
-template <typename T>
-__device__ __forceinline__ void gram_tile(const T *__restrict__ S, int64_t P, int F, int nt, int64_t chunk_len,
-                                          float2 *__restrict__ part, int pair, int c,
-                                          float2 (*As)[kGramTile + 1], float2 (*Bs)[kGramTile + 1])
+// FP32 on the CUDA cores.  A CTA takes a pixel chunk and up to 256 of the
+// upper triangle's 4 x 4 complex blocks, one per thread (16 complex sums in
+// registers, 64 FMAs per pixel against four 16-byte shared-memory loads).
+// It walks the chunk in panels of 16 pixels x F frames, double-buffered with
+// cp.async: S is read once per part (2 parts at 100 frames, 5 at 200), and
+// only blocks of the triangle are computed (F = 100: 5200 of 5050 products;
+// 32 x 32 tiles with 2 x 2 outputs per thread computed 10240 and read two
+// 8-byte operands per complex product).  2^21 pixels x 100 frames: 6.9 -> 3.2
+// ms; 65536 x 200: 0.60 -> 0.31 ms (57% of the FP32 rate for the products of
+// the triangle).  A panel row is two planes, columns
+// (4b, 4b + 1) and (4b + 2, 4b + 3), so that the 16-byte loads of 32
+// consecutive blocks are contiguous.
+__device__ __forceinline__ void gram_stage(const float *__restrict__ S, int64_t p0, int64_t pend, int F, int nb, float4 *buf)
 {
-    // decode upper-triangular tile pair
-    int t = pair, ti = 0;
-    while (t >= nt - ti) { t -= nt - ti; ++ti; }
-    const int tj = ti + t;
+    const int n = (int)min((int64_t)kGramPx, pend - p0);
+    if ((F & 1) == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0) {  // rows of whole 16-byte units
+        const int U = F >> 1;
+        const float *src = S + p0 * F * 2;
+        for (int i = threadIdx.x; i < n * U; i += kGramThreads) {
+            const int px = i / U, u = i - px * U;
+            fqi::cp_async<16>(buf + px * 2 * nb + (u & 1) * nb + (u >> 1), src + (size_t)i * 4);
+        }
+    } else {
+        const float *src = S + p0 * F * 2;
+        for (int i = threadIdx.x; i < n * F; i += kGramThreads) {
+            const int px = i / F, c = i - px * F;
+            float2 *d = reinterpret_cast<float2 *>(buf + px * 2 * nb + ((c >> 1) & 1) * nb + (c >> 2)) + (c & 1);
+            fqi::cp_async<8>(d, src + (size_t)i * 2);
+        }
+    }
+}
+__device__ __forceinline__ void gram_stage(const __nv_bfloat16 *__restrict__ S, int64_t p0, int64_t pend, int F, int nb, float4 *buf)
+{
+    const int n = (int)min((int64_t)kGramPx, pend - p0);
+    for (int i = threadIdx.x; i < n * F; i += kGramThreads) {
+        const int px = i / F, c = i - px * F;
+        float2 *d = reinterpret_cast<float2 *>(buf + px * 2 * nb + ((c >> 1) & 1) * nb + (c >> 2)) + (c & 1);
+        *d = fqi::load_c(S, p0 * F + i);
+    }
+}
+
+__device__ __forceinline__ void cmac(float2 &s, float ax, float ay, float bx, float by)  // s += conj(a) b
+{
+    s.x = fmaf(ax, bx, s.x);
+    s.y = fmaf(ax, by, s.y);
+    s.x = fmaf(ay, by, s.x);
+    s.y = fmaf(-ay, bx, s.y);
+}
+
+template <typename T>
+__device__ __forceinline__ void gram_part(const T *__restrict__ S, int64_t P, int F, int64_t chunk_len,
+                                          float2 *__restrict__ part, int which, int c, float4 *panel)
+{
+    const int nb = gram_cols(F), nblk = gram_blocks(F), parts = gram_parts(F);
+    const int per = (nblk + parts - 1) / parts;
     const int64_t pbeg = (int64_t)c * chunk_len;
     const int64_t pend = min(P, pbeg + chunk_len);
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    float2 acc[2][2] = {{{0, 0}, {0, 0}}, {{0, 0}, {0, 0}}};
-    for (int64_t p0 = pbeg; p0 < pend; p0 += kGramTile) {
-        for (int i = threadIdx.x; i < kGramTile * kGramTile; i += 256) {
-            int pr = i / kGramTile, col = i % kGramTile;
-            int64_t p = p0 + pr;
-            int ci = ti * kGramTile + col, cj = tj * kGramTile + col;
-            float2 a = make_float2(0, 0), b = make_float2(0, 0);
-            if (p < pend) {
-                if (ci < F) a = fqi::load_c(S, p * F + ci);
-                if (cj < F) b = fqi::load_c(S, p * F + cj);
-            }
-            As[pr][col] = a;
-            Bs[pr][col] = b;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int pr = 0; pr < kGramTile; ++pr) {
-            float2 a0 = As[pr][2 * ty], a1 = As[pr][2 * ty + 1];
-            float2 b0 = Bs[pr][2 * tx], b1 = Bs[pr][2 * tx + 1];
-            // conj(a) b
-            acc[0][0].x += a0.x * b0.x + a0.y * b0.y; acc[0][0].y += a0.x * b0.y - a0.y * b0.x;
-            acc[0][1].x += a0.x * b1.x + a0.y * b1.y; acc[0][1].y += a0.x * b1.y - a0.y * b1.x;
-            acc[1][0].x += a1.x * b0.x + a1.y * b0.y; acc[1][0].y += a1.x * b0.y - a1.y * b0.x;
-            acc[1][1].x += a1.x * b1.x + a1.y * b1.y; acc[1][1].y += a1.x * b1.y - a1.y * b1.x;
-        }
-        __syncthreads();
+    // this thread's block (bi, bj) of the row-major upper triangle
+    int t = which * per + (int)threadIdx.x;
+    const bool on = (int)threadIdx.x < per && t < nblk;
+    int bi = 0, bj = 0;
+    if (on) {
+        while (t >= nb - bi) { t -= nb - bi; ++bi; }
+        bj = bi + t;
     }
-    float2 *out = part + (size_t)c * F * F;
-    for (int a = 0; a < 2; ++a)
-        for (int b = 0; b < 2; ++b) {
-            int i = ti * kGramTile + 2 * ty + a, j = tj * kGramTile + 2 * tx + b;
-            if (i < F && j < F) out[(size_t)i * F + j] = acc[a][b];
+    const int psz = kGramPx * 2 * nb;  // units of a panel
+    __syncthreads();  // the previous item of a persistent CTA still reads the panels
+    // columns past F stay zero (every panel writes the same places)
+    if (F & 3)
+        for (int i = threadIdx.x; i < 2 * kGramPx; i += kGramThreads)
+            panel[i * 2 * nb + nb - 1] = panel[i * 2 * nb + 2 * nb - 1] = make_float4(0, 0, 0, 0);
+    __syncthreads();
+    float2 acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] = make_float2(0, 0);
+    if (pbeg < pend) gram_stage(S, pbeg, pend, F, nb, panel);
+    fqi::cp_async_commit();
+    int cur = 0;
+    for (int64_t p0 = pbeg; p0 < pend; p0 += kGramPx) {
+        if (p0 + kGramPx < pend) gram_stage(S, p0 + kGramPx, pend, F, nb, panel + (cur ^ 1) * psz);
+        fqi::cp_async_commit();
+        fqi::cp_async_wait<1>();
+        __syncthreads();
+        if (on) {
+            const int n = (int)min((int64_t)kGramPx, pend - p0);
+            const float4 *row = panel + cur * psz;
+#pragma unroll 2
+            for (int px = 0; px < n; ++px, row += 2 * nb) {
+                const float4 a0 = row[bi], a1 = row[nb + bi], b0 = row[bj], b1 = row[nb + bj];
+                const float ax[4] = {a0.x, a0.z, a1.x, a1.z}, ay[4] = {a0.y, a0.w, a1.y, a1.w};
+                const float bx[4] = {b0.x, b0.z, b1.x, b1.z}, by[4] = {b0.y, b0.w, b1.y, b1.w};
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) cmac(acc[r][q], ax[r], ay[r], bx[q], by[q]);
+            }
         }
+        __syncthreads();
+        cur ^= 1;
+    }
+    fqi::cp_async_wait<0>();
+    if (on) {
+        float2 *out = part + (size_t)c * F * F;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = 4 * bi + r, j = 4 * bj + q;
+                if (i < F && j < F) out[(size_t)i * F + j] = acc[r][q];
+            }
+    }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) gram_partial_kernel(const T *__restrict__ S, int64_t P, int F, int nt,
-                                                           int64_t chunk_len, float2 *__restrict__ part)
+__global__ void __launch_bounds__(kGramThreads, 2) gram_partial_kernel(const T *__restrict__ S, int64_t P, int F,
+                                                                       int64_t chunk_len, float2 *__restrict__ part)
 {
-    __shared__ float2 As[kGramTile][kGramTile + 1];
-    __shared__ float2 Bs[kGramTile][kGramTile + 1];
-    gram_tile<T>(S, P, F, nt, chunk_len, part, blockIdx.x, blockIdx.y, As, Bs);
+    extern __shared__ float4 panel[];
+    gram_part<T>(S, P, F, chunk_len, part, blockIdx.x, blockIdx.y, panel);
 }
 
+// 32 entries of G from the partial sums: eight threads per entry take every
+// eighth chunk, then one adds their sums in order; the lower triangle from
+// the upper one.
+constexpr int kReduceItem = 32;
 __device__ __forceinline__ void gram_reduce_at(const float2 *__restrict__ part, int n_chunks, int F,
-                                               float2 *__restrict__ G, int idx)
+                                               float2 *__restrict__ G, int item, float2 (*red)[kReduceItem])
 {
-    if (idx >= F * F) return;
-    int i = idx / F, j = idx % F;
-    bool upper = (i / kGramTile) <= (j / kGramTile);
-    int src = upper ? idx : j * F + i;
+    const int lane = threadIdx.x % kReduceItem, g = threadIdx.x / kReduceItem;
+    const int idx = item * kReduceItem + lane;
+    const int i = idx / F, j = idx % F;
+    const bool upper = idx < F * F && (i >> 2) <= (j >> 2);
     float2 s = make_float2(0, 0);
-    for (int c = 0; c < n_chunks; ++c) {
-        float2 v = part[(size_t)c * F * F + src];
-        s.x += v.x;
-        s.y += v.y;
+    if (upper) {
+#pragma unroll 4
+        for (int c = g; c < n_chunks; c += kGramThreads / kReduceItem) {
+            const float2 v = part[(size_t)c * F * F + idx];
+            s.x += v.x;
+            s.y += v.y;
+        }
     }
-    G[idx] = upper ? s : cconj(s);
+    __syncthreads();
+    red[g][lane] = s;
+    __syncthreads();
+    if (g == 0 && upper) {
+        for (int q = 1; q < kGramThreads / kReduceItem; ++q) {
+            s.x += red[q][lane].x;
+            s.y += red[q][lane].y;
+        }
+        G[idx] = s;
+        if ((i >> 2) < (j >> 2)) G[j * F + i] = cconj(s);
+    }
 }
 
-__global__ void gram_reduce_kernel(const float2 *__restrict__ part, int n_chunks, int F, float2 *__restrict__ G)
+__global__ void __launch_bounds__(kGramThreads) gram_reduce_kernel(const float2 *__restrict__ part, int n_chunks, int F,
+                                                                   float2 *__restrict__ G)
 {
-    gram_reduce_at(part, n_chunks, F, G, blockIdx.x * blockDim.x + threadIdx.x);
+    __shared__ float2 red[kGramThreads / kReduceItem][kReduceItem];
+    gram_reduce_at(part, n_chunks, F, G, blockIdx.x, red);
 }
 
 // ------------------------------------------------------------ eigen (1 CTA) --
@@ -813,28 +903,26 @@ fq_status launch_project(const void *S, int64_t P, int F, const float2 *Vt, cons
 
 // ------------------------------------------------------------- batched --
 template <typename T>
-__global__ void __launch_bounds__(256) gram_batched_kernel(const fqb::EnsDev *__restrict__ ens, const fqb::StageQueue q)
+__global__ void __launch_bounds__(kGramThreads, 2) gram_batched_kernel(const fqb::EnsDev *__restrict__ ens, const fqb::StageQueue q)
 {
-    __shared__ float2 As[kGramTile][kGramTile + 1];
-    __shared__ float2 Bs[kGramTile][kGramTile + 1];
+    extern __shared__ float4 panel[];
     __shared__ int s_buf[2];
     fqb::Item it;
     while (fqb::next_item(q, ens, fqb::ST_GRAM, s_buf, it)) {
         const fqb::EnsDev &e = ens[it.e];
-        const int nt = (e.F + kGramTile - 1) / kGramTile;
-        gram_tile<T>((const T *)e.iq, e.P, e.F, nt, e.chunk_len, (float2 *)(e.cws + e.cl_part), it.x, it.y, As, Bs);
+        gram_part<T>((const T *)e.iq, e.P, e.F, e.chunk_len, (float2 *)(e.cws + e.cl_part), it.x, it.y, panel);
     }
 }
 
 __global__ void __launch_bounds__(256) gram_reduce_batched_kernel(const fqb::EnsDev *__restrict__ ens,
                                                                   const fqb::StageQueue q)
 {
+    __shared__ float2 red[kGramThreads / kReduceItem][kReduceItem];
     __shared__ int s_buf[2];
     fqb::Item it;
     while (fqb::next_item(q, ens, fqb::ST_GRAM_REDUCE, s_buf, it)) {
         const fqb::EnsDev &e = ens[it.e];
-        gram_reduce_at((const float2 *)(e.cws + e.cl_part), e.n_chunks, e.F, (float2 *)(e.cws + e.cl_G),
-                       it.x * 256 + threadIdx.x);
+        gram_reduce_at((const float2 *)(e.cws + e.cl_part), e.n_chunks, e.F, (float2 *)(e.cws + e.cl_G), it.x, red);
     }
 }
 
@@ -888,12 +976,14 @@ __global__ void __launch_bounds__(256) power_doppler_kernel(const T *__restrict_
 template <typename T>
 fq_status launch_gram(const void *S, int64_t P, int F, const ClutterLayout &L, char *ws, float2 *G, cudaStream_t st)
 {
-    int nt = (F + kGramTile - 1) / kGramTile;
-    int pairs = nt * (nt + 1) / 2;
     float2 *part = (float2 *)(ws + L.part);
-    dim3 grid(pairs, L.n_chunks);
-    gram_partial_kernel<T><<<grid, 256, 0, st>>>((const T *)S, P, F, nt, L.chunk_len, part);
-    gram_reduce_kernel<<<(F * F + 255) / 256, 256, 0, st>>>(part, L.n_chunks, F, G);
+    const size_t smem = gram_smem(F);
+    fq_status s = fqi::cuda_check(cudaFuncSetAttribute(gram_partial_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)smem), "fq_casorati_gram: smem attribute");
+    if (s) return s;
+    dim3 grid(gram_parts(F), L.n_chunks);
+    gram_partial_kernel<T><<<grid, kGramThreads, smem, st>>>((const T *)S, P, F, L.chunk_len, part);
+    gram_reduce_kernel<<<(F * F + kReduceItem - 1) / kReduceItem, kGramThreads, 0, st>>>(part, L.n_chunks, F, G);
     return fqi::launch_check("fq_casorati_gram");
 }
 
@@ -945,7 +1035,7 @@ ClutterLayout layout_capped(int64_t P, int F, int max_chunks)
     L.G = o; o += al256(sizeof(float2) * F * F);
     L.n_chunks = max_chunks;
     int64_t per = (P + L.n_chunks - 1) / L.n_chunks;
-    L.chunk_len = (per + kGramTile - 1) / kGramTile * kGramTile;
+    L.chunk_len = (per + kGramRound - 1) / kGramRound * kGramRound;
     L.part = o; o += al256(sizeof(float2) * (size_t)L.n_chunks * F * F);
     L.V = o; o += al256(sizeof(float2) * F * F);
     L.Vt = o; o += al256(sizeof(float2) * F * F);
@@ -1227,15 +1317,28 @@ void clutter_layout_batched(int64_t P, int F, size_t off[10], int *n_chunks, int
     *total = L.total;
 }
 
-fq_status batched_gram(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int iq_dtype, cudaStream_t st)
+template <typename T>
+fq_status launch_gram_batched(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int F_max, cudaStream_t st)
 {
-    if (iq_dtype == FQ_F32)
-        gram_batched_kernel<float><<<fqb::persistent_grid(gram_batched_kernel<float>, 256, 0, items), 256, 0, st>>>(
-            ens, q);
-    else
-        gram_batched_kernel<__nv_bfloat16>
-            <<<fqb::persistent_grid(gram_batched_kernel<__nv_bfloat16>, 256, 0, items), 256, 0, st>>>(ens, q);
+    const size_t smem = gram_smem(F_max);
+    auto kern = gram_batched_kernel<T>;
+    fq_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                             "batched Gram: smem attribute");
+    if (s) return s;
+    kern<<<fqb::persistent_grid(kern, kGramThreads, smem, items), kGramThreads, smem, st>>>(ens, q);
     return launch_check("batched Gram");
+}
+
+fq_status batched_gram(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int iq_dtype, int F_max, cudaStream_t st)
+{
+    return iq_dtype == FQ_F32 ? launch_gram_batched<float>(ens, q, items, F_max, st)
+                              : launch_gram_batched<__nv_bfloat16>(ens, q, items, F_max, st);
+}
+
+void gram_item_counts(int F, int *parts, int *reduce_items)
+{
+    *parts = gram_parts(F);
+    *reduce_items = (F * F + kReduceItem - 1) / kReduceItem;
 }
 
 fq_status batched_gram_reduce(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, cudaStream_t st)

@@ -156,6 +156,23 @@ __device__ __forceinline__ ff ff_dot3_minus(df2 ux, df2 uy, df2 uz, df2 o, float
     return ff_fast_two_sum(t2.hi, lo);
 }
 
+// ----------------------------------------------------- asynchronous copy --
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(s), "l"(gmem), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // ------------------------------------------------------ packed FP32 x 2 --
 // Blackwell executes add / sub / mul / fma on a pair of binary32 values held
 // in one 64-bit register (f32x2) as a single instruction.  On GB300 it does
