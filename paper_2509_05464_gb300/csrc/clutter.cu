@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(kGramThreads, 2) gram_partial_kernel(const T *
 // eighth chunk, then one adds their sums in order; the lower triangle from
 // the upper one.
 constexpr int kReduceItem = 32;
+constexpr int kReduceItems = 8;  // of them in an item of the batched reduction
 __device__ __forceinline__ void gram_reduce_at(const float2 *__restrict__ part, int n_chunks, int F,
                                                float2 *__restrict__ G, int item, float2 (*red)[kReduceItem])
 {
@@ -922,7 +923,9 @@ __global__ void __launch_bounds__(256) gram_reduce_batched_kernel(const fqb::Ens
     fqb::Item it;
     while (fqb::next_item(q, ens, fqb::ST_GRAM_REDUCE, s_buf, it)) {
         const fqb::EnsDev &e = ens[it.e];
-        gram_reduce_at((const float2 *)(e.cws + e.cl_part), e.n_chunks, e.F, (float2 *)(e.cws + e.cl_G), it.x, red);
+        for (int i = 0; i < kReduceItems; ++i)
+            gram_reduce_at((const float2 *)(e.cws + e.cl_part), e.n_chunks, e.F, (float2 *)(e.cws + e.cl_G),
+                           it.x * kReduceItems + i, red);
     }
 }
 
@@ -1338,7 +1341,7 @@ fq_status batched_gram(const fqb::EnsDev *ens, const fqb::StageQueue &q, int ite
 void gram_item_counts(int F, int *parts, int *reduce_items)
 {
     *parts = gram_parts(F);
-    *reduce_items = (F * F + kReduceItem - 1) / kReduceItem;
+    *reduce_items = (F * F + kReduceItem * kReduceItems - 1) / (kReduceItem * kReduceItems);
 }
 
 fq_status batched_gram_reduce(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, cudaStream_t st)
