@@ -75,12 +75,18 @@ struct RfParams {
     // its own quantum and added to the FP32 output in turn (1 for 16-bit
     // outputs, whose storage rounding is far coarser than the records')
     int n_sg;
-    // quad kernel: (cos, sin) of the Hann phase of base taps jmin + 1 and jmin +
-    // 2 at the middle fraction, the base window's limit on |frac - 1/2| (beyond
-    // it a ninth tap lies inside the support), and the qn values from qlo of
-    // element 0's whole delay that keep all taps of a quad in the record
-    float st_c0, st_s0, st_c1, st_s1, thr9;
+    // quad kernel: polynomials in (frac - 1/2)^2 of cos(w / 2) cos(w (frac - 1/2))
+    // and sin(w / 2) sin(w (frac - 1/2)) / (frac - 1/2), the base window's limit
+    // on |frac - 1/2| (beyond it a ninth tap lies inside the support), half a
+    // sample as path and its attenuation exponent, and the qn values from qlo
+    // of element 0's whole delay that keep all taps of a quad in the record
+    float pc[4], ps[3];
+    float edge[3];                   // (1 - cos w y) / y^2 in y^2
+    float thr9;
+    fqi::df2 half_path;
+    float att_half, att_l2K;  // att_l2K: att_l2 per sample of path
     int qlo, qn;
+    unsigned seg_mul[3];  // ceil(2^26 / rows per segment) of blocks of 1, 2 and 4 angles (see QuadBlock)
     float dee_max;      // largest |r_e - r_0| of a quad (m)
     float bound_margin;
     float dbx_far;      // the directivity bound at its largest argument, k0 width_x / 2
@@ -119,23 +125,6 @@ __device__ __forceinline__ void sincos_poly(float x, float &s, float &c)
     pc = fmaf(pc, t, kCosPoly2);
     pc = fmaf(pc, t, kCosPoly1);
     c = fmaf(pc, t, kCosPoly0);
-}
-
-// the same for two arguments in packed f32x2 (the same operations per lane)
-__device__ __forceinline__ void sincos_poly2(fqi::f2 x, fqi::f2 &s, fqi::f2 &c)
-{
-    using namespace fqpoly;
-    using fqi::f2_dup;
-    using fqi::f2_fma;
-    const fqi::f2 t = fqi::f2_mul(x, x);
-    fqi::f2 ps = f2_fma(f2_dup(kSinPoly3), t, f2_dup(kSinPoly2));
-    ps = f2_fma(ps, t, f2_dup(kSinPoly1));
-    ps = f2_fma(ps, t, f2_dup(kSinPoly0));
-    s = fqi::f2_mul(x, ps);
-    fqi::f2 pc = f2_fma(f2_dup(kCosPoly4), t, f2_dup(kCosPoly3));
-    pc = f2_fma(pc, t, f2_dup(kCosPoly2));
-    pc = f2_fma(pc, t, f2_dup(kCosPoly1));
-    c = f2_fma(pc, t, f2_dup(kCosPoly0));
 }
 
 // sin(u) / u for two arguments in packed f32x2 (the same operations per lane)
@@ -231,7 +220,7 @@ __global__ void __launch_bounds__(NT, 2) rf_synth_kernel(const RfParams p, const
                                                          const float *__restrict__ rf_base,
                                                          OutT *__restrict__ rf)
 {
-    extern __shared__ int tile[];  // hi [E][Ns] then lo [E][Ns]
+    extern __shared__ __align__(16) int tile[];  // hi [E][Ns] then lo [E][Ns]
     __shared__ float ex_hi[E], ex_lo[E], ey_hi[E], ey_lo[E];
     __shared__ float s_red[NT / 32];
     const int ns = p.pr.ns;
@@ -661,7 +650,7 @@ __global__ void __launch_bounds__(NT, MINB) rf_synth_pair_kernel(const RfParams 
                                                               const float *__restrict__ rf_base,
                                                               OutT *__restrict__ rf)
 {
-    extern __shared__ int tile[];  // hi [2][Ns] then lo [2][Ns]
+    extern __shared__ __align__(16) int tile[];  // hi [2][Ns] then lo [2][Ns]
     __shared__ float s_red[NT / 32];
     rf_pair_tile<NT, OutT>(p, blockIdx.x, blockIdx.y, blockIdx.z, pos, amp, rf_base, rf, tile, s_red);
 }
@@ -673,7 +662,7 @@ template <int NT, int MINB, typename OutT>
 __global__ void __launch_bounds__(NT, MINB) rf_pair_batched_kernel(const fqb::EnsDev *__restrict__ ens,
                                                                 const fqb::StageQueue q)
 {
-    extern __shared__ int tile[];
+    extern __shared__ __align__(16) int tile[];
     __shared__ float s_red[NT / 32];
     __shared__ __align__(16) unsigned char s_par[kRfParamBytes];
     __shared__ int s_buf[2];
@@ -731,18 +720,101 @@ constexpr float kTwo31 = 2147483648.0f;
 
 struct QuadShared {
     float red[32];                     // one per warp
-    float invq[4 * FQ_MAX_ANGLES];     // 1 / q per record (angle in group, element)
-    float q[4 * FQ_MAX_ANGLES];
-    unsigned wmax[4 * FQ_MAX_ANGLES];  // window maximum of the pass-1 bounds (units)
-    unsigned bmax[4 * FQ_MAX_ANGLES];  // largest |static base| (float bits, >= 0)
+    float4 invq[FQ_MAX_ANGLES];        // 1 / q per angle in group: (pair 0, pair 1, pair 1, pair 0)
+    float q[2 * FQ_MAX_ANGLES];        // the quantum per record pair (angle in group, element pair)
+    unsigned wmax[2 * FQ_MAX_ANGLES];  // window maximum of the pass-1 bounds (units)
+    unsigned bmax[2 * FQ_MAX_ANGLES];  // largest |static base| (float bits, >= 0)
     float4 angK[FQ_MAX_ANGLES + 1];    // pass 1: fs / c, then per angle (u, -origin) fs / c
-    float4 angFF[2 * FQ_MAX_ANGLES];   // pass 2: per angle (ux, uy) and (uz, origin) as float pairs
+    float4 angFF[2 * FQ_MAX_ANGLES];   // pass 2: per angle (ux, uy) and (uz, origin + half a sample) as float pairs
+    int4 blk[FQ_MAX_ANGLES / 8 + 3];   // pass 2: the angle blocks: first angle, angles, first word, segment stride
+    unsigned blk_mul[FQ_MAX_ANGLES / 8 + 3];
 };
 
 // Largest record (or bound-bin) area of a quad CTA: a block holds at most
 // 227 KB (232,448 bytes) of shared memory on this GPU, less the kernels'
 // static QuadShared and, in the batched kernel, the parameter block.
 constexpr size_t kQuadSmemMax = 232448 - sizeof(QuadShared) - (size_t)kRfParamBytes - 64;
+
+// Layout of a quad CTA's records.  A warp's 32 lanes hold 32 scatterers; if
+// they add to one record at a time, 32 random samples take ~3.5 wavefronts
+// of the shared pipe, which bounded the kernel (8.8 atomics per pair).  So a
+// row of 32 words (one per bank) holds one sample of eight angles x four
+// elements, and at any time the 32 lanes work on 32 different (angle,
+// element) records: lane l starts its loop over the angles at l / 4 and takes
+// element s ^ (l & 3) in its slot s.  Every lane then has a bank of its own.
+// Angles are taken in blocks of 8 (at most), then 4, 2, 1; a block of nb < 8
+// angles splits its records into 8 / nb segments of `seg` samples, one per
+// set of four banks, so that its rows are full too (lanes of the same angle
+// still meet in a bank when their echoes fall in the same segment).  A row
+// before and eight rows after each segment take the taps of echoes that
+// straddle its ends; they belong to the neighbouring segments' samples.
+// Taps are 32 words apart in every block: immediate offsets from one address.
+struct QuadBlock {
+    int b0, lg, nb;  // first angle (in the CTA's group), log2 of the angles, angles
+    int seg, guard;  // samples per segment; 1 when there are guard rows, else 0
+    int rows, base;  // rows of the block, its first word
+    __host__ __device__ QuadBlock(int na, int ns) : base(0) { set(0, na, ns); }
+    __host__ __device__ void set(int b, int na, int ns)
+    {
+        const int left = na - b;
+        b0 = b;
+        lg = left >= 8 ? 3 : (left >= 4 ? 2 : (left >= 2 ? 1 : 0));
+        nb = 1 << lg;
+        const int nseg = 8 >> lg;
+        const int sl = (ns + nseg - 1) >> (3 - lg);
+        seg = sl > 8 ? sl : 8;  // at least 8: a guard row's sample is the next segment's
+        guard = lg < 3;
+        rows = seg + 9 * guard;
+    }
+    __host__ __device__ void next(int na, int ns)
+    {
+        base += 32 * rows;
+        set(b0 + nb, na, ns);
+    }
+    // word of sample k (of segment sg) of angle b0 + ai, element e
+    __device__ __forceinline__ int word(int ai, int e, int k, int sg) const
+    {
+        return base + 32 * (guard + k - sg * seg) + 4 * ((sg << lg) + ai) + e;
+    }
+};
+
+// words of the records of na angles
+inline size_t quad_words(int na, int ns)
+{
+    QuadBlock b(na, ns);
+    while (b.b0 + b.nb < na) b.next(na, ns);
+    return (size_t)b.base + 32 * (size_t)b.rows;
+}
+
+// eight consecutive values from p[k0], k0 + j < k1 only; `vec`: p + k0 is
+// 16-byte aligned and all eight are inside
+__device__ __forceinline__ void load8(const float *p, int k0, int k1, bool vec, float (&v)[8])
+{
+    if (vec) {
+        const float4 a = *reinterpret_cast<const float4 *>(p + k0), b = *reinterpret_cast<const float4 *>(p + k0 + 4);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = k0 + j < k1 ? p[k0 + j] : 0.0f;
+    }
+}
+template <typename T>
+__device__ __forceinline__ void store8(T *p, int k0, int k1, bool vec, const float (&v)[8])
+{
+    if (vec) {
+        __align__(16) T t[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) fqi::store_f(t, j, v[j]);
+#pragma unroll
+        for (int i = 0; i < (int)sizeof(t) / 16; ++i)
+            reinterpret_cast<uint4 *>(p + k0)[i] = reinterpret_cast<const uint4 *>(t)[i];
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (k0 + j < k1) fqi::store_f(p, k0 + j, v[j]);
+    }
+}
 
 // an upper bound of |sin(u) / u| for |u| <= 5 (the fitted directivity's
 // range): 1 - u^2/6 + u^4/120 bounds sin(u)/u from above for every u (the
@@ -766,60 +838,109 @@ __device__ __forceinline__ float block_max(float v, float *red)
     return v;
 }
 
-// a non-negative float below 2^22 rounded to the nearest integer
-__device__ __forceinline__ int rint_small(float v) { return __float_as_int(v + kMagic) - kMagicBits; }
+// a non-negative float below 2^22 rounded to the nearest integer (the addition
+// not contracted with a product in v: every kernel gets the same bounds)
+__device__ __forceinline__ int rint_small(float v) { return __float_as_int(__fadd_rn(v, kMagic)) - kMagicBits; }
 
-// one tap of two records: V = (V0, V1) in quanta (|V| < 2^31) rounded to the
-// nearest integers and added
-__device__ __forceinline__ void add_tap2(int *r0, int *r1, int k0, int k1, f2 V)
-{
-    float a, b;
-    fqi::f2_split(V, a, b);
-    atomicAdd(r0 + k0, __float2int_rn(a));
-    atomicAdd(r1 + k1, __float2int_rn(b));
-}
-
-// Taps of the two-cycle pulse A (1 + C)/2 (2 C^2 - 1) = ((A C + A) C - A/2) C
-// - A/2 of two elements from their Hann-phase cosines C_j.  The recurrence
-// runs on E_j = s_j C_j with the signs s = + + - - + + - -, which turn
-// C_{j+1} = 2 cos(w) C_j - C_{j-1} into E_{j+1} = +- 2 cos(w) E_j + E_{j-1}:
-// one packed operation and no negated copy of the cosines; a tap of negative
-// sign takes the coefficients negated where C enters oddly (the same
-// roundings).
-struct Tap2 {
-    f2 A, nA, hA, nhA;
-    __device__ __forceinline__ explicit Tap2(f2 a)
-        : A(a), nA(fqi::f2_mul(a, fqi::f2_dup(-1.0f))), hA(fqi::f2_mul(a, fqi::f2_dup(0.5f))),
-          nhA(fqi::f2_mul(a, fqi::f2_dup(-0.5f)))
-    {
-    }
+// Taps of the two-cycle pulse A (1 + C)/2 (2 C^2 - 1) = A (1 + C) (C^2 - 1/2)
+// of two elements from their Hann-phase cosines C_0 .. C_7 at the base taps
+// (offsets j - 7/2 - phi, phi = frac - 1/2).  The middle two come from two
+// short polynomials: C_3, C_4 = cos(w/2) cos(w phi) -+ sin(w/2) sin(w phi).
+// The others follow outwards by the Chebyshev recurrence (three steps to
+// either end, so its rounding stays small), on E_j = s_j C_j with the signs
+// s = + - - + + - - +, which turn C_{j+1} = 2 cos(w) C_j - C_{j-1} into
+// E_{j+1} = +- 2 cos(w) E_j + E_{j-1}: one packed operation and no negated
+// copy of the cosines.
+struct Pulse2 {
+    f2 A, nA;
+    __device__ __forceinline__ explicit Pulse2(f2 a) : A(a), nA(fqi::f2_mul(a, fqi::f2_dup(-1.0f))) {}
     template <int J>
-    __device__ __forceinline__ f2 at(f2 E) const
+    __device__ __forceinline__ f2 tap(f2 E) const
     {
-        constexpr bool neg = (J & 2) != 0;
-        return fqi::f2_fma(fqi::f2_fma(fqi::f2_fma(neg ? nA : A, E, A), E, neg ? hA : nhA), E, nhA);
+        constexpr bool neg = ((J + 1) & 2) != 0;
+        return fqi::f2_mul(fqi::f2_fma(neg ? nA : A, E, A), fqi::f2_fma(E, E, fqi::f2_dup(-0.5f)));
+    }
+    // emit(integral_constant j, taps j of both elements)
+    template <typename Emit>
+    __device__ __forceinline__ void taps(const RfParams &p, f2 PH, Emit emit) const
+    {
+        using std::integral_constant;
+        const f2 t = fqi::f2_mul(PH, PH);
+        f2 P = fqi::f2_fma(t, fqi::f2_dup(p.pc[3]), fqi::f2_dup(p.pc[2]));
+        P = fqi::f2_fma(P, t, fqi::f2_dup(p.pc[1]));
+        P = fqi::f2_fma(P, t, fqi::f2_dup(p.pc[0]));
+        f2 Q = fqi::f2_fma(t, fqi::f2_dup(p.ps[2]), fqi::f2_dup(p.ps[1]));
+        Q = fqi::f2_fma(Q, t, fqi::f2_dup(p.ps[0]));
+        // P -+ Q phi as multiply-adds: a product and a sum of their own may be
+        // contracted in one kernel and not in another
+        const f2 E3 = fqi::f2_fma(Q, fqi::f2_mul(PH, fqi::f2_dup(-1.0f)), P), E4 = fqi::f2_fma(Q, PH, P);
+        const f2 T = fqi::f2_dup(p.two_cos_h), NT = fqi::f2_dup(-p.two_cos_h);
+        emit(integral_constant<int, 3>{}, tap<3>(E3));
+        emit(integral_constant<int, 4>{}, tap<4>(E4));
+        const f2 E5 = fqi::f2_fma(NT, E4, E3);
+        emit(integral_constant<int, 5>{}, tap<5>(E5));
+        const f2 E6 = fqi::f2_fma(T, E5, E4);
+        emit(integral_constant<int, 6>{}, tap<6>(E6));
+        emit(integral_constant<int, 7>{}, tap<7>(fqi::f2_fma(NT, E6, E5)));
+        const f2 E2 = fqi::f2_fma(NT, E3, E4);
+        emit(integral_constant<int, 2>{}, tap<2>(E2));
+        const f2 E1 = fqi::f2_fma(T, E2, E3);
+        emit(integral_constant<int, 1>{}, tap<1>(E1));
+        emit(integral_constant<int, 0>{}, tap<0>(fqi::f2_fma(NT, E1, E2)));
     }
 };
 
-// the ninth tap, x = w (|frac - 1/2| - thr9) inside the support's edge (at most
-// 0.35 rad: C = -cos x from its series, truncated below 1e-9)
-__device__ __forceinline__ float edge_tap(float A, float x)
+// The ninth taps: y = |frac - 1/2| - thr9 >= 0 inside the support's edge
+// (w y at most 0.35 rad), where C = -cos(w y): A (1 - cos) (cos^2 - 1/2) with u
+// = 1 - cos(w y) from its series (truncated below 1e-7 of it) and cos^2 - 1/2
+// = u^2 - 2 u + 1/2.
+__device__ __forceinline__ f2 edge_tap2(const RfParams &p, f2 A, f2 y)
 {
-    const float t = x * x;
-    const float C = -fmaf(t, fmaf(t, fmaf(t, -1.0f / 720.0f, 1.0f / 24.0f), -0.5f), 1.0f);
-    return tap2(A, 0.5f * A, C);
+    const f2 t = fqi::f2_mul(y, y);
+    const f2 u = fqi::f2_mul(t, fqi::f2_fma(fqi::f2_fma(t, fqi::f2_dup(p.edge[2]), fqi::f2_dup(p.edge[1])), t, fqi::f2_dup(p.edge[0])));
+    const f2 w = fqi::f2_fma(u, u, fqi::f2_fma(u, fqi::f2_dup(-2.0f), fqi::f2_dup(0.5f)));
+    return fqi::f2_mul(fqi::f2_mul(A, u), w);
 }
 
-// The setup of an echo (not its taps) is most of the instructions: base taps
-// that start at jmin + 1 whatever the fraction (no selects of start phases),
-// whole delays from the bits of a rounded sum (no floor and conversion), one
-// range test per angle for four elements, dead elements as zero amplitudes,
-// and the signed recurrence took 2D (100k scatterers, 16 frames, FP32) from
-// 5.31 to 4.87 ms and 3D (500k, 12 frames, BF16) from 208.3 to 198.4 ms, with
-// the same error against 64 bits (7.4e-7 -> 7.3e-7 in 2D).
+// one tap of one record at shared-memory byte address a + OFF
+template <int OFF>
+__device__ __forceinline__ void red_tap(unsigned a, float v)
+{
+    asm volatile("red.shared.add.u32 [%0 + %2], %1;" ::"r"(a), "r"(__float2int_rn(v)), "n"(OFF) : "memory");
+}
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ void red_tap_if(unsigned a, float v, bool on)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p red.shared.add.u32 [%0], %1;\n\t}" ::"r"(a),
+                 "r"(__float2int_rn(v)), "r"((unsigned)on)
+                 : "memory");
+}
+
+// What bounds it: per echo (of 84 warp instructions in 3D) 8 conversions on
+// the XU pipe (60% busy), 47 packed operations' FMA cycles (58%), 8 shared
+// atomics (46% of the shared pipe since the lanes have banks of their own,
+// 78% before) and issue (75%).  Steps since the version that held each record
+// in a row of its own, 2D (100k scatterers, 16 frames, FP32) / 3D (500k, 12
+// frames, BF16): 5.31 / 208.3 ms; no selects of start phases, whole delays
+// from the bits of a rounded sum, one range test for four elements, dead
+// elements as zero amplitudes 4.87 / 198.4; a bank per lane (see QuadBlock)
+// 5.26 / 194.6, its address arithmetic eating the gain; taps from the middle
+// outwards in three operations each, no floor 4.62 / 167.1; no loads ahead
+// (the registers go to the taps) and one vote for the ninth taps of a pair
+// 4.57 / 167.2; whole warps without a divergent end-of-record path 4.39 /
+// 161.8.  896, 768 or 640 threads with more registers each measured 0-5%
+// slower; the constants as packed parameters 178.7 (spills).  Error against 64
+// bits in 2D 7.5e-7 throughout.
 //
 // One tile: elements 4 bx .. 4 bx + 3, angles ag * p.ag .. (of the group),
-// frame f.  `tile` is the dynamic shared memory (p.ag * 4 * Ns ints).
+// frame f.  `tile` is the dynamic shared memory (quad_words(p.ag, Ns) ints).
 // Delays: float-float (~48 bits) for FP32 outputs; for 16-bit outputs the
 // binary32 delay (error ~1e-4 sample, a carrier-phase error ~2e-4 rad, below
 // the BF16 / FP16 storage rounding of 2^-9 / 2^-11) saves the error-free
@@ -834,49 +955,48 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
     const int ns = p.pr.ns;
     const int M = p.pr.M;
     const int m0 = bx * E;
-    const int ne = min(E, M - m0);
     const int64_t S = p.S;
     const int a0 = ag * p.ag;
     const int na = min(p.ag, p.A - a0);
-    const int nrec = na * E;
+    const int npair = na * 2;
     const bool matrix = p.pr.ny > 1;
+    unsigned tid;  // pinned: ptxas re-reads the special register at every use otherwise
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+    const int lane = tid & 31, wid = tid >> 5;
     const float *X = pos + (int64_t)f * 3 * S;
     const float *Y = X + S;
     const float *Z = Y + S;
 
-    // element abscissae: the first as a float pair, the others as binary32
-    // offsets x_0 - x_e and sums x_0 + x_e (all in one row: nx % 4 == 0)
+    // element abscissae (all in one row: nx % 4 == 0); this lane's slot s holds
+    // element s ^ pm, at offset eo[s] from element 0
     const int row = m0 / p.pr.nx, col0 = m0 % p.pr.nx;
     const ff ex0 = fqi::elem_coord(col0, p.pr.nx, p.pr.pitch_x);
     const ff ey = fqi::elem_coord(row, p.pr.ny, p.pr.pitch_y);
-    float cd[E], csh[E], csl[E], exf[E];
+    const int pm = lane & 3;
+    float exf[E], eo[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        const ff xe = fqi::elem_coord(min(col0 + e, p.pr.nx - 1), p.pr.nx, p.pr.pitch_x);
+        const ff xe = fqi::elem_coord(col0 + e, p.pr.nx, p.pr.pitch_x);
         exf[e] = xe.hi + xe.lo;
-        cd[e] = (ex0.hi - xe.hi) + (ex0.lo - xe.lo);
-        const ff sum = fqi::ff_add(ex0, xe);  // x_0 + x_e as a float pair: 2 x - sum cancels exactly
-        csh[e] = sum.hi;
-        csl[e] = sum.lo;
+        eo[e] = __fmul_rn((float)(e ^ pm), p.pr.pitch_x.hi);
     }
-    bool live_e[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) live_e[e] = e < ne;
     const float eyf = ey.hi + ey.lo;
-    // the quad's abscissae span [xlo, xhi] (dead lanes repeat the last element)
-    const float xlo = fminf(fminf(exf[0], exf[1]), fminf(exf[2], exf[3]));
-    const float xhi = fmaxf(fmaxf(exf[0], exf[1]), fmaxf(exf[2], exf[3]));
+    const float xlo = exf[0], xhi = exf[E - 1];  // the quad's abscissae span [xlo, xhi]
 
     // the previous item of a persistent CTA may still read the tile
     __syncthreads();
-    if ((int)threadIdx.x <= na) {  // [0].w = fs / c; [1 + al] = the transmit direction and origin x fs / c
+    if ((int)threadIdx.x <= na) {
+        // [0].w = fs / c; [1 + al] = the transmit direction and -origin x fs / c,
+        // less half a sample: delays here are delay - 1/2, whose nearest whole
+        // number is the floor of the delay
         const float K = p.pr.fs_over_c.hi;
         float4 g = make_float4(0.0f, 0.0f, 0.0f, K);
         if (threadIdx.x > 0) {
             const fqi::AngleFF &an = p.ang[a0 + threadIdx.x - 1];
-            g = make_float4(an.ux.hi * K, an.uy.hi * K, an.uz.hi * K, -an.origin.hi * K);
+            g = make_float4(an.ux.hi * K, an.uy.hi * K, an.uz.hi * K, fmaf(-an.origin.hi, K, -0.5f));
+            const ff o = fqi::ff_add(fqi::ff_load(an.origin), fqi::ff_load(p.half_path));
             sh.angFF[2 * threadIdx.x - 2] = make_float4(an.ux.hi, an.ux.lo, an.uy.hi, an.uy.lo);
-            sh.angFF[2 * threadIdx.x - 1] = make_float4(an.uz.hi, an.uz.lo, an.origin.hi, an.origin.lo);
+            sh.angFF[2 * threadIdx.x - 1] = make_float4(an.uz.hi, an.uz.lo, o.hi, o.lo);
         }
         sh.angK[threadIdx.x] = g;
     }
@@ -886,12 +1006,25 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
     // the sum of |taps|, which grows linearly, while the echo grows as its
     // square root), so FP32 outputs of large media take several groups,
     // each with its own quanta, summed into the output in FP32.
+    int words;
+    {
+        QuadBlock b(na, ns);
+        for (int i = 0;; ++i) {
+            if (threadIdx.x == 0) {
+                sh.blk[i] = make_int4(b.b0, b.nb, b.base + 32 * b.guard, 4 * b.nb - 32 * b.seg);
+                sh.blk_mul[i] = b.lg < 3 ? p.seg_mul[b.lg] : 0u;
+            }
+            if (b.b0 + b.nb >= na) break;
+            b.next(na, ns);
+        }
+        words = b.base + 32 * b.rows;
+    }
     for (int sg = 0; sg < p.n_sg; ++sg) {
     const int64_t sb = S * sg / p.n_sg, se = S * (sg + 1) / p.n_sg, Sg = se - sb;
     const bool with_base = rf_base != nullptr && sg == 0;
     __syncthreads();  // the previous group's store still reads the tile
     for (int i = threadIdx.x; i < na * 2 * (ns + 2 * p.win); i += NT) tile[i] = 0;
-    if ((int)threadIdx.x < nrec) {
+    if ((int)threadIdx.x < npair) {
         sh.wmax[threadIdx.x] = 0u;
         sh.bmax[threadIdx.x] = 0u;
     }
@@ -909,14 +1042,13 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
         bm = fmaxf(bm, fabsf(R) * fminf(rsqrtf(r2), kInvRCap));
     }
     if (with_base) {
-        for (int rec = 0; rec < nrec; ++rec) {
+        for (int rec = 0; rec < na * E; ++rec) {
             const int al = rec >> 2, e = rec & 3;
-            if (e >= ne) continue;
             const float *b = rf_base + ((int64_t)(a0 + al) * M + m0 + e) * ns;
             float v = 0.0f;
             for (int k = threadIdx.x; k < ns; k += NT) v = fmaxf(v, fabsf(b[k]));
             for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-            if ((threadIdx.x & 31) == 0) atomicMax(&sh.bmax[rec], __float_as_uint(v));
+            if ((threadIdx.x & 31) == 0) atomicMax(&sh.bmax[rec >> 1], __float_as_uint(v));
         }
     }
     bm = block_max<NT>(bm, sh.red);
@@ -936,7 +1068,7 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
     unsigned *bins = reinterpret_cast<unsigned *>(tile);
     if (bm > 0.0f) {
         const float K = sh.angK[0].w;
-        const float hpK0 = 0.5f * (exf[1] - exf[0]) * K, hpK1 = 0.5f * (exf[3] - exf[2]) * K;
+        const float hpK0 = fmaf(0.5f * (exf[1] - exf[0]), K, 0.5f), hpK1 = fmaf(0.5f * (exf[3] - exf[2]), K, 0.5f);
         float nR = 0.0f, nx = 0.0f, ny = 0.0f, nz = 0.0f;  // one scatterer ahead
         if (sb + threadIdx.x < se) {
             nR = amp[sb + threadIdx.x];
@@ -969,10 +1101,10 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
                 // scatterers closer than the 1/r cap; the matrix probe's
                 // y-directivity bounded by 1
                 const float D = rs > kInvRCap ? 1.0f : fmaxf(sinc_bound(p.kbx * dxs * rs), p.dbx_far);
-                ub[h] = (live_e[2 * h] || live_e[2 * h + 1]) ? rint_small(aR * fminf(rs, kInvRCap) * D) + 1 : 0;
+                ub[h] = rint_small(aR * fminf(rs, kInvRCap) * D) + 1;
             }
             for (int al = 0; al < na; ++al) {
-                const float4 g = sh.angK[al + 1];  // (ux, uy, uz, -origin) fs / c
+                const float4 g = sh.angK[al + 1];  // (ux, uy, uz, -origin) fs / c, less 1/2
                 const float ptxK = fmaf(g.x, x, fmaf(g.y, y, fmaf(g.z, z, g.w)));
                 unsigned *rb = bins + al * 2 * wstride;
 #pragma unroll
@@ -1005,55 +1137,57 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
         }
     }
     __syncthreads();
-    if ((int)threadIdx.x < nrec) {
-        const int rec = threadIdx.x;
-        const float B = bm > 0.0f ? (float)sh.wmax[rec >> 1] / unit : 0.0f;  // bound of sum |taps| (amplitude units)
-        const float den = B * margin + __uint_as_float(sh.bmax[rec]) * 1.0009765625f;
+    if ((int)threadIdx.x < npair) {
+        const int rp = threadIdx.x;
+        const float B = bm > 0.0f ? (float)sh.wmax[rp] / unit : 0.0f;  // bound of sum |taps| (amplitude units)
+        const float den = __fmaf_rn(B, margin, __fmul_rn(__uint_as_float(sh.bmax[rp]), 1.0009765625f));
         float iq = (kTwo31 - (0.5f * (float)Sg + 64.0f)) / den;
         if (!(iq > 0.0f && iq < 1e30f)) iq = 1.0f;
-        sh.invq[rec] = iq;
-        sh.q[rec] = 1.0f / iq;
+        float *v = reinterpret_cast<float *>(&sh.invq[rp >> 1]);
+        v[rp & 1] = v[3 - (rp & 1)] = iq;
+        sh.q[rp] = 1.0f / iq;
     }
+    for (int i = threadIdx.x; i < words; i += NT) tile[i] = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < nrec * ns; i += NT) {
-        const int rec = i / ns, k = i - rec * ns;
-        const int e = rec & 3;
-        int v = 0;
-        if (with_base && e < ne)
-            v = __float2int_rn(rf_base[((int64_t)(a0 + (rec >> 2)) * M + m0 + e) * ns + k] * sh.invq[rec]);
-        tile[i] = v;
+    if (with_base) {
+        // a lane per column of a block's rows (no bank conflicts), eight samples each
+        const bool vec = (ns & 7) == 0 && (reinterpret_cast<uintptr_t>(rf_base) & 15) == 0;
+        for (QuadBlock b(na, ns); b.b0 < na; b.next(na, ns)) {
+            const int sg8 = (lane >> 2) >> b.lg, ai = (lane >> 2) & (b.nb - 1), e = lane & 3;
+            const int k1 = min(ns, (sg8 + 1) * b.seg);
+            const float *src = rf_base + ((int64_t)(a0 + b.b0 + ai) * M + m0 + e) * ns;
+            const float iq = reinterpret_cast<const float *>(&sh.invq[b.b0 + ai])[e >> 1];
+            for (int c = wid; 8 * c < b.seg; c += NT / 32) {
+                const int k0 = sg8 * b.seg + 8 * c;
+                float v[8];
+                load8(src, k0, k1, vec && (b.seg & 7) == 0 && k0 + 8 <= k1, v);
+                int *t = tile + b.word(ai, e, k0, sg8);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (k0 + j < k1) t[32 * j] = __float2int_rn(v[j] * iq);
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
 
     // ---- pass 2: the taps
     const float Kh = p.pr.fs_over_c.hi, Kl = p.pr.fs_over_c.lo;
-    const float att_l2K = p.att_l2 / Kh;  // per sample of delay
-    const float att_l2 = p.att_l2, thr9 = p.thr9, wh = p.w_h;
-    const f2 KH2 = fqi::f2_dup(Kh), WH2 = fqi::f2_dup(wh), MAGIC2 = fqi::f2_dup(kMagic);
-    const f2 STC0 = fqi::f2_dup(p.st_c0), NSTS0 = fqi::f2_dup(-p.st_s0);
-    const f2 STC1 = fqi::f2_dup(p.st_c1), NSTS1 = fqi::f2_dup(-p.st_s1);
-    const f2 TWOCOS = fqi::f2_dup(p.two_cos_h), NTWOCOS = fqi::f2_dup(-p.two_cos_h);
-    const f2 DCC = fqi::f2_dup(p.dc_corr);
+    const float att_l2 = p.att_l2, thr9 = p.thr9;
+    const f2 KH2 = fqi::f2_dup(Kh), MAGIC2 = fqi::f2_dup(kMagic);
+    const unsigned tile_a = (unsigned)__cvta_generic_to_shared(tile);
 
-    // the next scatterer's inputs are loaded one iteration ahead
-    float nR = 0.0f, nx = 0.0f, ny = 0.0f, nz = 0.0f;
-    if (bm > 0.0f && sb + threadIdx.x < se) {
-        nR = amp[sb + threadIdx.x];
-        nx = X[sb + threadIdx.x];
-        ny = Y[sb + threadIdx.x];
-        nz = Z[sb + threadIdx.x];
-    }
-    for (int64_t s = sb + threadIdx.x; bm > 0.0f && s < se; s += NT) {
-        const float R = nR, x = nx, y = ny, z = nz;
-        if (s + NT < se) {
-            nR = amp[s + NT];
-            nx = X[s + NT];
-            ny = Y[s + NT];
-            nz = Z[s + NT];
-        }
-        if (R == 0.0f) continue;
+    // (no loads ahead: the 4 A echoes of a scatterer and the other warps cover
+    // them, and the registers go to the taps)
+    // Warps stay whole: a lane without a scatterer (or whose geometry is not a
+    // number) carries amplitude 0, so the taps take no branch.
+    const int s1 = bm > 0.0f ? (int)se : (int)sb;  // quad_ok: S < 2^30
+    for (int sw = (int)sb + 32 * wid; sw < s1; sw += NT) {
+        const int s = min(sw + lane, s1 - 1);
+        const float x = X[s], y = Y[s], z = Z[s];
+        float R = sw + lane < s1 ? amp[s] : 0.0f;
+        if (__all_sync(0xffffffffu, R == 0.0f)) continue;
         const bool use_y = matrix || y != 0.0f;
-        float dxh, dyh = 0.0f, q2 = 0.0f, zzh, rs0, r0, rl;
+        float dxh, dxl = 0.0f, dyh = 0.0f, q2 = 0.0f, zzh, rs0, r0, rl;
         bool pos0;
         if constexpr (FFD) {
             const ff zz = fqi::ff_two_prod(z, z);
@@ -1061,7 +1195,7 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
             // ---- receive side, element 0: float-float distance
             dxh = __fsub_rn(x, ex0.hi);
             const float bb = __fsub_rn(dxh, x);
-            const float dxl = __fsub_rn(__fadd_rn(__fsub_rn(x, __fsub_rn(dxh, bb)), __fsub_rn(-ex0.hi, bb)), ex0.lo);
+            dxl = __fsub_rn(__fadd_rn(__fsub_rn(x, __fsub_rn(dxh, bb)), __fsub_rn(-ex0.hi, bb)), ex0.lo);
             const float p2 = __fmul_rn(dxh, dxh);
             float lo = __fmaf_rn(2.0f * dxh, dxl, __fmaf_rn(dxh, dxh, -p2));
             ff r2 = fqi::ff_two_sum(p2, zz.hi);
@@ -1106,22 +1240,15 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
         bool sane = true;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            float dxe, rse;
-            bool ok;
-            if (e == 0) {
-                dxe = dxh;
-                rse = rs0;
-                dee[e] = 0.0f;
-                ok = pos0;
-            } else {
-                dxe = __fsub_rn(x, exf[e]);
-                const float re2 = fmaf(dxe, dxe, zy2);
-                rse = rsqrtf(re2);
-                const float re = __fmul_rn(re2, rse);
-                dee[e] = __fdividef(__fmul_rn(cd[e], __fsub_rn(fmaf(2.0f, x, -csh[e]), csl[e])),
-                                    __fadd_rn(re, r0f));  // r_e - r_0
-                ok = re2 > 0.0f;
-            }
+            // x - x_e = dx - eo; r_e - r_0 = eo (eo - 2 dx) / (r_e + r_0)
+            const float dxe = __fsub_rn(dxh, eo[e]);
+            const float re2 = fmaf(dxe, dxe, zy2);
+            const float rse = rsqrtf(re2);
+            float t = fmaf(-2.0f, dxh, eo[e]);
+            if constexpr (FFD) t = fmaf(-2.0f, dxl, t);
+            // (the reciprocal and the product spelled out: the same in every kernel)
+            dee[e] = __fmul_rn(__fmul_rn(eo[e], t), rcp_approx(__fadd_rn(__fmul_rn(re2, rse), r0f)));
+            const bool ok = re2 > 0.0f;
             // an element at zero distance: no echo, and a delay offset that
             // stays in range (as one that is not a number would not)
             if (!ok) dee[e] = 0.0f;
@@ -1129,7 +1256,11 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
             dxa[e] = dxe;
             rsa[e] = ok ? fminf(rse, kInvRCap) : 0.0f;
         }
-        if (!sane) continue;
+        if (!sane) {
+            R = 0.0f;
+#pragma unroll
+            for (int e = 0; e < E; ++e) dee[e] = dxa[e] = rsa[e] = 0.0f;
+        }
         // R D / r per element pair, D = sinc(k0 w/2 dx / r) (x sinc(k0 h/2 dy / r))
         f2 RD2[2];
 #pragma unroll
@@ -1142,11 +1273,17 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
         // the attenuation exp(-att (path_0 + r_e - r_0)) as the per-transmit
         // factor of element 0 times a per-element factor that does not depend
         // on the transmit (1 for element 0)
-        RD2[0] = fqi::f2_mul(RD2[0], fqi::f2_make(1.0f, ex2_approx(att_l2 * dee[1])));
-        RD2[1] = fqi::f2_mul(RD2[1], fqi::f2_make(ex2_approx(att_l2 * dee[2]), ex2_approx(att_l2 * dee[3])));
-        const f2 DE2[2] = {fqi::f2_make(0.0f, dee[1]), fqi::f2_make(dee[2], dee[3])};
-        for (int al = 0; al < na; ++al) {
-            float fl0, fr0, path_hi;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            RD2[h] = fqi::f2_mul(RD2[h], fqi::f2_make(ex2_approx(att_l2 * dee[2 * h]), ex2_approx(att_l2 * dee[2 * h + 1])));
+        const f2 DE2[2] = {fqi::f2_make(dee[0], dee[1]), fqi::f2_make(dee[2], dee[3])};
+        // angle al of the CTA (place ai in a block at word `base`, segment
+        // stride `adj`); SEG: the block has segments
+        auto angle = [&](int al, int ai, int base, int adj, unsigned mul, auto seg_tag) {
+            constexpr bool SEG = decltype(seg_tag)::value;
+            // element 0's delay less 1/2 as a whole number n0 and the rest v in
+            // [-1/2, 1/2]: adding 1.5 2^23 rounds and leaves the number in the low bits
+            float n0m, v, ex;
             if constexpr (FFD) {
                 const float4 g0 = sh.angFF[2 * al], g1 = sh.angFF[2 * al + 1];
                 const ff ptx = fqi::ff_dot3_minus({g0.x, g0.y}, {g0.z, g0.w}, {g1.x, g1.y}, {g1.z, g1.w}, x, y, z);
@@ -1154,105 +1291,164 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
                 path.lo = __fadd_rn(path.lo, __fadd_rn(ptx.lo, rl));
                 const float uh = __fmul_rn(path.hi, Kh);
                 const float ul = __fmaf_rn(path.hi, Kl, __fmaf_rn(path.lo, Kh, __fmaf_rn(path.hi, Kh, -uh)));
-                fl0 = floorf(uh);
-                fr0 = __fadd_rn(__fsub_rn(uh, fl0), ul);
-                path_hi = path.hi;
+                n0m = __fadd_rn(uh, kMagic);
+                v = __fadd_rn(__fsub_rn(uh, __fsub_rn(n0m, kMagic)), ul);
+                ex = __fmaf_rn(att_l2, path.hi, p.att_half);
             } else {
                 // binary32: (u . r - origin) fs / c + r fs / c in samples
                 const float4 g = sh.angK[al + 1];
                 const float u = __fadd_rn(r0K, fmaf(g.x, x, fmaf(g.y, y, fmaf(g.z, z, g.w))));
-                fl0 = floorf(u);
-                fr0 = __fsub_rn(u, fl0);
-                path_hi = u;  // the attenuation exponent takes samples here
+                n0m = __fadd_rn(u, kMagic);
+                v = __fsub_rn(u, __fsub_rn(n0m, kMagic));
+                ex = __fmaf_rn(p.att_l2K, u, p.att_half);
             }
-            // per element pair (0, 1), (2, 3), two lanes of packed f32x2 (element
-            // 0's offset from itself is 0).  T = delay - fl0 - 1/2; adding 1.5
-            // 2^23 rounds it to the whole part C (in the low bits of R, so the
-            // sample index takes no conversion) and leaves phi = frac - 1/2.
-            // Base taps jmin + 1 .. jmin + 8 lie inside the support for every
-            // frac; a ninth does when |phi| >= thr9, below them (phi < 0) or
-            // above, at the same distance from the edge.
-            const ulonglong2 iqv = *reinterpret_cast<const ulonglong2 *>(&sh.invq[al * E]);
-            const f2 IQ2[2] = {f2{iqv.x}, f2{iqv.y}};
-            const f2 FR0 = fqi::f2_dup(fr0 - 0.5f);
-            const f2 ATT0 = fqi::f2_dup(ex2_approx((FFD ? att_l2 : att_l2K) * path_hi));
-            const int fl0i = (int)fl0;
-            const int kofs = fl0i + p.jmin + 1 - kMagicBits;
-            const bool fast = (unsigned)(fl0i - p.qlo) < (unsigned)p.qn;
-            int *rec = tile + al * E * ns;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const f2 T = fqi::f2_fma(DE2[h], KH2, FR0);
+            // away from the record's ends (else this pass adds zeros at its start)
+            const int n0x = __float_as_int(n0m) - kMagicBits;
+            const bool fast = (unsigned)(n0x - p.qlo) < (unsigned)p.qn;
+            const float att = ex2_approx(ex);
+            const float2 iqv = *reinterpret_cast<const float2 *>(reinterpret_cast<const float *>(&sh.invq[al]) + (pm & 2));
+            // per element pair, two lanes of packed f32x2: T = v + the element's
+            // offset, rounded to its whole part C, leaves phi = frac - 1/2.  Base
+            // taps jmin + 1 .. jmin + 8 lie inside the support for every frac; a
+            // ninth does when |phi| >= thr9, below them (phi < 0) or above, at the
+            // same distance from the edge.
+            auto pair = [&](int h, f2 V, float att, auto emit, auto edge) {
+                const f2 T = fqi::f2_fma(DE2[h], KH2, V);
                 const f2 Rb = fqi::f2_add(T, MAGIC2);
                 const f2 PH = fqi::f2_sub(T, fqi::f2_sub(Rb, MAGIC2));
-                float rb0, rb1, ph0, ph1;
+                float rb0, rb1;
                 fqi::f2_split(Rb, rb0, rb1);
+                const Pulse2 pulse(fqi::f2_mul(RD2[h], fqi::f2_dup((h ? iqv.y : iqv.x) * att)));
+                emit(__float_as_int(rb0), __float_as_int(rb1), pulse, PH);
+                // ninth taps: one echo in 78 at these pulses, so a warp vote and
+                // then both elements at once, without a branch per element
+                float ph0, ph1;
                 fqi::f2_split(PH, ph0, ph1);
-                const int k0 = __float_as_int(rb0) + kofs, k1 = __float_as_int(rb1) + kofs;
-                const Tap2 tp(fqi::f2_mul(fqi::f2_mul(RD2[h], IQ2[h]), ATT0));
-                f2 SF, CF;
-                sincos_poly2(fqi::f2_mul(WH2, PH), SF, CF);
-                f2 E0 = fqi::f2_fma(CF, STC0, fqi::f2_mul(SF, NSTS0));
-                f2 E1 = fqi::f2_fma(CF, STC1, fqi::f2_mul(SF, NSTS1));
-                int *r0p = rec + 2 * h * ns, *r1p = r0p + ns;
-                const bool n0 = fabsf(ph0) >= thr9, n1 = fabsf(ph1) >= thr9;
-                if (fast) {
-                    int *a = r0p + k0, *b = r1p + k1;
-                    add_tap2(a, b, 0, 0, tp.at<0>(E0));
-                    add_tap2(a, b, 1, 1, tp.at<1>(E1));
-                    E0 = fqi::f2_fma(NTWOCOS, E1, E0);
-                    add_tap2(a, b, 2, 2, tp.at<2>(E0));
-                    E1 = fqi::f2_fma(TWOCOS, E0, E1);
-                    add_tap2(a, b, 3, 3, tp.at<3>(E1));
-                    E0 = fqi::f2_fma(NTWOCOS, E1, E0);
-                    f2 t4 = tp.at<4>(E0);
-                    // the mean error of the recurrence's taps, taken out (see pulse_dc_bias)
-                    if constexpr (FFD) t4 = fqi::f2_fma(DCC, tp.A, t4);
-                    add_tap2(a, b, 4, 4, t4);
-                    E1 = fqi::f2_fma(TWOCOS, E0, E1);
-                    add_tap2(a, b, 5, 5, tp.at<5>(E1));
-                    E0 = fqi::f2_fma(NTWOCOS, E1, E0);
-                    add_tap2(a, b, 6, 6, tp.at<6>(E0));
-                    E1 = fqi::f2_fma(TWOCOS, E0, E1);
-                    add_tap2(a, b, 7, 7, tp.at<7>(E1));
-                    if (n0 || n1) {
-                        float a0, a1;
-                        fqi::f2_split(tp.A, a0, a1);
-                        if (n0) atomicAdd(a + (ph0 < 0.0f ? -1 : 8), __float2int_rn(edge_tap(a0, wh * (fabsf(ph0) - thr9))));
-                        if (n1) atomicAdd(b + (ph1 < 0.0f ? -1 : 8), __float2int_rn(edge_tap(a1, wh * (fabsf(ph1) - thr9))));
-                    }
-                } else {
-                    // an echo at or near a record end: per-tap bounds
-                    float a0, a1, c00, c01, c10, c11;
-                    fqi::f2_split(tp.A, a0, a1);
-                    fqi::f2_split(E0, c00, c01);
-                    fqi::f2_split(E1, c10, c11);
-                    for (int j = 0; j < 8; ++j) {
-                        if ((unsigned)(k0 + j) < (unsigned)ns) atomicAdd(r0p + k0 + j, __float2int_rn(tap2(a0, 0.5f * a0, c00)));
-                        if ((unsigned)(k1 + j) < (unsigned)ns) atomicAdd(r1p + k1 + j, __float2int_rn(tap2(a1, 0.5f * a1, c01)));
-                        const float c20 = fmaf(p.two_cos_h, c10, -c00), c21 = fmaf(p.two_cos_h, c11, -c01);
-                        c00 = c10;
-                        c01 = c11;
-                        c10 = c20;
-                        c11 = c21;
-                    }
-                    const int x0 = k0 + (ph0 < 0.0f ? -1 : 8), x1 = k1 + (ph1 < 0.0f ? -1 : 8);
-                    if (n0 && (unsigned)x0 < (unsigned)ns)
-                        atomicAdd(r0p + x0, __float2int_rn(edge_tap(a0, wh * (fabsf(ph0) - thr9))));
-                    if (n1 && (unsigned)x1 < (unsigned)ns)
-                        atomicAdd(r1p + x1, __float2int_rn(edge_tap(a1, wh * (fabsf(ph1) - thr9))));
+                if (__any_sync(0xffffffffu, fmaxf(fabsf(ph0), fabsf(ph1)) >= thr9)) {
+                    const f2 AP{PH.v & 0x7fffffff7fffffffull};
+                    float t0, t1;
+                    fqi::f2_split(edge_tap2(p, pulse.A, fqi::f2_add(AP, fqi::f2_dup(-thr9))), t0, t1);
+                    edge(0, fabsf(ph0) >= thr9, ph0 < 0.0f ? -1 : 8, t0);
+                    edge(1, fabsf(ph1) >= thr9, ph1 < 0.0f ? -1 : 8, t1);
+                }
+            };
+            {
+                const int kofs = (fast ? n0x : p.qlo) + (p.jmin + 1 - kMagicBits);
+                const f2 V = fqi::f2_dup(fast ? v : 0.0f);
+                const float at = fast ? att : 0.0f;
+                // byte address of record word 0 of this angle, less the rounding bias of kofs
+                // (16-byte aligned), and this lane's slot 0
+                const unsigned lw = (tile_a + 4u * (unsigned)(base + 4 * ai) + 128u * (unsigned)kofs) | 4u * (unsigned)pm;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    unsigned a = 0, c = 0;
+                    pair(h, V, at,
+                         [&](int r0, int r1, const Pulse2 &pulse, f2 PH) {
+                             a = (lw ^ (unsigned)(8 * h)) + 128u * (unsigned)r0;
+                             c = (lw ^ (unsigned)(8 * h + 4)) + 128u * (unsigned)r1;
+                             if constexpr (SEG) {
+                                 a += (((unsigned)(r0 + kofs) * mul) >> 26) * (unsigned)(4 * adj);
+                                 c += (((unsigned)(r1 + kofs) * mul) >> 26) * (unsigned)(4 * adj);
+                             }
+                             pulse.taps(p, PH, [&](auto j, f2 t) {
+                                 // the mean error of the taps, taken out (see pulse_dc_bias)
+                                 if constexpr (FFD && decltype(j)::value == 4) t = fqi::f2_fma(fqi::f2_dup(p.dc_corr), pulse.A, t);
+                                 float t0, t1;
+                                 fqi::f2_split(t, t0, t1);
+                                 red_tap<128 * decltype(j)::value>(a, t0);
+                                 red_tap<128 * decltype(j)::value>(c, t1);
+                             });
+                         },
+                         [&](int i, bool on, int j, float t) { red_tap_if((i ? c : a) + 128u * (unsigned)j, t, on); });
                 }
             }
+            // echoes at or near a record end (|n0| < 2^21 keeps the sums below exact;
+            // others lie far outside): per-tap bounds
+            const bool near = !fast && R != 0.0f && (unsigned)(n0x + (1 << 21)) < (1u << 22);
+            if (__any_sync(0xffffffffu, near)) {
+                const int kofs = (near ? n0x : 0) + (p.jmin + 1 - kMagicBits);
+                const f2 V = fqi::f2_dup(near ? v : 0.0f);
+                const float at = near ? att : 0.0f;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    int k[2] = {0, 0};
+                    auto put = [&](int i, int j, float t) {
+                        const unsigned kk = (unsigned)(k[i] + j);
+                        if (near && kk < (unsigned)ns) {
+                            const int sgm = SEG ? (int)((kk * mul) >> 26) : 0;
+                            atomicAdd(tile + base + 4 * ai + ((2 * h + i) ^ pm) + 32 * (int)kk + sgm * adj, __float2int_rn(t));
+                        }
+                    };
+                    pair(h, V, at,
+                         [&](int r0, int r1, const Pulse2 &pulse, f2 PH) {
+                             k[0] = r0 + kofs;
+                             k[1] = r1 + kofs;
+                             pulse.taps(p, PH, [&](auto j, f2 t) {
+                                 float t0, t1;
+                                 fqi::f2_split(t, t0, t1);
+                                 put(0, decltype(j)::value, t0);
+                                 put(1, decltype(j)::value, t1);
+                             });
+                         },
+                         [&](int i, bool on, int j, float t) { if (on) put(i, j, t); });
+                }
+            }
+        };
+        for (int bi = 0;; ++bi) {
+            const int4 b = sh.blk[bi];
+            if (b.y == 8) {
+                for (int i = 0; i < 8; ++i) {
+                    const int ai = (i + (lane >> 2)) & 7;
+                    angle(b.x + ai, ai, b.z, 0, 0u, std::false_type{});
+                }
+            } else {
+                const unsigned mul = sh.blk_mul[bi];
+                for (int i = 0; i < b.y; ++i) {
+                    const int ai = (i + (lane >> 2)) & (b.y - 1);
+                    angle(b.x + ai, ai, b.z, b.w, mul, std::true_type{});
+                }
+            }
+            if (b.x + b.y >= na) break;
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < nrec * ns; i += NT) {
-        const int rec = i / ns, k = i - rec * ns;
-        const int e = rec & 3;
-        if (e >= ne) continue;
-        OutT *out = rf + (((int64_t)f * p.A + a0 + (rec >> 2)) * M + m0 + e) * ns;
-        const float v = __fmul_rn((float)tile[i], sh.q[rec]);
-        fqi::store_f(out, k, sg == 0 ? v : __fadd_rn(fqi::load_f(out, k), v));  // this CTA owns these samples
+    // the records out: a lane per column of a block's rows, eight samples each
+    {
+        const bool vec = (ns & 7) == 0 && (reinterpret_cast<uintptr_t>(rf) & 15) == 0;
+        for (QuadBlock b(na, ns); b.b0 < na; b.next(na, ns)) {
+            const int sg8 = (lane >> 2) >> b.lg, ai = (lane >> 2) & (b.nb - 1), e = lane & 3;
+            const int ks = sg8 * b.seg, k1 = min(ns, ks + b.seg);
+            OutT *out = rf + (((int64_t)f * p.A + a0 + b.b0 + ai) * M + m0 + e) * ns;
+            const float q = sh.q[2 * (b.b0 + ai) + (e >> 1)];
+            for (int c = wid; 8 * c < b.seg; c += NT / 32) {
+                const int k0 = ks + 8 * c;
+                const int *t = tile + b.word(ai, e, k0, sg8);
+                float v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int k = k0 + j;
+                    int w = 0;
+                    if (k < k1) {
+                        w = t[32 * j];
+                        if (b.guard) {  // taps that echoes of the neighbouring segments left in their guard rows
+                            if (sg8 > 0 && k < ks + 8) w += tile[b.word(ai, e, k, sg8 - 1)];
+                            if (k + 1 == ks + b.seg && k + 1 < ns) w += tile[b.word(ai, e, k, sg8 + 1)];
+                        }
+                    }
+                    v[j] = __fmul_rn((float)w, q);
+                }
+                const bool v8 = vec && (b.seg & 7) == 0 && k0 + 8 <= k1;
+                if constexpr (FFD) {  // this CTA owns these samples; 16-bit outputs have one group
+                    if (sg > 0) {
+                        float o[8];
+                        load8(out, k0, k1, v8, o);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) v[j] = __fadd_rn(o[j], v[j]);
+                    }
+                }
+                store8(out, k0, k1, v8, v);
+            }
+        }
     }
     }  // scatterer groups
 }
@@ -1263,15 +1459,15 @@ __global__ void __launch_bounds__(NT, MINB) rf_synth_quad_kernel(const RfParams 
                                                               const float *__restrict__ rf_base,
                                                               OutT *__restrict__ rf)
 {
-    extern __shared__ int tile[];  // [angles in group][4][Ns]
+    extern __shared__ __align__(16) int tile[];  // see QuadBlock
     __shared__ __align__(16) QuadShared sh;
     rf_quad_tile<NT, OutT>(p, blockIdx.x, blockIdx.y, blockIdx.z, pos, amp, rf_base, rf, tile, sh);
 }
 
 size_t quad_smem(const RfParams &p)
 {
-    // the records (4 x Ns per angle) and, before them, the pass-1 bins (2 x (Ns + 2 win))
-    return (size_t)p.ag * sizeof(int) * std::max<size_t>(4 * (size_t)p.pr.ns, 2 * (size_t)(p.pr.ns + 2 * p.win));
+    // the records and, before them, the pass-1 bins (2 x (Ns + 2 win) per angle)
+    return sizeof(int) * std::max<size_t>(quad_words(p.ag, p.pr.ns), 2 * (size_t)p.ag * (p.pr.ns + 2 * p.win));
 }
 
 template <typename OutT>
@@ -1294,7 +1490,7 @@ template <int NT, int MINB, typename OutT>
 __global__ void __launch_bounds__(NT, MINB) rf_quad_batched_kernel(const fqb::EnsDev *__restrict__ ens,
                                                                 const fqb::StageQueue q)
 {
-    extern __shared__ int tile[];
+    extern __shared__ __align__(16) int tile[];
     __shared__ __align__(16) QuadShared sh;
     __shared__ __align__(16) unsigned char s_par[kRfParamBytes];
     __shared__ int s_buf[2];
@@ -1437,43 +1633,45 @@ float pulse_dc_bias(const RfParams &p, double f0, double fs, int n_cycles)
     using namespace fqpoly;
     const double hw = n_cycles * fs / (2.0 * f0);
     const double wh = 2.0 * M_PI * f0 / (n_cycles * fs), wc = 2.0 * M_PI * f0 / fs;
-    const float st_c0 = p.st_c0, nst_s0 = -p.st_s0, st_c1 = p.st_c1, nst_s1 = -p.st_s1, two = p.two_cos_h, w_h = p.w_h;
+    const float *pc = p.pc, *ps = p.ps, *eg = p.edge;
+    const float two = p.two_cos_h;
     double sum[kBiasL] = {}, taps = 0.0;
     for (int b = 0; b < kBiasN; b += kBiasL) {
-        float c0[kBiasL], c1[kBiasL];
+        float c3[kBiasL], c4[kBiasL];
         for (int l = 0; l < kBiasL; ++l) {
             const float ph = ((float)(b + l) + 0.5f) / (float)kBiasN - 0.5f;
-            const float x = w_h * ph;
-            const float t = x * x;
-            float ps = std::fmaf(kSinPoly3, t, kSinPoly2);
-            ps = std::fmaf(ps, t, kSinPoly1);
-            ps = std::fmaf(ps, t, kSinPoly0);
-            const float sf = x * ps;
-            float pc = std::fmaf(kCosPoly4, t, kCosPoly3);
-            pc = std::fmaf(pc, t, kCosPoly2);
-            pc = std::fmaf(pc, t, kCosPoly1);
-            const float cf = std::fmaf(pc, t, kCosPoly0);
-            const float s0 = sf * nst_s0, s1 = sf * nst_s1;
-            c0[l] = std::fmaf(cf, st_c0, s0);
-            c1[l] = std::fmaf(cf, st_c1, s1);
+            const float t = ph * ph;
+            float P = std::fmaf(t, pc[3], pc[2]);
+            P = std::fmaf(P, t, pc[1]);
+            P = std::fmaf(P, t, pc[0]);
+            float Q = std::fmaf(t, ps[2], ps[1]);
+            Q = std::fmaf(Q, t, ps[0]);
+            c3[l] = std::fmaf(Q, -ph, P);
+            c4[l] = std::fmaf(Q, ph, P);
         }
         // the kernel's signed recurrence rounds like this one (fma is symmetric in sign)
-        for (int j = 0; j < 8; ++j)
+        for (int dir = 0; dir < 2; ++dir)
             for (int l = 0; l < kBiasL; ++l) {
-                const float tap = std::fmaf(std::fmaf(std::fmaf(1.0f, c0[l], 1.0f), c0[l], -0.5f), c0[l], -0.5f);
-                sum[l] += (double)tap;
-                const float c2 = std::fmaf(two, c1[l], -c0[l]);
-                c0[l] = c1[l];
-                c1[l] = c2;
+                float x0 = dir ? c4[l] : c3[l], x1 = dir ? c3[l] : c4[l];
+                for (int j = 0; j < 4; ++j) {
+                    const float v = x1 + 1.0f, u = std::fmaf(x1, x1, -0.5f);
+                    const float tap = v * u;
+                    sum[l] += (double)tap;
+                    const float x2 = std::fmaf(two, x1, -x0);
+                    x0 = x1;
+                    x1 = x2;
+                }
             }
     }
     for (int l = 0; l < kBiasL; ++l) taps += sum[l];
-    for (int i = 0; i < kBiasN; ++i) {  // the ninth taps, as edge_tap
+    for (int i = 0; i < kBiasN; ++i) {  // the ninth taps, as edge_tap2
         const float ap = std::fabs(((float)i + 0.5f) / (float)kBiasN - 0.5f);
         if (ap < p.thr9) continue;
-        const float x = w_h * (ap - p.thr9), t = x * x;
-        const float C = -std::fmaf(t, std::fmaf(t, std::fmaf(t, -1.0f / 720.0f, 1.0f / 24.0f), -0.5f), 1.0f);
-        taps += (double)std::fmaf(std::fmaf(std::fmaf(1.0f, C, 1.0f), C, -0.5f), C, -0.5f);
+        const float y = ap - p.thr9, t = y * y;
+        const float e1 = std::fmaf(t, eg[2], eg[1]);
+        const float u = t * std::fmaf(e1, t, eg[0]);
+        const float w = std::fmaf(u, u, std::fmaf(u, -2.0f, 0.5f));
+        taps += (double)(u * w);
     }
     // (1 + cos wh t) / 2 cos wc t = cos(wc t) / 2 + cos((wc - wh) t) / 4 + cos((wc + wh) t) / 4 on |t| < hw
     const int M = (int)std::ceil(hw * kBiasN - 0.5);
@@ -1523,14 +1721,13 @@ fq_status make_rf_params(const fq_probe *probe, const fq_tx *tx, int64_t S, int 
     fqi::make_angles_ff(probe, tx, p.ang);
     // quad kernel: angle groups as large as the shared memory allows, balanced
     // (FQ_RF_AG_KB, at least 16, lowers the budget in KB for tuning)
-    const size_t per_angle = 4 * sizeof(int) * (size_t)probe->n_samples;
     size_t budget = kQuadSmemMax;
     if (const char *env = std::getenv("FQ_RF_AG_KB")) {
         const long kb = std::atol(env);
         if (kb >= 16 && (size_t)kb * 1024 <= kQuadSmemMax) budget = (size_t)kb * 1024;
     }
-    int ag = (int)std::max<size_t>(1, budget / per_angle);
-    ag = std::min(ag, p.A);
+    int ag = p.A;
+    while (ag > 1 && sizeof(int) * quad_words(ag, probe->n_samples) > budget) --ag;
     p.n_ag = (p.A + ag - 1) / ag;
     p.ag = (p.A + p.n_ag - 1) / p.n_ag;
     // taps t of an echo at delay u have |t - u| <= half_w; the pass-1 sample
@@ -1543,17 +1740,35 @@ fq_status make_rf_params(const fq_probe *probe, const fq_tx *tx, int64_t S, int 
     }
     p.bound_margin = (float)(std::exp((double)p.att * (hw + 1.0) / (probe->fs / probe->c)) * (1.0 + 1.0 / 128.0));
     {
-        // base taps jmin + 1 .. jmin + 8, phases at frac = 1/2 + phi
-        const double a0 = wh * (0.5 - (p.jmin + 1)), a1 = wh * (-0.5 - (p.jmin + 1));
-        p.st_c0 = (float)std::cos(a0);
-        p.st_s0 = (float)std::sin(a0);
-        p.st_c1 = (float)std::cos(a1);
-        p.st_s1 = (float)std::sin(a1);
+        // cos(wh phi) and sin(wh phi) / phi in t = phi^2 on [0, 1/4]: Taylor terms
+        // to t^4 and t^3, the last of each economised onto the lower ones
+        // (Chebyshev: y^4 ~ (256 y^3 - 160 y^2 + 32 y - 1) / 128 and y^3 ~ (48 y^2 -
+        // 18 y + 1) / 32 on [0, 1], y = 4 t); truncation below 1e-8 for wh < pi / 4
+        const double w2 = wh * wh, cw = std::cos(0.5 * wh), sw = std::sin(0.5 * wh);
+        const double a4 = w2 * w2 * w2 * w2 / 40320.0 / 256.0 / 128.0, b3 = -w2 * w2 * w2 * wh / 5040.0 / 64.0 / 32.0;
+        p.pc[0] = (float)(cw * (1.0 - a4));
+        p.pc[1] = (float)(cw * (-w2 / 2.0 + 128.0 * a4));
+        p.pc[2] = (float)(cw * (w2 * w2 / 24.0 - 2560.0 * a4));
+        p.pc[3] = (float)(cw * (-w2 * w2 * w2 / 720.0 + 16384.0 * a4));
+        p.ps[0] = (float)(sw * (wh + b3));
+        p.ps[1] = (float)(sw * (-wh * w2 / 6.0 - 72.0 * b3));
+        p.ps[2] = (float)(sw * (wh * w2 * w2 / 120.0 + 768.0 * b3));
+        p.half_path = fqi::split_double(0.5 * probe->c / probe->fs);
+        p.att_half = (float)((double)p.att_l2 * 0.5 * probe->c / probe->fs);
+        p.att_l2K = (float)((double)p.att_l2 * probe->c / probe->fs);
+        p.edge[0] = (float)(w2 / 2.0);
+        p.edge[1] = (float)(-w2 * w2 / 24.0);
+        p.edge[2] = (float)(w2 * w2 * w2 / 720.0);
         p.thr9 = (float)(0.5 - (p.jmin + hw));
         // elements 1 .. 3 of a quad are within 3 pitches of element 0
         const int dmax = (int)std::min(1e6, std::ceil(3.0 * pitch_k) + 2.0);
         p.qlo = dmax - p.jmin;
         p.qn = std::max(0, probe->n_samples - 9 - p.jmin - dmax - p.qlo);
+        for (int lg = 0; lg < 3; ++lg) {
+            // k / seg = (k mul) >> 26 for k < 2^13, seg <= 2^12
+            const unsigned seg = (unsigned)std::max(8, (probe->n_samples + (8 >> lg) - 1) >> (3 - lg));
+            p.seg_mul[lg] = ((1u << 26) + seg - 1) / seg;
+        }
         p.dee_max = (float)(3.0 * probe->pitch_x * (1.0 + 1e-4) + 1e-9);
     }
     p.n_sg = 1;

@@ -1,11 +1,13 @@
-"""The hot kernels at the edges of their layouts: pixel panels and column
-blocks of the FP32 Gram."""
+"""The hot kernels at the edges of their layouts: angle blocks and record
+segments of the RF kernel, pixel panels and column blocks of the FP32 Gram."""
 import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2509_05464_gb300 import build as fqbuild
 from paper_2509_05464_gb300 import fq
+from paper_2509_05464_gb300 import workload as W
 
 pytestmark = pytest.mark.gpu
 
@@ -14,6 +16,34 @@ pytestmark = pytest.mark.gpu
 def _lib():
     fqbuild.build()
     fq.lib()
+
+
+def rel_l2(a, b):
+    return float(np.linalg.norm((a - b).ravel()) / np.linalg.norm(b.ravel()))
+
+
+# blocks of 8, 4, 2 and 1 angles and their sums; record lengths around whole
+# segments (the shortest: segments of their least 8 samples), aligned and not;
+# echoes from before the record to past its end.  Bars as for the other RF
+# routes: 1e-5 in FP32, the storage rounding in 16 bits.
+@pytest.mark.parametrize("A", [1, 2, 3, 5, 7, 8, 9, 11])
+@pytest.mark.parametrize("ns,dt", [(40, "f32"), (301, "f32"), (1000, "f32"), (1000, "bf16"), (999, "f16")])
+def test_rf_angle_blocks_and_segments(A, ns, dt):
+    p = W.Probe(8, 1, 0.1e-3, 0.1e-3, 0.1e-3, 0.1e-3, 15.6e6, 62.5e6, 1540.0, 0.5, 2, ns)
+    rng = np.random.default_rng(100 * A + ns)
+    S, z1 = 517, 1.15 * ns * 1540.0 / 62.5e6 / 2
+    pos = np.stack([rng.uniform(-1e-3, 1e-3, S), np.zeros(S), rng.uniform(0.02e-3, z1, S)]).astype(np.float32)
+    amp = rng.standard_normal(S).astype(np.float32)
+    tx = list(np.radians(np.linspace(-6.0, 6.0, A))) if A > 1 else [0.0]
+    base = rng.standard_normal((A, 8, ns)).astype(np.float32)
+    t = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}[dt]
+    for b in (None, base):
+        got = fq.fq_simulate_rf(p, tx, [0.0] * A, torch.from_numpy(pos[None]).cuda(), torch.from_numpy(amp).cuda(), 1,
+                                rf_base=None if b is None else torch.from_numpy(b).cuda(), out_dtype=t)
+        want = oracle.simulate_rf(p, tx, [0.0] * A, pos, amp, rf=None if b is None else b.astype(np.float64),
+                                  accumulate=b is not None)
+        err = rel_l2(got[0].float().cpu().numpy().astype(np.float64), want)
+        assert err <= {"f32": 1e-5, "bf16": 1e-2, "f16": 1e-3}[dt], (b is None, err)
 
 
 # products of a sum of 2 P terms in binary32, any order: within gamma_2P of
