@@ -482,7 +482,7 @@ __device__ __forceinline__ void widen_pair(uint32_t a, uint32_t b, fqi::f2 &re, 
 // rotated sums of two frames per pair of registers, (re_k, re_k+1) and
 // (im_k, im_k+1): four f32x2 operations per two frames, and half the
 // registers of SepAcc's form.
-template <int FPT, int GS, typename H>
+template <int FPT, typename H>
 struct RotAcc {
     using H2 = typename std::conditional<std::is_same<H, __half>::value, __half2, __nv_bfloat162>::type;
     fqi::f2 R[FPT / 2], I[FPT / 2];
@@ -491,19 +491,27 @@ struct RotAcc {
 #pragma unroll
         for (int m = 0; m < FPT / 2; ++m) R[m] = I[m] = fqi::f2_dup(0.0f);
     }
-    __device__ __forceinline__ void add(const H *b0, int64_t stride, float phi, float cs, float sn)
+    // the interpolation weight in the storage type, twice, as one word
+    static __device__ __forceinline__ float weight(float phi)
     {
-        const uint4 *q0 = reinterpret_cast<const uint4 *>(b0);
-        const uint4 *q1 = reinterpret_cast<const uint4 *>(b0 + stride);
-        uint4 t0[FPT / 4], t1[FPT / 4];
-#pragma unroll
-        for (int g = 0; g < FPT / 4; ++g) {
-            t0[g] = __ldg(q0 + g * GS);
-            t1[g] = __ldg(q1 + g * GS);
-        }
         H2 ph;
         if constexpr (std::is_same<H, __half>::value) ph = __float2half2_rn(phi);
         else ph = __float2bfloat162_rn(phi);
+        return __uint_as_float(*reinterpret_cast<const uint32_t *>(&ph));
+    }
+    // the sample at byte `o` and the next, `rb` bytes on; groups of four frames dg bytes apart
+    template <typename Off>
+    __device__ __forceinline__ void add(const char *base, Off o, Off rb, Off dg, float weight, float cs, float sn)
+    {
+        uint4 t0[FPT / 4], t1[FPT / 4];
+#pragma unroll
+        for (int g = 0; g < FPT / 4; ++g) {
+            const Off og = g ? o + dg : o;
+            t0[g] = __ldg(reinterpret_cast<const uint4 *>(base + og));
+            t1[g] = __ldg(reinterpret_cast<const uint4 *>(base + (og + rb)));
+        }
+        const uint32_t pw = __float_as_uint(weight);
+        const H2 ph = *reinterpret_cast<const H2 *>(&pw);
         const fqi::f2 CS = fqi::f2_dup(cs), SN = fqi::f2_dup(sn), NSN = fqi::f2_dup(-sn);
 #pragma unroll
         for (int g = 0; g < FPT / 4; ++g) {
@@ -732,35 +740,39 @@ __device__ __forceinline__ void das_tile(const DasParams &p, int64_t bx, int by,
 }
 
 
-// ---- one warp per pixel (16-bit channel data) ---------------------------
-// A CTA of NW = blockDim.x / 32 warps takes NW consecutive voxels along x of
-// one (y, z) row (das_ctas with W = NW), frames 128 by .. 128 by + 127:
-// lane l sums frames 128 by + 4 l .. + 3, so that a load instruction reads
-// one element's samples of 128 consecutive frames (512 bytes of 16-bit data,
-// 1024 of FP32).  Per group of 32 columns of an aperture row, lane l
-// evaluates column g0 + l's receive distance once and, per transmit, its
-// delay and carrier rotation into the warp's slot table; then the warp walks
-// the group's elements with an echo in the record, each read back from the
-// table by every lane (a broadcast), so the loop has no divergence.  Lanes
-// whose frames lie beyond the padded count repeat the last frame group and
-// discard it (F = 100: 28 of 32 lanes carry frames).  3D workload (128^3 voxels, 100 frames, BF16 channels): 662 ms
-// against 783 ms for four threads per pixel with two element and two frame
-// slots (8 frames per delay and thread, the first of these kernels to
-// share a delay over more than 4 frames) and 1031 ms for four threads per
-// pixel over 4 frames each; loading two elements before summing either
-// (with the earlier per-lane test in the loop: 684 ms against 690 for BF16,
-// 793 against 719 for FP16) and precomputing the broadcast values (778 ms)
-// are not used.
+// ---- half a warp per voxel (16-bit channel data) -------------------------
+// A CTA of NW = blockDim.x / 32 warps takes 2 NW consecutive voxels along x of
+// one (y, z) row (das_ctas with W = 2 NW): each half warp one voxel, 16 FPT
+// frames at once (lane l: frames 4 l .. + 3 and, with FPT = 8, 64 + 4 l .. + 3,
+// so that a load instruction reads 256 contiguous bytes of one sample row per
+// voxel).  Per group of 16 columns of an aperture row, a lane evaluates its
+// voxel's receive distance of one column once and, per transmit, the delay and
+// carrier rotation into the warp's slot table; then the warp walks the columns
+// that are active for both voxels, every lane reading its voxel's entry back
+// (a broadcast), and last those at the rim of one aperture.  The two voxels
+// are neighbours, so their sample rows mostly coincide.  Groups of frames past
+// the padded count repeat the last one and are not stored.
+//
+// Bound by the latency of L2 (ncu, 72 frames: issue 55%, long scoreboard 7.3 an
+// issue, L1 hits 29%, 5.9 TB/s from L2) and so by resident warps: 128 x 32 x 64
+// voxels, 100 frames, BF16: one warp per voxel, 4 frames a lane 95.2 ms; this
+// split at 87 registers (what ptxas takes unbounded) 95, at 64 (four CTAs per
+// SM) 77.6, at 48 (spilling) 91.7; 4 frames a lane at 32 registers 84.7; 8 lanes
+// a voxel 87.2; prefetch.global.L1 two elements ahead 76.4 (and 3.55 against
+// 3.39 ms in 2D, not used); a barrier per column group to keep the CTA's
+// voxels on the same rows 79.5.  128^3 voxels: 660 -> 523 ms.  Up to 64 frames,
+// 4 frames a lane at 32 registers (seven CTAs): 64^3 voxels, 40 frames, FP16
+// 87.8 -> 42.1 ms.
 constexpr int kDasWarpFrames = 128;
 
-__host__ __device__ inline int das_w_off_slot(int M, int A, int NW) { return das_off_ptx(M) + ((2 * A * NW + 3) & ~3); }
+__host__ __device__ inline int das_w_off_slot(int M, int A, int NW) { return das_off_ptx(M) + ((4 * A * NW + 3) & ~3); }
 __host__ __device__ inline int das_w_off_rot(int M, int A, int NW) { return das_w_off_slot(M, A, NW) + 4 * 32 * NW; }
 __host__ __device__ inline size_t das_w_smem_bytes(int M, int A, int NW, int rot_ns)
 {
     return sizeof(float) * (size_t)das_w_off_rot(M, A, NW) + sizeof(float2) * (size_t)rot_ns;
 }
 
-template <typename ChT, typename OutT>
+template <typename ChT, typename OutT, int FPT, typename Off>
 __device__ __forceinline__ void das_tile_w(const DasParams &p, int64_t bx, int by, const ChT *__restrict__ ch,
                                            OutT *__restrict__ iq, float *etab)
 {
@@ -769,7 +781,8 @@ __device__ __forceinline__ void das_tile_w(const DasParams &p, int64_t bx, int b
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     float *exf = etab, *exh = etab + nxe, *exl = etab + 2 * nxe;
     float *eyf = etab + 3 * nxe, *eyh = eyf + nye, *eyl = eyf + 2 * nye;
-    float2 *ptx_s = reinterpret_cast<float2 *>(etab + das_off_ptx(M));                      // [A][NW]
+    const int vx = threadIdx.x >> 4, l16 = lane & 15, VX = 2 * NW;                            // this half warp's voxel
+    float2 *ptx_s = reinterpret_cast<float2 *>(etab + das_off_ptx(M));                      // [A][VX]
     float4 *slot = reinterpret_cast<float4 *>(etab + das_w_off_slot(M, p.A, NW)) + 32 * wid;  // [32] this warp's
     float2 *rot_s = reinterpret_cast<float2 *>(etab + das_w_off_rot(M, p.A, NW));             // [ns]
     for (int c = threadIdx.x; c < nxe + nye; c += blockDim.x) {
@@ -783,16 +796,15 @@ __device__ __forceinline__ void das_tile_w(const DasParams &p, int64_t bx, int b
             eyf[i] = (float)e; eyh[i] = sp.hi; eyl[i] = sp.lo;
         }
     }
-    const int nxb = (p.gx + NW - 1) / NW;
+    const int nxb = (p.gx + VX - 1) / VX;
     const int xb = (int)(bx % nxb);
     const int64_t t = bx / nxb;
     const int iy = (int)(t % p.gy);
     const int iz = (int)(t / p.gy);
-    const int ix = xb * NW + wid;
-    const bool live = ix < p.gx && iz < p.gz;  // warp-uniform
+    const int ix = xb * VX + vx;
+    const bool live = ix < p.gx && iz < p.gz;  // one value per half warp
     const int64_t pix = ((int64_t)iy * p.gz + iz) * p.gx + ix;
-    const int f0 = by * kDasWarpFrames + 4 * lane;  // this lane's first frame
-    const bool fon = f0 < p.Fp;
+    const int f0 = by * (16 * FPT) + 4 * l16;  // this lane's first frame
     const double xd = __dadd_rn(p.x0, __dmul_rn((double)(live ? ix : 0), p.dx));
     const double yd = __dadd_rn(p.y0, __dmul_rn((double)iy, p.dy));
     const double zd = __dadd_rn(p.z0, __dmul_rn((double)iz, p.dz));
@@ -805,8 +817,6 @@ __device__ __forceinline__ void das_tile_w(const DasParams &p, int64_t bx, int b
     const ff fs_c = fqi::ff_load(p.pr.fs_over_c);
     const ff f0_fs = fqi::ff_load(p.pr.f0_over_fs);
     const int ns = p.pr.ns;
-    const int64_t row_stride = (int64_t)p.Fp * 2;
-    const int64_t line_stride = (int64_t)ns * row_stride;
 
     if (p.rot_tab) {
         for (int n = threadIdx.x; n < ns; n += blockDim.x) {
@@ -815,12 +825,12 @@ __device__ __forceinline__ void das_tile_w(const DasParams &p, int64_t bx, int b
             rot_s[n] = make_float2(cs, sn);
         }
     }
-    for (int a = lane; a < p.A; a += 32) {
+    for (int a = l16; a < p.A; a += 16) {
         const fqi::AngleFF an = p.ang[a];
         ff ptx = fqi::ff_add(fqi::ff_mul(fqi::ff_load(an.ux), X), fqi::ff_mul(fqi::ff_load(an.uy), Y));
         ptx = fqi::ff_add(ptx, fqi::ff_mul(fqi::ff_load(an.uz), Z));
         ptx = fqi::ff_add(ptx, fqi::ff_neg(fqi::ff_load(an.origin)));
-        ptx_s[a * NW + wid] = make_float2(ptx.hi, ptx.lo);
+        ptx_s[a * VX + vx] = make_float2(ptx.hi, ptx.lo);
     }
     __syncthreads();
 
@@ -851,21 +861,23 @@ __device__ __forceinline__ void das_tile_w(const DasParams &p, int64_t bx, int b
             c_hi = nxe - 1;
         }
     }
+    c_lo = min(c_lo, __shfl_xor_sync(0xffffffffu, c_lo, 16));
+    c_hi = max(c_hi, __shfl_xor_sync(0xffffffffu, c_hi, 16));
 
     static_assert(sizeof(ChT) == 2, "das_tile_w takes 16-bit channel data");
-    RotAcc<4, 1, ChT> acc;
+    RotAcc<FPT, ChT> acc;
     acc.init();
-    // lanes past the padded frame count read the last frame group (their
-    // sums are never stored), so the element loop has no branch: 690 ->
-    // 662 ms on the 3D workload against a test per element
-    const ChT *chp = ch + (int64_t)(fon ? f0 : p.Fp - 4) * 2;
-    const unsigned rs32 = (unsigned)(p.Fp * 2);
+    // groups of four frames past the padded frame count repeat the last one
+    // (their sums are never stored), so the element loop has no test of them
+    const Off rb = (Off)p.Fp * (Off)(2 * sizeof(ChT));  // bytes per sample row
+    const Off lo = (Off)(min(f0, p.Fp - 4) * (int)(2 * sizeof(ChT)));
+    const Off dg = (Off)(min(f0 + 64, p.Fp - 4) * (int)(2 * sizeof(ChT))) - lo;
 
     for (int r = row_lo; r <= row_hi; ++r) {
-        for (int g0 = c_lo; g0 <= c_hi; g0 += 32) {
-            const int cq = g0 + lane;
+        for (int g0 = c_lo; g0 <= c_hi; g0 += 16) {
+            const int cq = g0 + l16;
             const int cc = min(cq, nxe - 1);
-            const bool on = cq <= c_hi && fabsf(__fsub_rn(xf, exf[cc])) <= half;
+            const bool on = live && cq <= c_hi && fabsf(__fsub_rn(xf, exf[cc])) <= half;
             if (!__any_sync(0xffffffffu, on)) continue;
             ff rm = {0.0f, 0.0f};
             if (on) {
@@ -882,7 +894,7 @@ __device__ __forceinline__ void das_tile_w(const DasParams &p, int64_t bx, int b
                 float phi = 0.0f, sn = 0.0f, cs = 1.0f;
                 bool ok = on;
                 if (on) {
-                    const float2 pt = ptx_s[a * NW + wid];
+                    const float2 pt = ptx_s[a * VX + vx];
                     const ff path = fqi::ff_add(ff{pt.x, pt.y}, rm);
                     const ff u = fqi::ff_mul(path, fs_c);
                     fqi::ff_floor_frac(u, i, phi);
@@ -903,44 +915,51 @@ __device__ __forceinline__ void das_tile_w(const DasParams &p, int64_t bx, int b
                 }
                 // the channel row (element, sample) within this angle's lines
                 // (M ns < 2^28: it fits an int)
-                slot[lane] = make_float4(__int_as_float(ok ? (r * nxe + cq) * ns + i : 0), phi, cs, sn);
+                slot[lane] = make_float4(__uint_as_float((unsigned)((r * nxe + cq) * ns) + (unsigned)i), RotAcc<FPT, ChT>::weight(phi), cs, sn);
                 __syncwarp();
-                unsigned m = __ballot_sync(0xffffffffu, ok);
-                const ChT *cha = chp + (int64_t)a * M * line_stride;
-                while (m) {
-                    const int j = __ffs(m) - 1;
-                    m &= m - 1;
-                    const float4 d = slot[j];
-                    acc.add(cha + (uint64_t)(unsigned)__float_as_int(d.x) * rs32, row_stride, d.y, d.z, d.w);
+                const unsigned m = __ballot_sync(0xffffffffu, ok);
+                const char *cha = reinterpret_cast<const char *>(ch) + (uint64_t)a * ((uint64_t)M * ns * p.Fp * (2 * sizeof(ChT)));
+                const float4 *sl = slot + (lane & 16);
+                unsigned both = m & (m >> 16) & 0xffffu;
+                unsigned one = (m ^ (m >> 16)) & 0xffffu;
+                while (both) {
+                    const int j = __ffs(both) - 1;
+                    both &= both - 1;
+                    const float4 d = sl[j];
+                    acc.add(cha, (Off)__float_as_uint(d.x) * rb + lo, rb, dg, d.y, d.z, d.w);
+                }
+                while (one) {  // columns at the rim of one voxel's aperture or record
+                    const int j = __ffs(one) - 1;
+                    one &= one - 1;
+                    if ((m >> ((lane & 16) + j)) & 1u) {
+                        const float4 d = sl[j];
+                        acc.add(cha, (Off)__float_as_uint(d.x) * rb + lo, rb, dg, d.y, d.z, d.w);
+                    }
                 }
                 __syncwarp();
             }
         }
     }
-    if (live && fon) {
+    if (live) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < FPT; ++k) {
             const float2 v = acc.get(k);
-            if (f0 + k < p.F) fqi::store_c(iq, pix * p.F + f0 + k, make_float2(v.x * p.inv_A, v.y * p.inv_A));
+            const int f = f0 + 64 * (k >> 2) + (k & 3);
+            if (f < p.F) fqi::store_c(iq, pix * p.F + f, make_float2(v.x * p.inv_A, v.y * p.inv_A));
         }
     }
     __syncthreads();  // a persistent CTA's next tile rewrites the shared tables
 }
 
-// Launch bounds give the thread count alone; ptxas picks the register
-// count (48 for the branch-free element loop, 662 ms on the 3D workload; a
-// 6-CTA bound, at most 42, 669 ms).  With the earlier per-lane test in the
-// loop it picked 40 (a few spilled values, 690 ms), where bounds allowing
-// 42-48 registers without spills measured 795-799 ms and 70 registers
-// 1089 ms; 128- or 512-thread CTAs 865 and 897 ms.
+// (the launch bounds of das_w_kernel: see above das_tile_w)
 constexpr int kDasWarpThreads = 256;
 static_assert(kDasWarpFrames == fqb::kDasWarpFramesB, "batched item shapes");
 
-template <typename ChT, typename OutT, int NT>
-__global__ void __launch_bounds__(NT) das_w_kernel(const DasParams p, const ChT *__restrict__ ch, OutT *__restrict__ iq)
+template <typename ChT, typename OutT, int NT, int MINB, int FPT, typename Off>
+__global__ void __launch_bounds__(NT, MINB) das_w_kernel(const DasParams p, const ChT *__restrict__ ch, OutT *__restrict__ iq)
 {
     extern __shared__ __align__(16) float etab[];  // das_w_smem_bytes
-    das_tile_w<ChT, OutT>(p, blockIdx.x, blockIdx.y, ch, iq, etab);
+    das_tile_w<ChT, OutT, FPT, Off>(p, blockIdx.x, blockIdx.y, ch, iq, etab);
 }
 
 template <typename ChT, typename OutT, int NT, int MINB>
@@ -953,7 +972,7 @@ __global__ void __launch_bounds__(NT, MINB) das_kernel(const DasParams p, const 
 constexpr int kDasParamBytes = (sizeof(DasParams) + 15) & ~15;
 
 template <typename ChT, typename OutT, int NT>
-__global__ void __launch_bounds__(NT) das_batched_kernel(const fqb::EnsDev *__restrict__ ens, const fqb::StageQueue q)
+__global__ void __launch_bounds__(NT, sizeof(ChT) == 2 ? 1024 / NT : 0) das_batched_kernel(const fqb::EnsDev *__restrict__ ens, const fqb::StageQueue q)
 {
     extern __shared__ __align__(16) float etab[];
     __shared__ __align__(16) unsigned char s_par[kDasParamBytes];
@@ -968,7 +987,7 @@ __global__ void __launch_bounds__(NT) das_batched_kernel(const fqb::EnsDev *__re
             __syncthreads();
         }
         if constexpr (sizeof(ChT) == 2)
-            das_tile_w<ChT, OutT>(*reinterpret_cast<const DasParams *>(s_par), it.x, it.y, (const ChT *)e.ch,
+            das_tile_w<ChT, OutT, 8, uint64_t>(*reinterpret_cast<const DasParams *>(s_par), it.x, it.y, (const ChT *)e.ch,
                                   (OutT *)e.iq, etab);
         else
             das_tile<ChT, OutT>(*reinterpret_cast<const DasParams *>(s_par), it.x, it.y, (const ChT *)e.ch,
@@ -993,15 +1012,22 @@ template <typename ChT, typename OutT>
 fq_status launch_das(const DasParams &p, const void *ch, void *iq, cudaStream_t st)
 {
     if constexpr (sizeof(ChT) == 2) {
-        constexpr int NW = kDasWarpThreads / 32;
+        constexpr int NW = kDasWarpThreads / 32, NT = kDasWarpThreads;
         const size_t smem = das_w_smem_bytes(p.pr.M, p.A, NW, p.rot_tab ? p.pr.ns : 0);
-        auto kern = das_w_kernel<ChT, OutT, kDasWarpThreads>;
+        // 64 frames a pass when they hold the ensemble; 32-bit byte offsets when
+        // an angle's lines (and the second row and frame group of the last
+        // sample) stay below 4 GB
+        const bool f64 = p.Fp <= 64;
+        const bool o32 = ((uint64_t)p.pr.M * p.pr.ns + 2) * p.Fp * (2 * sizeof(ChT)) < (uint64_t(1) << 32);
+        auto kern = f64 ? (o32 ? das_w_kernel<ChT, OutT, NT, 7, 4, uint32_t> : das_w_kernel<ChT, OutT, NT, 7, 4, uint64_t>)
+                        : (o32 ? das_w_kernel<ChT, OutT, NT, 4, 8, uint32_t> : das_w_kernel<ChT, OutT, NT, 4, 8, uint64_t>);
         if (smem > 48 * 1024) {
             fq_status s = fqi::cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                                (int)smem), "fq_das: smem attribute");
             if (s) return s;
         }
-        dim3 grid((unsigned)das_ctas(p.gx, p.gy, p.gz, NW), (p.Fp + kDasWarpFrames - 1) / kDasWarpFrames);
+        dim3 grid((unsigned)das_ctas(p.gx, p.gy, p.gz, 2 * NW),
+                  f64 ? 1 : (p.Fp + kDasWarpFrames - 1) / kDasWarpFrames);
         kern<<<grid, kDasWarpThreads, smem, st>>>(p, (const ChT *)ch, (OutT *)iq);
         return fqi::launch_check("fq_das");
     } else {
@@ -1190,9 +1216,10 @@ template <typename ChT, typename OutT>
 fq_status das_by_threads(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int M_max, int A_max,
                          int ns_max, int threads, cudaStream_t st)
 {
-    if (threads == 64) return launch_das_batched<ChT, OutT, 64>(ens, q, items, M_max, A_max, ns_max, st);
-    if (threads == 256) return launch_das_batched<ChT, OutT, 256>(ens, q, items, M_max, A_max, ns_max, st);
-    return launch_das_batched<ChT, OutT, 128>(ens, q, items, M_max, A_max, ns_max, st);
+    constexpr int H = sizeof(ChT) == 2 ? 2 : 1;  // 16-bit data: das_threads / 32 voxels, half a warp each
+    if (threads == 64) return launch_das_batched<ChT, OutT, 64 / H>(ens, q, items, M_max, A_max, ns_max, st);
+    if (threads == 256) return launch_das_batched<ChT, OutT, 256 / H>(ens, q, items, M_max, A_max, ns_max, st);
+    return launch_das_batched<ChT, OutT, 128 / H>(ens, q, items, M_max, A_max, ns_max, st);
 }
 
 fq_status batched_das(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int ch_dtype, int iq_dtype,

@@ -1,5 +1,6 @@
 """The hot kernels at the edges of their layouts: angle blocks and record
-segments of the RF kernel, pixel panels and column blocks of the FP32 Gram."""
+segments of the RF kernel, pixel panels and column blocks of the FP32 Gram,
+frame groups and voxel pairs of the 16-bit delay-and-sum."""
 import numpy as np
 import pytest
 import torch
@@ -58,3 +59,24 @@ def test_gram_panels(F, P, dt):
     mag = (S.double().abs().sum(2)).mT @ S.double().abs().sum(2)
     err = (G - s.mH @ s).abs()
     assert bool((err <= 2.0 ** -24 * (2 * P + 16) * mag).all())
+
+
+# 16-bit channel data against the FP32 kernel on the same values: the
+# interpolation rounds b - a, its weight and the result to u, so a term is
+# within u (2 |b - a| + |v|), at most ~4 u of it on white data
+@pytest.mark.parametrize("dt,u", [(torch.bfloat16, 2.0 ** -8), (torch.float16, 2.0 ** -11)])
+@pytest.mark.parametrize("F", [1, 17, 64, 65, 100, 129, 200])
+@pytest.mark.parametrize("nx,matrix", [(1, False), (17, False), (37, False), (19, True)])
+def test_das_frame_groups_and_voxel_pairs(dt, u, F, nx, matrix):
+    p = (W.Probe(8, 6, 0.3e-3, 0.3e-3, 0.3e-3, 0.3e-3, 7.8e6, 31.25e6, 1540.0, 0.5, 2, 500) if matrix else
+         W.Probe(40, 1, 0.1e-3, 0.1e-3, 0.1e-3, 0.1e-3, 15.6e6, 62.5e6, 1540.0, 0.5, 2, 500))
+    ny = 3 if matrix else 1
+    grid = W.Grid(nx, ny, 9, -1.9e-3, -0.4e-3 if matrix else 0.0, 1e-3, 0.11e-3, 0.4e-3 if matrix else 0.0, 0.55e-3, 1.0)
+    tx = [-0.06, 0.0, 0.06]
+    g = torch.Generator(device="cuda").manual_seed(F + nx)
+    ch = torch.randn((3 * p.nx * p.ny, p.n_samples, fq.frame_pad(F), 2), generator=g, device="cuda").to(dt)
+    got = fq.fq_das(p, tx, [0.0] * 3, ch, F, grid)
+    want = fq.fq_das(p, tx, [0.0] * 3, ch.float(), F, grid)
+    assert rel_l2(got.double().cpu().numpy(), want.double().cpu().numpy()) <= 4 * u
+    for f in {0, F // 2, F - 1}:
+        assert rel_l2(got[:, f].double().cpu().numpy(), want[:, f].double().cpu().numpy()) <= 8 * u
