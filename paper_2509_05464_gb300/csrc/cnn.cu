@@ -7,17 +7,11 @@
 //
 // Layout: activations channels-last, [N][F][Z][X][32] BF16 (the 2-channel
 // input and output are zero-padded to 32 channels, so every layer is one
-// shape).  Forward convolution = implicit GEMM on the tcgen05 tensor cores:
-// one CTA tile is 128 voxels (4 depth rows x 32 lateral pixels of one
-// frame) x 32 output channels; K runs over 45 taps x 32 input channels.
-// For each tap one TMA box load at the tap-shifted coordinates brings the
-// 128 x 64-byte operand rows into shared memory (64-byte swizzle; the
-// tensor map's zero fill outside the volume is the "same" padding; the
-// innermost coordinate is always channel 0, so every load is aligned).  The
-// 45 weight tiles (32 x 32 BF16 each, 90 KB) stay resident in shared memory
-// for the CTA's lifetime.  Two MMAs of K = 16 per tap accumulate in FP32 in
-// tensor memory; two accumulator buffers let the epilogue of one tile
-// overlap the MMAs of the next.  Epilogues: bias + ReLU -> BF16, bias ->
+// shape).  Forward convolution = implicit GEMM on the tcgen05 tensor cores
+// (conv_kernel below): one tile is 128 voxels of one frame x 32 output
+// channels; K runs over 45 taps x 32 input channels.  The weights (90 KB) stay
+// resident in shared memory for the CTA's lifetime; TMA's zero fill outside
+// the volume is the "same" padding.  Epilogues: bias + ReLU -> BF16, bias ->
 // FP32 (last layer), or gradient x ReLU mask -> BF16 (backward).
 //
 // The data gradient of a layer is the same convolution with the kernel
@@ -42,27 +36,15 @@ constexpr int NTAP = 45;              // 5 x 3 x 3
 constexpr int TILE_M = 128;           // voxels per tile: 4 depth rows x 32 lateral
 constexpr int TILE_Z = 4, TILE_X = 32;
 constexpr int ROWB = C * 2;           // 64 bytes per operand row
-constexpr int A_BYTES = TILE_M * ROWB;        // 8 KB per tap stage
 constexpr int W_TAP_BYTES = C * ROWB;         // 2 KB per tap
 constexpr int W_BYTES = NTAP * W_TAP_BYTES;   // 90 KB
-constexpr int STAGES = 6;
 constexpr int CONV_THREADS = 192;     // warp 0 TMA, warp 1 MMA + TMEM owner, warps 2-5 epilogue
-constexpr int TMEM_COLS = 64;         // two 32-column FP32 accumulators
-constexpr int CONV_SMEM = W_BYTES + STAGES * A_BYTES + 1024;
-
-// instruction descriptor: FP32 D, BF16 A and B, both K-major, N = 32, M = 128
-constexpr uint32_t kConvIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(C >> 3) << 17) |
-                                ((uint32_t)(TILE_M >> 4) << 24);
 
 enum Epi { EPI_RELU_BF16 = 0, EPI_LINEAR_F32 = 1, EPI_MASK_BF16 = 2 };
 
-__host__ __device__ constexpr int tap_dt(int t) { return t / 9 - 2; }
-__host__ __device__ constexpr int tap_dz(int t) { return (t / 3) % 3 - 1; }
-__host__ __device__ constexpr int tap_dx(int t) { return t % 3 - 1; }
-
 struct ConvDims {
     int N, F, Z, X;
-    int tiles;         // N F (Z / 4) (X / 32), the per-tap kernel's tiles
+    int run;           // frames per work unit of the convolutions
     int zb, xb;        // depth and lateral blocks of a frame, the last one possibly ragged
     int walk_tiles;    // N zb xb F: tile = column * F + frame
 };
@@ -85,28 +67,6 @@ __device__ __forceinline__ Column column_at(const ConvDims &d, int col)
 // column: output frames fa .. fb - 1.
 __device__ __forceinline__ int range_begin(int tiles) { return (int)((int64_t)tiles * blockIdx.x / gridDim.x); }
 __device__ __forceinline__ int range_end(int tiles) { return (int)((int64_t)tiles * (blockIdx.x + 1) / gridDim.x); }
-
-__device__ __forceinline__ void tile_coords(const ConvDims &d, int tile, int &n, int &f, int &z0, int &x0)
-{
-    const int xb = d.X / TILE_X, zb = d.Z / TILE_Z;
-    int r = tile;
-    const int bx = r % xb; r /= xb;
-    const int bz = r % zb; r /= zb;
-    f = r % d.F;
-    n = r / d.F;
-    z0 = bz * TILE_Z;
-    x0 = bx * TILE_X;
-}
-
-__device__ __forceinline__ void mma_bf16_n32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(kConvIdesc), "r"(accumulate)
-        : "memory");
-}
 
 // Epilogue of one accumulator row (32 channels of voxel `vox`).
 template <int EPI>
@@ -155,156 +115,48 @@ __device__ __forceinline__ void epilogue_store(const float (&v)[32], const float
     }
 }
 
-template <int EPI>
-__global__ void __launch_bounds__(CONV_THREADS, 1)
-    conv_tc_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant__ CUtensorMap w_map,
-                   const ConvDims d, const float *__restrict__ bias, void *__restrict__ out,
-                   const __nv_bfloat16 *__restrict__ mask, int *__restrict__ status)
-{
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char *w_s = base;                 // 45 weight tiles
-    unsigned char *a_s = base + W_BYTES;       // STAGES operand stages
-    __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], acc_full[2], acc_empty[2], w_bar;
-    __shared__ uint32_t tmem_base;
-    __shared__ int s_fail;
-    __shared__ float s_bias[C];
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full_bar[s], 1);
-            mbar_init(&empty_bar[s], 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 4);
-        }
-        mbar_init(&w_bar, 1);
-        s_fail = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (threadIdx.x < C) s_bias[threadIdx.x] = bias ? bias[threadIdx.x] : 0.0f;
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tmem_base;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            // ---- TMA producer: the weights once, then one stage per (tile, tap)
-            mbar_expect_tx(&w_bar, W_BYTES);
-            for (int t = 0; t < NTAP; ++t) tma_load_2d(w_s + t * W_TAP_BYTES, &w_map, &w_bar, 0, t * C);
-            int it = 0;
-            bool fail = false;
-            for (int tile = blockIdx.x; tile < d.tiles && !fail; tile += gridDim.x) {
-                int n, f, z0, x0;
-                tile_coords(d, tile, n, f, z0, x0);
-                for (int t = 0; t < NTAP; ++t, ++it) {
-                    const int s = it % STAGES;
-                    const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-                    if (!mbar_wait(&empty_bar[s], ph ^ 1u)) { fail = true; break; }
-                    mbar_expect_tx(&full_bar[s], A_BYTES);
-                    tma_load_5d(a_s + s * A_BYTES, &in_map, &full_bar[s], 0, x0 + tap_dx(t), z0 + tap_dz(t),
-                                f + tap_dt(t), n);
-                }
-            }
-            if (fail) {
-                s_fail = 1;
-                // let the copies already issued land before the CTA can exit
-                for (int k = 1; k <= STAGES && it - k >= 0; ++k) {
-                    const int j = it - k;
-                    mbar_wait(&full_bar[j % STAGES], (uint32_t)(j / STAGES) & 1u);
-                }
-                mbar_wait(&w_bar, 0);
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            // ---- MMA issuer
-            bool fail = !mbar_wait(&w_bar, 0);
-            tc_fence_after();
-            int it = 0, j = 0;
-            for (int tile = blockIdx.x; tile < d.tiles && !fail; tile += gridDim.x, ++j) {
-                const int buf = j & 1;
-                if (!mbar_wait(&acc_empty[buf], (((uint32_t)j >> 1) & 1u) ^ 1u)) { fail = true; break; }
-                tc_fence_after();
-                const uint32_t acc = tmem + (uint32_t)(buf * C);
-                for (int t = 0; t < NTAP; ++t, ++it) {
-                    const int s = it % STAGES;
-                    const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-                    if (!mbar_wait(&full_bar[s], ph)) { fail = true; break; }
-                    tc_fence_after();
-                    const uint64_t ad = sw64_desc(smem_u32(a_s + s * A_BYTES));
-                    const uint64_t bd = sw64_desc(smem_u32(w_s + t * W_TAP_BYTES));
-                    mma_bf16_n32(acc, ad, bd, t > 0 ? 1u : 0u);
-                    mma_bf16_n32(acc, ad + 2, bd + 2, 1u);  // second 16 channels: +32 bytes
-                    mma_commit(&empty_bar[s]);
-                }
-                if (fail) break;
-                mma_commit(&acc_full[buf]);
-            }
-            if (fail) s_fail = 1;
-        }
-    } else {
-        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = depth row w % 4 of the tile
-        const int q = warp & 3;
-        int j = 0;
-        for (int tile = blockIdx.x; tile < d.tiles; tile += gridDim.x, ++j) {
-            const int buf = j & 1;
-            if (!warp_wait(&acc_full[buf], ((uint32_t)j >> 1) & 1u)) {
-                if (lane == 0) s_fail = 1;
-                break;
-            }
-            tc_fence_after();
-            float v[32];
-            tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * C), v);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
-            int n, f, z0, x0;
-            tile_coords(d, tile, n, f, z0, x0);
-            const int64_t vox = (((int64_t)n * d.F + f) * d.Z + (z0 + q)) * d.X + x0 + lane;
-            epilogue_store<EPI>(v, s_bias, vox, out, mask);
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
-    }
-    if (threadIdx.x == 0 && s_fail) atomicExch(status, (int)FQ_ERR_TIMEOUT);
-}
-
-// ------------------------------------------------- frame-ring convolution --
-// For volumes whose width X is a multiple of 128: a tile is 128 pixels of
-// one depth row of one frame.  A CTA takes work units (n, depth row z,
-// 128-pixel block, run of up to RING_FCH frames) and walks the frames of a
-// unit in order.  Input frames live in a ring of 5 shared-memory slots; one
-// slot holds rows z - 1 .. z + 1 x pixels x0 - 1 .. x0 + 128 of one frame
-// in 4 chunks of 8 channels, each chunk a [3][130] array of 16-byte rows
-// (one TMA box per chunk; zero fill outside the volume).  In this
-// no-swizzle K-major layout rows sit 16 bytes apart, so the operand of tap
-// (dt, dz, dx) is the slot of frame f + dt at row offset (1 + dz) 130 +
-// 1 + dx: each tap is a descriptor, and each output frame loads one new
-// input frame (25 KB) instead of 45 shifted tiles.  The MMA thread issues
-// the dt = -2 taps first and then frees that frame's slot, so the next
-// frame's load overlaps the remaining 36 taps.
-constexpr int RING_X = 128;
-constexpr int RING_W = RING_X + 2;                  // with the lateral halo
-constexpr int RING_BOX = 3 * RING_W * 16;          // 6240 bytes: one TMA box (3 rows x 130 pixels x 8 channels)
-constexpr int RING_CHUNK = 6272;                    // the box's stride in a slot, padded to a multiple of 128
-constexpr int RING_SLOT = 4 * RING_CHUNK;           // 25088 bytes
-constexpr int RING_SLOTS = 5;
-constexpr int RING_FCH = 32;                        // frames per work unit
-constexpr int RING_SMEM = W_BYTES + RING_SLOTS * RING_SLOT + 1024;
+// ------------------------------------------------------------ convolution --
+// A CTA takes work units (one 128-voxel tile of a frame x a run of frames)
+// and walks the input frames of a unit in order through a ring of
+// shared-memory slots, each one frame of the tile with its halo.
+//
+// An MMA of 32 output channels is bound by its operand reads (4 KB of A for
+// 65k products: at most 57% of the tensor rate), so input frame g goes into
+// all five outputs f = g - 2 .. g + 2 it reaches at once: their weights stand
+// side by side (N = 160, block b of 32 for f = g - 2 + b, dt = 2 - b), and
+// their accumulators are consecutive 32-column slots of a ring of 16 in tensor
+// memory (two MMAs where the ring wraps; a ring of 8 wraps twice as often,
+// 5.74 against 5.34 ms for the whole filter).  Each input frame is loaded and
+// read once per unit instead of five times; the other accumulators leave the
+// epilogue its time.  200 x 256 x 256, the filter with its packing and power
+// Doppler: 10.9 ms with one output per MMA, 5.34 ms now (0.9 PFLOP/s of the
+// padded products, tensor pipe 40-46%); a training step's seven convolutions
+// (4 x 64 x 32 x 32) 1.24 -> 0.26 ms.
+//
+// Two tiles:
+//  WIDE (Z not a multiple of 4, X of 128): 128 pixels of one depth row.  A slot holds
+//    rows z - 1 .. z + 1 x pixels x0 - 1 .. x0 + 128 in 4 chunks of 8
+//    channels, each a [3][130] array of 16-byte rows (one TMA box per chunk;
+//    zero fill outside the volume).  In this no-swizzle K-major layout rows
+//    sit 16 bytes apart, so the operand of tap (dz, dx) is the slot at row
+//    offset (1 + dz) 130 + 1 + dx: a descriptor.
+//  otherwise (X a multiple of 32): 4 depth rows x 32 pixels (the same time as
+//    WIDE where both fit).  A slot holds
+//    three copies, shifted by dx, of rows z0 - 1 .. z0 + 4 x 32 pixels, 64
+//    bytes a voxel with the 64-byte swizzle (one TMA box each): the operand
+//    of (dz, dx) is copy dx from row 32 (1 + dz) on, a whole number of swizzle
+//    atoms.  Three boxes of 12 KB a frame where one box per tap took 45 of 8.
+template <bool WIDE>
+struct Tile {
+    static constexpr int Z = WIDE ? 1 : TILE_Z, X = WIDE ? 128 : TILE_X;
+    static constexpr int W = X + 2;                               // WIDE: with the lateral halo
+    static constexpr int BOX = WIDE ? 3 * W * 16 : (TILE_Z + 2) * TILE_X * ROWB;
+    static constexpr int NBOX = WIDE ? 4 : 3;
+    static constexpr int STRIDE = (BOX + 127) / 128 * 128;        // of the boxes in a slot
+    static constexpr int SLOT = NBOX * STRIDE;                    // 25088 or 36864 bytes
+    static constexpr int SLOTS = WIDE ? 5 : 3;
+    static constexpr int SMEM = W_BYTES + SLOTS * SLOT + 1024;
+};
 
 // K-major shared-memory matrix descriptor without swizzle: 8-row core
 // matrices of 16-byte rows; `lbo` = bytes between core matrices along K,
@@ -328,37 +180,60 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
 }
 
 struct RingUnit {
-    int n, z, x0, fa, fb;
+    int n, z0, x0, fa, fb;
 };
 
+template <bool WIDE>
 __device__ __forceinline__ RingUnit ring_unit(const ConvDims &d, int u)
 {
-    const int nfc = (d.F + RING_FCH - 1) / RING_FCH, nxb = d.X / RING_X;
+    const int nfc = (d.F + d.run - 1) / d.run, nxb = d.X / Tile<WIDE>::X, nzb = d.Z / Tile<WIDE>::Z;
     RingUnit r;
     const int fc = u % nfc;
     u /= nfc;
-    r.x0 = (u % nxb) * RING_X;
+    r.x0 = (u % nxb) * Tile<WIDE>::X;
     u /= nxb;
-    r.z = u % d.Z;
-    r.n = u / d.Z;
-    r.fa = fc * RING_FCH;
-    r.fb = min(d.F, r.fa + RING_FCH);
+    r.z0 = (u % nzb) * Tile<WIDE>::Z;
+    r.n = u / nzb;
+    r.fa = fc * d.run;
+    r.fb = min(d.F, r.fa + d.run);
     return r;
 }
 
-__device__ __forceinline__ int ring_slot(int g) { return (g + 10) % RING_SLOTS; }  // g >= -2
+constexpr int RING_ACC = 16;                         // accumulators of 32 columns in tensor memory
+constexpr int RING_TMEM = RING_ACC * C;
+constexpr int RING_WTAP = 5 * W_TAP_BYTES;           // weights of one (dz, dx), all dt
+constexpr int RING_WCHUNK = RING_WTAP / 4;           // WIDE: of 8 input channels
+constexpr uint32_t kRingIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TILE_M >> 4) << 24);  // | N / 8 << 17
 
-template <int EPI>
-__global__ void __launch_bounds__(CONV_THREADS, 1)
-    conv_ring_kernel(const __grid_constant__ CUtensorMap in_map, const __nv_bfloat16 *__restrict__ wchunk,
-                     const ConvDims d, int units, const float *__restrict__ bias, void *__restrict__ out,
-                     const __nv_bfloat16 *__restrict__ mask, int *__restrict__ status)
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                         uint32_t accumulate)
 {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// input frames of a unit: those in the volume that reach its outputs (a frame
+// outside contributes nothing)
+__device__ __forceinline__ int ring_g0(const RingUnit &r) { return max(0, r.fa - 2); }
+__device__ __forceinline__ int ring_g1(const RingUnit &r, int F) { return min(F - 1, r.fb + 1); }
+
+template <int EPI, bool WIDE>
+__global__ void __launch_bounds__(CONV_THREADS, 1)
+    conv_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant__ CUtensorMap w_map,
+                const __nv_bfloat16 *__restrict__ wchunk, const ConvDims d, int units, const float *__restrict__ bias, void *__restrict__ out,
+                const __nv_bfloat16 *__restrict__ mask, int *__restrict__ status)
+{
+    using T = Tile<WIDE>;
+    constexpr int RING_SLOTS = T::SLOTS;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char *w_s = base;
     unsigned char *ring = base + W_BYTES;
-    __shared__ __align__(8) uint64_t slot_full[RING_SLOTS], slot_free[RING_SLOTS], acc_full[2], acc_empty[2], w_bar;
+    __shared__ __align__(8) uint64_t slot_full[RING_SLOTS], slot_free[RING_SLOTS], acc_full[RING_ACC], acc_empty[RING_ACC], w_bar;
     __shared__ uint32_t tmem_base;
     __shared__ int s_fail;
     __shared__ float s_bias[C];
@@ -369,7 +244,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
             mbar_init(&slot_full[s], 1);
             mbar_init(&slot_free[s], 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < RING_ACC; ++b) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], 4);
         }
@@ -380,7 +255,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     if (threadIdx.x < C) s_bias[threadIdx.x] = bias ? bias[threadIdx.x] : 0.0f;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(TMEM_COLS)
+                     "r"(RING_TMEM)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -391,34 +266,40 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
 
     if (warp == 0) {
         if (lane == 0) {
-            // ---- producer: weights once, then the frames of each unit in order.
-            // Per slot: bit s of `loaded` = the slot has been filled before,
-            // bit s of `par` = parity of its fill count.
+            // ---- producer: weights once, then the frames of each unit in order,
+            // load i into slot i % RING_SLOTS
             mbar_expect_tx(&w_bar, W_BYTES);
-            bulk_load(w_s, wchunk, W_BYTES, &w_bar);
-            uint32_t loaded = 0, par = 0;
+            if constexpr (WIDE) {
+                // [tap][4 chunks][32 rows][8] to [dz, dx][chunk][2 - dt][row][8]
+                for (int t = 0; t < NTAP; ++t)
+                    for (int c = 0; c < 4; ++c)
+                        bulk_load(w_s + (t % 9) * RING_WTAP + c * RING_WCHUNK + (4 - t / 9) * (RING_WCHUNK / 5),
+                                  (const unsigned char *)wchunk + (t * 4 + c) * (W_TAP_BYTES / 4), W_TAP_BYTES / 4, &w_bar);
+            } else {
+                for (int t = 0; t < NTAP; ++t)  // tap (dt, dz, dx) to block 2 - dt of (dz, dx)
+                    tma_load_2d(w_s + ((t % 9) * 5 + 4 - t / 9) * W_TAP_BYTES, &w_map, &w_bar, 0, t * C);
+            }
+            uint32_t i = 0;
             bool fail = false;
             for (int u = blockIdx.x; u < units && !fail; u += gridDim.x) {
-                const RingUnit r = ring_unit(d, u);
-                for (int g = r.fa - 2; g <= r.fb + 1; ++g) {
-                    const int s = ring_slot(g);
-                    // the previous fill of this slot has count parity par ^ 1 ... its release phase
-                    if (((loaded >> s) & 1u) && !mbar_wait(&slot_free[s], ((par >> s) & 1u) ^ 1u)) {
+                const RingUnit r = ring_unit<WIDE>(d, u);
+                for (int g = ring_g0(r); g <= ring_g1(r, d.F); ++g, ++i) {
+                    const int s = i % RING_SLOTS;
+                    if (!mbar_wait(&slot_free[s], ((i / RING_SLOTS) & 1u) ^ 1u)) {
                         fail = true;
                         break;
                     }
-                    mbar_expect_tx(&slot_full[s], 4 * RING_BOX);
-                    unsigned char *dst = ring + s * RING_SLOT;
-                    for (int k = 0; k < 4; ++k)
-                        tma_load_5d(dst + k * RING_CHUNK, &in_map, &slot_full[s], 8 * k, r.x0 - 1, r.z - 1, g, r.n);
-                    loaded |= 1u << s;
-                    par ^= 1u << s;
+                    mbar_expect_tx(&slot_full[s], T::NBOX * T::BOX);
+                    unsigned char *dst = ring + s * T::SLOT;
+                    for (int k = 0; k < T::NBOX; ++k)
+                        tma_load_5d(dst + k * T::STRIDE, &in_map, &slot_full[s], WIDE ? 8 * k : 0,
+                                    WIDE ? r.x0 - 1 : r.x0 - 1 + k, r.z0 - 1, g, r.n);
                 }
             }
             if (fail) {
                 s_fail = 1;
-                for (int s = 0; s < RING_SLOTS; ++s)  // let issued copies land
-                    if ((loaded >> s) & 1u) mbar_wait(&slot_full[s], ((par >> s) & 1u) ^ 1u);
+                for (uint32_t k = i > RING_SLOTS ? i - RING_SLOTS : 0; k < i; ++k)  // let issued copies land
+                    mbar_wait(&slot_full[k % RING_SLOTS], (k / RING_SLOTS) & 1u);
                 mbar_wait(&w_bar, 0);
             }
         }
@@ -429,68 +310,85 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
             // field (addresses stay below 256 KB, so the field never carries).
             bool fail = !mbar_wait(&w_bar, 0);
             tc_fence_after();
-            uint32_t wpar = 0;  // bit s: parity of the waits on slot s so far
-            int j = 0;
-            const uint64_t ring_d = nosw_desc(smem_u32(ring), RING_CHUNK, 128);
-            const uint64_t w_d = nosw_desc(smem_u32(w_s), C * 16, 128);
+            uint32_t i = 0, jb = 0;  // loads consumed; outputs of the units before this one
+            const uint64_t ring_d = WIDE ? nosw_desc(smem_u32(ring), T::STRIDE, 128) : sw64_desc(smem_u32(ring));
+            const uint64_t w_d = WIDE ? nosw_desc(smem_u32(w_s), RING_WCHUNK, 128) : sw64_desc(smem_u32(w_s));
+            constexpr int BLOCK = WIDE ? C * 16 : W_TAP_BYTES;  // weight bytes between outputs
             for (int u = blockIdx.x; u < units && !fail; u += gridDim.x) {
-                const RingUnit r = ring_unit(d, u);
-                for (int f = r.fa; f < r.fb && !fail; ++f, ++j) {
-                    const int buf = j & 1;
-                    if (!mbar_wait(&acc_empty[buf], (((uint32_t)j >> 1) & 1u) ^ 1u)) { fail = true; break; }
-                    tc_fence_after();
-                    const uint32_t acc = tmem + (uint32_t)(buf * C);
-#pragma unroll
-                    for (int dt = -2; dt <= 2; ++dt) {
-                        const int s = ring_slot(f + dt);
-                        if (f == r.fa || dt == 2) {  // first use of frame f + dt in this unit
-                            if (!mbar_wait(&slot_full[s], (wpar >> s) & 1u)) { fail = true; break; }
-                            wpar ^= 1u << s;
-                            tc_fence_after();
-                        }
-                        const uint64_t a0 = ring_d + (uint64_t)((s * RING_SLOT) >> 4);
-#pragma unroll
-                        for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-                            for (int dx = -1; dx <= 1; ++dx) {
-                                const int t = (dt + 2) * 9 + (dz + 1) * 3 + (dx + 1);
-                                const uint64_t ad = a0 + (uint64_t)((((1 + dz) * RING_W + 1 + dx) * 16) >> 4);
-                                const uint64_t bd = w_d + (uint64_t)((t * W_TAP_BYTES) >> 4);
-                                mma_bf16_n32(acc, ad, bd, t > 0 ? 1u : 0u);
-                                mma_bf16_n32(acc, ad + (uint64_t)((2 * RING_CHUNK) >> 4),
-                                             bd + (uint64_t)((2 * C * 16) >> 4), 1u);
-                            }
-                        if (dt == -2) mma_commit(&slot_free[ring_slot(f - 2)]);  // its last use
+                const RingUnit r = ring_unit<WIDE>(d, u);
+                const int g0 = ring_g0(r), g1 = ring_g1(r, d.F);
+                for (int g = g0; g <= g1; ++g, ++i) {
+                    // outputs lo .. hi take frame g; from `fresh` on for the first time
+                    const int lo = max(r.fa, g - 2), hi = min(r.fb - 1, g + 2);
+                    const int fresh = g == g0 ? lo : g + 2;
+                    for (int f = fresh; f <= hi && !fail; ++f) {
+                        const uint32_t j = jb + (uint32_t)(f - r.fa);
+                        if (!mbar_wait(&acc_empty[j % RING_ACC], ((j / RING_ACC) & 1u) ^ 1u)) fail = true;
                     }
-                    if (fail) break;
-                    mma_commit(&acc_full[buf]);
+                    const int s = i % RING_SLOTS;
+                    if (fail || !mbar_wait(&slot_full[s], (i / RING_SLOTS) & 1u)) { fail = true; break; }
+                    tc_fence_after();
+                    const uint64_t a0 = ring_d + (uint64_t)((s * T::SLOT) >> 4);
+                    // K step 0 or steps 1 .. 17 (step = 2 tap + half of the channels) of
+                    // outputs fa .. fb, in two runs where the accumulator ring wraps
+                    auto run = [&](int fa, int fb, bool first) {
+                        const uint32_t c0 = (jb + (uint32_t)(fa - r.fa)) % RING_ACC;
+                        const int n = fb - fa + 1, n1 = min(n, RING_ACC - (int)c0);
+                        for (int part = 0; part < 2; ++part) {
+                            const int m = part ? n - n1 : n1;
+                            if (m <= 0) break;
+                            const uint32_t acc = part ? tmem : tmem + c0 * C;
+                            const uint32_t idesc = kRingIdesc | ((uint32_t)(m * C / 8) << 17);
+                            const uint64_t bd = w_d + (uint64_t)(((fa - (g - 2) + (part ? n1 : 0)) * BLOCK) >> 4);
+                            if (first) {
+                                mma_bf16(acc, a0, bd, idesc, fa >= fresh ? 0u : 1u);
+                                continue;
+                            }
+#pragma unroll
+                            for (int k = 1; k < 18; ++k) {
+                                const int dz = k / 6, dx = (k / 2) % 3, kk = k & 1;
+                                // second 16 channels: two chunks on, or 32 bytes on in the row
+                                const int ao = WIDE ? (dz * T::W + dx) * 16 + kk * 2 * T::STRIDE
+                                                    : dx * T::STRIDE + dz * TILE_X * ROWB + kk * 32;
+                                const int bo = (k / 2) * RING_WTAP + kk * (WIDE ? 2 * RING_WCHUNK : 32);
+                                mma_bf16(acc, a0 + (uint64_t)(ao >> 4), bd + (uint64_t)(bo >> 4), idesc, 1u);
+                            }
+                        }
+                    };
+                    if (lo < fresh) run(lo, min(hi, fresh - 1), true);
+                    if (fresh <= hi) run(fresh, hi, true);
+                    run(lo, hi, false);
+                    mma_commit(&slot_free[s]);
+                    // outputs that frame g completes
+                    for (int f = lo; f <= hi; ++f)
+                        if (f == g - 2 || g == g1) mma_commit(&acc_full[(jb + (uint32_t)(f - r.fa)) % RING_ACC]);
                 }
-                if (fail) break;
-                for (int g = r.fb - 2; g <= r.fb + 1; ++g) mma_commit(&slot_free[ring_slot(g)]);
+                jb += (uint32_t)(r.fb - r.fa);
             }
             if (fail) s_fail = 1;
         }
     } else {
-        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = pixels x0 + 32 (w % 4) + lane
+        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = pixels x0 + 32 (w % 4) + lane (WIDE)
+        // or depth row z0 + w % 4
         const int q = warp & 3;
-        int j = 0;
+        uint32_t j = 0;
         bool stop = false;
         for (int u = blockIdx.x; u < units && !stop; u += gridDim.x) {
-            const RingUnit r = ring_unit(d, u);
+            const RingUnit r = ring_unit<WIDE>(d, u);
             for (int f = r.fa; f < r.fb; ++f, ++j) {
-                const int buf = j & 1;
-                if (!warp_wait(&acc_full[buf], ((uint32_t)j >> 1) & 1u)) {
+                const uint32_t buf = j % RING_ACC;
+                if (!warp_wait(&acc_full[buf], (j / RING_ACC) & 1u)) {
                     if (lane == 0) s_fail = 1;
                     stop = true;
                     break;
                 }
                 tc_fence_after();
                 float v[32];
-                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * C), v);
+                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + buf * C, v);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_empty[buf]);
-                const int64_t vox = (((int64_t)r.n * d.F + f) * d.Z + r.z) * d.X + r.x0 + q * 32 + lane;
+                const int64_t vox = (((int64_t)r.n * d.F + f) * d.Z + r.z0 + (WIDE ? 0 : q)) * d.X + r.x0 + (WIDE ? q * 32 : 0) + lane;
                 epilogue_store<EPI>(v, s_bias, vox, out, mask);
             }
         }
@@ -499,7 +397,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(RING_TMEM) : "memory");
     }
     if (threadIdx.x == 0 && s_fail) atomicExch(status, (int)FQ_ERR_TIMEOUT);
 }
@@ -509,7 +407,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
 // pass (rows = out channel, 32 in channels each) and for the data gradient
 // (kernel flipped in all three axes: tap 44 - t; rows = in channel).
 // The chunked images hold the same tiles as [tap][K chunk of 8][row][8]
-// (16-byte core-matrix rows) for the frame-ring kernel.
+// (16-byte core-matrix rows) for the WIDE tile.
 __global__ void pack_weights_kernel(const float *__restrict__ w, __nv_bfloat16 *__restrict__ wf,
                                     __nv_bfloat16 *__restrict__ wb, __nv_bfloat16 *__restrict__ wfc,
                                     __nv_bfloat16 *__restrict__ wbc)
@@ -956,10 +854,10 @@ fq_status encode_act_map(CUtensorMap *map, const void *p, int N, int F, int Z, i
     cuuint64_t dims[5] = {(cuuint64_t)C, (cuuint64_t)X, (cuuint64_t)Z, (cuuint64_t)F, (cuuint64_t)N};
     cuuint64_t strides[4] = {(cuuint64_t)C * 2, (cuuint64_t)X * C * 2, (cuuint64_t)Z * X * C * 2,
                              (cuuint64_t)F * Z * X * C * 2};
-    // per-tap kernel: 32 channels x 32 pixels x 4 rows, 64-byte swizzle;
-    // frame-ring kernel: 8 channels x 130 pixels x 3 rows, no swizzle
-    cuuint32_t box_tap[5] = {(cuuint32_t)C, (cuuint32_t)TILE_X, (cuuint32_t)TILE_Z, 1, 1};
-    cuuint32_t box_ring[5] = {8, (cuuint32_t)RING_W, 3, 1, 1};
+    // 32 channels x 32 pixels x 6 rows, 64-byte swizzle; WIDE: 8 channels x 130
+    // pixels x 3 rows, no swizzle
+    cuuint32_t box_tap[5] = {(cuuint32_t)C, (cuuint32_t)TILE_X, (cuuint32_t)TILE_Z + 2, 1, 1};
+    cuuint32_t box_ring[5] = {8, (cuuint32_t)Tile<true>::W, 3, 1, 1};
     cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(p), dims, strides,
                      ring ? box_ring : box_tap, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -1017,47 +915,57 @@ int num_sms()
     return sms;
 }
 
-// One convolution of layer `layer` (forward or data-gradient kernel): the
-// frame-ring kernel when the width is a multiple of 128, else the per-tap one.
+// Frames per work unit: a run of L output frames walks L + 4 input frames (the
+// first and last with part of the outputs), so few long runs cost least and
+// enough runs for every SM the least time.
+int conv_run(int columns, int F, int sms)
+{
+    int best = F;
+    double cost = 1e300;
+    for (int runs = 1; runs <= F; ++runs) {
+        const int len = (F + runs - 1) / runs, units = columns * ((F + len - 1) / len);
+        const double c = (double)((units + sms - 1) / sms) * (len + 3.0);
+        if (c < cost) { cost = c; best = len; }
+    }
+    return best;
+}
+
+// One convolution of layer `layer` (forward or data-gradient kernel).
+template <bool WIDE>
+fq_status launch_conv(int epi, const CUtensorMap &in_map, const CUtensorMap &w_map, const __nv_bfloat16 *wc, ConvDims d,
+                      const float *bias, void *out, const __nv_bfloat16 *mask, int *status, cudaStream_t st)
+{
+    using T = Tile<WIDE>;
+    const int columns = d.N * (d.Z / T::Z) * (d.X / T::X);
+    d.run = conv_run(columns, d.F, num_sms());
+    const int units = columns * ((d.F + d.run - 1) / d.run);
+    const int grid = units < num_sms() ? units : num_sms();
+    auto launch = [&](auto kern) -> fq_status {
+        fq_status r = fqi::cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM),
+                                      "cnn: smem attribute");
+        if (r) return r;
+        kern<<<grid, CONV_THREADS, T::SMEM, st>>>(in_map, w_map, wc, d, units, bias, out, mask, status);
+        return fqi::launch_check("cnn: conv");
+    };
+    if (epi == EPI_RELU_BF16) return launch(conv_kernel<EPI_RELU_BF16, WIDE>);
+    if (epi == EPI_LINEAR_F32) return launch(conv_kernel<EPI_LINEAR_F32, WIDE>);
+    return launch(conv_kernel<EPI_MASK_BF16, WIDE>);
+}
+
 fq_status conv(int epi, const void *in, const void *params, int layer, bool backward, const float *bias, void *out,
                const __nv_bfloat16 *mask, const ConvDims &d, int *status, cudaStream_t st)
 {
     const ParamLayout L = param_layout();
     const char *pb = (const char *)params;
     const size_t lo = (size_t)layer * NTAP * C * C * 2;
-    const bool ring = d.X % RING_X == 0;
-    CUtensorMap in_map;
-    fq_status s = encode_act_map(&in_map, in, d.N, d.F, d.Z, d.X, ring);
+    const bool wide = d.Z % TILE_Z != 0;  // then X is a multiple of 128
+    CUtensorMap in_map, w_map;
+    fq_status s = encode_act_map(&in_map, in, d.N, d.F, d.Z, d.X, wide);
+    if (!s) s = encode_w_map(&w_map, pb + (backward ? L.wb_bytes_off : L.wf_bytes_off) + lo);
     if (s) return s;
-    if (ring) {
-        const __nv_bfloat16 *wc = (const __nv_bfloat16 *)(pb + (backward ? L.wbc_bytes_off : L.wfc_bytes_off) + lo);
-        const int units = d.N * d.Z * (d.X / RING_X) * ((d.F + RING_FCH - 1) / RING_FCH);
-        const int grid = units < num_sms() ? units : num_sms();
-        auto launch = [&](auto kern) -> fq_status {
-            fq_status r = fqi::cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                               RING_SMEM), "cnn: smem attribute");
-            if (r) return r;
-            kern<<<grid, CONV_THREADS, RING_SMEM, st>>>(in_map, wc, d, units, bias, out, mask, status);
-            return fqi::launch_check("cnn: conv (frame ring)");
-        };
-        if (epi == EPI_RELU_BF16) return launch(conv_ring_kernel<EPI_RELU_BF16>);
-        if (epi == EPI_LINEAR_F32) return launch(conv_ring_kernel<EPI_LINEAR_F32>);
-        return launch(conv_ring_kernel<EPI_MASK_BF16>);
-    }
-    CUtensorMap w_map;
-    s = encode_w_map(&w_map, pb + (backward ? L.wb_bytes_off : L.wf_bytes_off) + lo);
-    if (s) return s;
-    const int grid = d.tiles < num_sms() ? d.tiles : num_sms();
-    auto launch = [&](auto kern) -> fq_status {
-        fq_status r = fqi::cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           CONV_SMEM), "cnn: smem attribute");
-        if (r) return r;
-        kern<<<grid, CONV_THREADS, CONV_SMEM, st>>>(in_map, w_map, d, bias, out, mask, status);
-        return fqi::launch_check("cnn: conv");
-    };
-    if (epi == EPI_RELU_BF16) return launch(conv_tc_kernel<EPI_RELU_BF16>);
-    if (epi == EPI_LINEAR_F32) return launch(conv_tc_kernel<EPI_LINEAR_F32>);
-    return launch(conv_tc_kernel<EPI_MASK_BF16>);
+    const __nv_bfloat16 *wc = (const __nv_bfloat16 *)(pb + (backward ? L.wbc_bytes_off : L.wfc_bytes_off) + lo);
+    return wide ? launch_conv<true>(epi, in_map, w_map, wc, d, bias, out, mask, status, st)
+                : launch_conv<false>(epi, in_map, w_map, wc, d, bias, out, mask, status, st);
 }
 
 template <int NT>
@@ -1081,7 +989,7 @@ fq_status launch_wgrad(const void *x, const void *dy, const ConvDims &d, int n_p
 fq_status check_dims(int N, int F, int Z, int X, const char *who)
 {
     FQ_REQUIRE(N >= 1 && F >= 1 && Z >= 1 && X >= TILE_X, FQ_ERR_SHAPE, "%s: bad volume size", who);
-    FQ_REQUIRE(X % RING_X == 0 || (Z % TILE_Z == 0 && X % TILE_X == 0), FQ_ERR_SHAPE,
+    FQ_REQUIRE(X % Tile<true>::X == 0 || (Z % TILE_Z == 0 && X % TILE_X == 0), FQ_ERR_SHAPE,
                "%s: X must be a multiple of 128, or of 32 with Z a multiple of 4 (got Z %d, X %d)", who, Z, X);
     FQ_REQUIRE(tile_count(N, F, Z, X) < ((int64_t)1 << 31), FQ_ERR_SHAPE, "%s: too many tiles",
                who);
@@ -1092,7 +1000,7 @@ ConvDims make_dims(int N, int F, int Z, int X)
 {
     ConvDims d;
     d.N = N; d.F = F; d.Z = Z; d.X = X;
-    d.tiles = N * F * (Z / TILE_Z) * (X / TILE_X);
+    d.run = F;
     d.zb = (Z + TILE_Z - 1) / TILE_Z;
     d.xb = X / TILE_X;
     d.walk_tiles = (int)tile_count(N, F, Z, X);

@@ -1,11 +1,13 @@
 """The hot kernels at the edges of their layouts: angle blocks and record
 segments of the RF kernel, pixel panels and column blocks of the FP32 Gram,
-frame groups and voxel pairs of the 16-bit delay-and-sum."""
+frame groups and voxel pairs of the 16-bit delay-and-sum, accumulator runs
+of the convolution."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
+from oracle import cnn as ocnn
 from paper_2509_05464_gb300 import build as fqbuild
 from paper_2509_05464_gb300 import fq
 from paper_2509_05464_gb300 import workload as W
@@ -80,3 +82,26 @@ def test_das_frame_groups_and_voxel_pairs(dt, u, F, nx, matrix):
     assert rel_l2(got.double().cpu().numpy(), want.double().cpu().numpy()) <= 4 * u
     for f in {0, F // 2, F - 1}:
         assert rel_l2(got[:, f].double().cpu().numpy(), want[:, f].double().cpu().numpy()) <= 8 * u
+
+
+# runs of one to many frames (every number of new and finished outputs), both
+# tiles (a depth that is not a multiple of 4 takes the 128-pixel rows)
+@pytest.mark.parametrize("shape", [(1, 1, 4, 32), (1, 2, 4, 32), (1, 3, 3, 128), (2, 4, 1, 128), (1, 5, 8, 96),
+                                   (1, 9, 4, 160), (1, 33, 2, 128), (3, 17, 4, 32)])
+def test_conv_frame_runs(shape):
+    n, F, Z, X = shape
+    rng = np.random.default_rng(sum(shape))
+    layers = [(rng.standard_normal((45, 32, 32)) * np.sqrt(2.0 / 1440), rng.standard_normal(32) * 0.1) for _ in range(4)]
+    net = fq.CNN(3)
+    net.set_weights(layers)
+    x = torch.from_numpy(rng.standard_normal(shape + (32,)).astype(np.float32)).bfloat16().cuda()
+    w = torch.from_numpy(layers[1][0].astype(np.float32)).bfloat16().double().numpy()
+    b = layers[1][1].astype(np.float32).astype(np.float64)
+    x64 = x.double().cpu().numpy()
+    ref = np.stack([ocnn.conv3d(x64[i], w, b) for i in range(n)])
+    out = torch.empty(shape + (32,), dtype=torch.float32, device="cuda")
+    fq.fq_cnn_conv(fq.CNN_MODE_LINEAR, x, net, 1, 0, out)
+    torch.cuda.synchronize()
+    assert int(net.status.item()) == 0
+    # FP32 sums of at most 1440 exact products of BF16 values
+    assert np.abs(out.double().cpu().numpy() - ref).max() <= 1e-5 * np.abs(ref).max()
