@@ -777,7 +777,7 @@ def run_cnn(args, rank, world, local):
                    "data_generation_s": gen_s,
                    "l2": "inference working set (activations 0.84 GB per layer) far above L2"},
         "quality": quality,
-        "roofline": {"bound": "tensor", "kernel": "conv_ring_kernel", "achieved": ach, "peak": peak,
+        "roofline": {"bound": "tensor", "kernel": "conv_kernel", "achieved": ach, "peak": peak,
                      "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
                      "peak_source": f"bf16_tflops of {src} peaks (cuBLAS burst)",
                      "work": f"2 x {mac_true} MAC per voxel (the 2-32-32-32-2 network); the kernels execute "

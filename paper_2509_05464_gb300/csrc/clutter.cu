@@ -28,6 +28,7 @@ struct ClutterLayout {
 
 constexpr int kGramThreads = 256;
 constexpr int kGramPx = 16;     // pixels per shared-memory panel of the Gram kernel
+constexpr int kGramCtas = 3;    // CTAs of the Gram kernel per SM
 constexpr int kGramRound = 32;  // pixel chunks are multiples of this
 
 // 4 x 4 complex blocks of the upper triangle (block rows bi <= bj)
@@ -41,15 +42,15 @@ inline size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 int gram_chunks(int64_t P, int F)
 {
-    // two CTAs per SM (gram_partial_kernel), all in one wave
-    int want = 2 * 152 / gram_parts(F);
+    // the CTAs that fit (gram_partial_kernel), all in one wave
+    int want = kGramCtas * 152 / gram_parts(F);
     int64_t max_chunks = (P + kGramRound - 1) / kGramRound;
     if (want > max_chunks) want = (int)max_chunks;
     if (want < 1) want = 1;
     return want;
 }
 
-bool eig_in_smem(int F) { return (size_t)F * (F + 1) / 2 * sizeof(float2) <= 190 * 1024; }
+__host__ __device__ inline bool eig_in_smem(int F) { return (size_t)F * (F + 1) / 2 * sizeof(float2) <= 190 * 1024; }
 
 // Operand bytes of the tensor-core Gram modes (0 = CUDA-core FP32 Gram).
 int tc_esz(int gram_mode) { return gram_mode == FQ_GRAM_BF16 ? 2 : (gram_mode == FQ_GRAM_TF32 ? 4 : 0); }
@@ -97,9 +98,9 @@ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y
 // cp.async: S is read once per part (2 parts at 100 frames, 5 at 200), and
 // only blocks of the triangle are computed (F = 100: 5200 of 5050 products;
 // 32 x 32 tiles with 2 x 2 outputs per thread computed 10240 and read two
-// 8-byte operands per complex product).  2^21 pixels x 100 frames: 6.9 -> 3.2
-// ms; 65536 x 200: 0.60 -> 0.31 ms (57% of the FP32 rate for the products of
-// the triangle).  A panel row is two planes, columns
+// 8-byte operands per complex product).  2^21 pixels x 100 frames: 6.9 -> 2.8
+// ms; 65536 x 200: 0.60 -> 0.30 ms, with three CTAs per SM (two 3.1; FMA pipe
+// 51% busy, the rest issue: four loads, the panels' copies and barriers).  A panel row is two planes, columns
 // (4b, 4b + 1) and (4b + 2, 4b + 3), so that the 16-byte loads of 32
 // consecutive blocks are contiguous.
 __device__ __forceinline__ void gram_stage(const float *__restrict__ S, int64_t p0, int64_t pend, int F, int nb, float4 *buf)
@@ -108,9 +109,17 @@ __device__ __forceinline__ void gram_stage(const float *__restrict__ S, int64_t 
     if ((F & 1) == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0) {  // rows of whole 16-byte units
         const int U = F >> 1;
         const float *src = S + p0 * F * 2;
+        // (pixel, unit) of this thread's next copy by steps of 256 units
+        const int dp = kGramThreads / U, du = kGramThreads - dp * U;
+        int px = threadIdx.x / U, u = threadIdx.x - px * U;
         for (int i = threadIdx.x; i < n * U; i += kGramThreads) {
-            const int px = i / U, u = i - px * U;
             fqi::cp_async<16>(buf + px * 2 * nb + (u & 1) * nb + (u >> 1), src + (size_t)i * 4);
+            px += dp;
+            u += du;
+            if (u >= U) {
+                u -= U;
+                ++px;
+            }
         }
     } else {
         const float *src = S + p0 * F * 2;
@@ -206,7 +215,7 @@ __device__ __forceinline__ void gram_part(const T *__restrict__ S, int64_t P, in
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kGramThreads, 2) gram_partial_kernel(const T *__restrict__ S, int64_t P, int F,
+__global__ void __launch_bounds__(kGramThreads, kGramCtas) gram_partial_kernel(const T *__restrict__ S, int64_t P, int F,
                                                                        int64_t chunk_len, float2 *__restrict__ part)
 {
     extern __shared__ float4 panel[];
@@ -255,172 +264,705 @@ __global__ void __launch_bounds__(kGramThreads) gram_reduce_kernel(const float2 
 }
 
 // ------------------------------------------------------------ eigen (1 CTA) --
-constexpr int kEigThreads = 1024;
+constexpr int kEigThreads = 1024;  // all eigenvectors (QL)
+constexpr int kTopThreads = 512;   // eigenvalues and the first vectors
 
 __device__ __forceinline__ int pidx(int i, int j) { return i * (i + 1) / 2 + j; }  // i >= j
 
-// block-wide sum of one float per thread
-__device__ float block_sum(float v, float *red)
+// V[:, j] = H_0 ... H_{F-3} D Z[:, perm[j]] for j < ncol: warp per column, NQ
+// values per lane.  With `buf` (shared memory for 2 x nbuf reflectors) the CTA
+// copies the next nbuf reflectors while the warps apply the last ones (read
+// one by one from global memory they took 0.09 ms at 200 frames); else they
+// are read in place.  Called by every thread of the CTA.
+template <int NQ>
+__device__ __forceinline__ void back_transform_nq(int F, int ncol, const float *Z, int zs, const int *perm,
+                                                  const float2 *delta, const float2 *__restrict__ hv,
+                                                  const float *__restrict__ tau_g, float2 *__restrict__ V,
+                                                  float2 *__restrict__ Vt, float2 *buf, int nbuf, int lane, int wid, int nw)
 {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        float x = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0f;
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) red[32] = x;
-    }
-    __syncthreads();
-    return red[32];
-}
-
-// V[:, j] = H_0 ... H_{F-3} D Z[:, perm[j]] for j < ncol (warp per column).
-__device__ void back_transform(int F, int ncol, const float *Z, int zs, const int *perm, const float2 *delta,
-                               const float2 *__restrict__ hv, const float *__restrict__ tau_g, float2 *__restrict__ V,
-                               float2 *__restrict__ Vt, int lane, int wid, int nw)
-{
-    for (int j = wid; j < ncol; j += nw) {
-        const int src = perm[j];
-        float2 y[16];  // F <= 512: 16 values per lane
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            int i = lane + 32 * q;
-            y[q] = i < F ? make_float2(delta[i].x * Z[i * zs + src], delta[i].y * Z[i * zs + src]) : make_float2(0, 0);
+    const int n = F > 2 ? F - 2 : 0;  // reflectors; number r is H_{n-1-r}
+    auto stage = [&](int c) {
+        float2 *b = buf + (size_t)(c & 1) * nbuf * F;
+        const int r0 = c * nbuf, cnt = min(nbuf, n - r0);
+        for (int t = threadIdx.x; t < cnt * F; t += blockDim.x) {
+            const int r = t / F, i = t - r * F, k = n - 1 - (r0 + r);
+            if (i > k) fqi::cp_async<8>(b + t, hv + (size_t)k * F + i);
+            else b[t] = make_float2(0, 0);
         }
-        for (int k = F - 3; k >= 0; --k) {
-            const float t = tau_g[k];
-            if (t == 0.0f) continue;
-            const float2 *v = hv + (size_t)k * F;
-            float2 s = make_float2(0, 0);
+        fqi::cp_async_commit();
+    };
+    for (int j0 = 0; j0 < ncol; j0 += nw) {
+        const int j = j0 + wid;
+        const bool on = j < ncol;
+        float2 y[NQ];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                int i = lane + 32 * q;
-                if (i > k && i < F) {
-                    float2 vi = v[i];
-                    s.x += vi.x * y[q].x + vi.y * y[q].y;  // conj(v) y
-                    s.y += vi.x * y[q].y - vi.y * y[q].x;
-                }
+        for (int q = 0; q < NQ; ++q) {
+            const int i = lane + 32 * q;
+            const float z = on && i < F ? Z[i * zs + perm[j]] : 0.0f;
+            y[q] = i < F ? make_float2(delta[i].x * z, delta[i].y * z) : make_float2(0, 0);
+        }
+        auto apply = [&](const float2 *v, int k, bool padded) {
+            const float t = tau_g[k];
+            float2 x[NQ], s = make_float2(0, 0);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int i = lane + 32 * q;
+                x[q] = i < F && (padded || i > k) ? v[i] : make_float2(0, 0);
+                cmac(s, x[q].x, x[q].y, y[q].x, y[q].y);
             }
             for (int o = 16; o > 0; o >>= 1) {
                 s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
                 s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
             }
-            s.x *= t;
-            s.y *= t;
+            s.x *= -t;
+            s.y *= -t;
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                int i = lane + 32 * q;
-                if (i > k && i < F) {
-                    float2 u = cmul(v[i], s);
-                    y[q].x -= u.x;
-                    y[q].y -= u.y;
-                }
+            for (int q = 0; q < NQ; ++q) {  // y -= t (v^H y) v
+                y[q].x = fmaf(x[q].x, s.x, fmaf(-x[q].y, s.y, y[q].x));
+                y[q].y = fmaf(x[q].x, s.y, fmaf(x[q].y, s.x, y[q].y));
             }
+        };
+        if (nbuf > 0) {
+            const int nc = (n + nbuf - 1) / nbuf;
+            if (nc > 0) stage(0);
+            for (int c = 0; c < nc; ++c) {
+                if (c + 1 < nc) stage(c + 1);
+                else fqi::cp_async_commit();
+                fqi::cp_async_wait<1>();
+                __syncthreads();
+                if (on)
+                    for (int r = 0; r < min(nbuf, n - c * nbuf); ++r)
+                        apply(buf + ((size_t)(c & 1) * nbuf + r) * F, n - 1 - c * nbuf - r, true);
+                __syncthreads();
+            }
+            fqi::cp_async_wait<0>();
+        } else if (on) {
+            for (int k = n - 1; k >= 0; --k) apply(hv + (size_t)k * F, k, false);
         }
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            int i = lane + 32 * q;
-            if (i < F) {
+        for (int q = 0; q < NQ; ++q) {
+            const int i = lane + 32 * q;
+            if (on && i < F) {
                 if (V) V[(size_t)i * F + j] = y[q];
                 Vt[(size_t)j * F + i] = y[q];
             }
         }
     }
 }
-
-// Number of eigenvalues of the real symmetric tridiagonal (d, e) below x
-// (Sturm count by the LDL^T pivot recurrence; tiny pivots are replaced by
-// -pivmin so that the count stays monotone).
-__device__ int sturm_below(const float *d, const float *e2, int n, float x, float pivmin)
+__device__ __forceinline__ void back_transform(int F, int ncol, const float *Z, int zs, const int *perm, const float2 *delta,
+                               const float2 *__restrict__ hv, const float *__restrict__ tau_g, float2 *__restrict__ V,
+                               float2 *__restrict__ Vt, float2 *buf, int nbuf, int lane, int wid, int nw)
 {
-    int cnt = 0;
-    float q = d[0] - x;
-    if (fabsf(q) < pivmin) q = -pivmin;
-    cnt += q < 0.0f;
-    for (int i = 1; i < n; ++i) {
-        q = (d[i] - x) - e2[i - 1] / q;
-        if (fabsf(q) < pivmin) q = -pivmin;
-        cnt += q < 0.0f;
-    }
-    return cnt;
+    if (F <= 128) back_transform_nq<4>(F, ncol, Z, zs, perm, delta, hv, tau_g, V, Vt, buf, nbuf, lane, wid, nw);
+    else if (F <= 224) back_transform_nq<7>(F, ncol, Z, zs, perm, delta, hv, tau_g, V, Vt, buf, nbuf, lane, wid, nw);
+    else back_transform_nq<16>(F, ncol, Z, zs, perm, delta, hv, tau_g, V, Vt, buf, nbuf, lane, wid, nw);
 }
 
-// The m-th smallest eigenvalue (0-based) by bisection on [lo, hi].
-__device__ float bisect_eig(const float *d, const float *e2, int n, int m, float lo, float hi, float pivmin)
+// Number of eigenvalues of the real symmetric tridiagonal (d, e) below x
+// (Sturm count by the signs of the LDL^T pivots).
+// The quotient is a product with the hardware reciprocal (1.5 units in its
+// last place, a relative change of e2 far below the tridiagonalisation's own
+// rounding).  No test of tiny pivots: a zero pivot gives an infinite quotient
+// and the next pivot the opposite sign, counted by sign bits (e2 > 0).  Two
+// points at once: their recurrences hide each other's latency.
+__device__ __forceinline__ void sturm_below(const float *d, const float *e2, int n, float xa, float xb, int &ca, int &cb)
 {
-    for (int it = 0; it < 80; ++it) {
-        const float mid = 0.5f * (lo + hi);
-        if (mid <= lo || mid >= hi) break;
-        if (sturm_below(d, e2, n, mid, pivmin) >= m + 1) hi = mid;
-        else lo = mid;
+    float qa = d[0] - xa, qb = d[0] - xb;
+    int c0 = (int)(__float_as_uint(qa) >> 31), c1 = (int)(__float_as_uint(qb) >> 31);
+#pragma unroll 4
+    for (int i = 1; i < n; ++i) {
+        const float b = e2[i - 1], di = d[i];
+        auto step = [&](float &q, float x, int &c) {
+            float r;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(q));
+            q = __fmaf_rn(-b, r, __fsub_rn(di, x));
+            c += (int)(__float_as_uint(q) >> 31);
+        };
+        step(qa, xa, c0);
+        step(qb, xb, c1);
     }
-    return 0.5f * (lo + hi);
+    ca = c0;
+    cb = c1;
+}
+
+// The eigenvalues in descending order by multisection on [lo, hi]: np threads
+// (a power of two that divides the warp) per eigenvalue evaluate two points of
+// its bracket each a round (np = 2 at 200 frames, where 13 warps still fit
+// under the latency of the pivot recurrences), until the bracket is below 2^-31 of
+// the largest row sum -- a hundredth of the tridiagonalisation's rounding --
+// or holds no other number.
+__device__ void multisect(const float *d, const float *e2, int n, float lo0, float hi0, float tnorm, float *lam)
+{
+    int np = 1;
+    while (np < 32 && 2 * np * n <= (int)blockDim.x / 2) np *= 2;
+    const int per = blockDim.x / np;  // eigenvalues of a pass
+    const int lane = threadIdx.x & 31, p = threadIdx.x % np;
+    const unsigned grp = (np == 32 ? 0xffffffffu : (1u << np) - 1u) << (lane - p);
+    const float width = tnorm * 4.6566129e-10f;
+    for (int j0 = 0; j0 < n; j0 += per) {
+        const int j = j0 + (int)threadIdx.x / np;
+        const int m = n - 1 - j;  // m-th smallest
+        float lo = lo0, hi = hi0;
+        bool act = j < n;
+        for (int it = 0; it < 80; ++it) {
+            const float mid = 0.5f * (lo + hi);
+            act = act && mid > lo && mid < hi && hi - lo > width;
+            if (!__any_sync(0xffffffffu, act)) break;
+            // the 2 np points, computed alike by every thread of the group
+            const float h = hi - lo, inv = 1.0f / (float)(2 * np + 1);
+            auto point = [&](int i) { return fminf(fmaxf(fmaf(h, (float)(i + 1) * inv, lo), lo), hi); };
+            int ca = 0, cb = 0;
+            if (act) sturm_below(d, e2, n, point(2 * p), point(2 * p + 1), ca, cb);
+            const unsigned ba = __ballot_sync(0xffffffffu, act && ca < m + 1) & grp;
+            const unsigned bb = __ballot_sync(0xffffffffu, act && cb < m + 1) & grp;
+            const int c = __popc(ba) + __popc(bb);  // points below the eigenvalue
+            if (act) {
+                const float nlo = c > 0 ? point(c - 1) : lo, nhi = c < 2 * np ? point(c) : hi;
+                lo = nlo;
+                hi = nhi;
+            }
+        }
+        if (j < n && p == 0) lam[j] = 0.5f * (lo + hi);
+    }
 }
 
 // One eigenvector of the real tridiagonal for eigenvalue sigma by inverse
-// iteration: Gaussian elimination with partial pivoting of T - sigma I
-// (kept in per-thread local arrays), three solves from a fixed pseudo-random
-// start, each normalised.  Writes column `col` of Z (row stride zs).
-__device__ void inverse_iteration(const float *d, const float *e, int n, float sigma, float tiny, int seed,
-                                  float *Z, int zs, int col, float *__restrict__ scr)
+// iteration: Gaussian elimination with partial pivoting of T - sigma I, three
+// solves from a fixed pseudo-random start, each normalised.  Writes column
+// `col` of Z (row stride zs).  scr: 6 n floats of shared or global memory
+// (1 / u0, u1, u2, multipliers, swaps, x), value i of array a at
+// scr[(a n + i) stride].
+__device__ __forceinline__ void inverse_iteration(const float *d, const float *e, int n, float sigma, float tiny, int seed,
+                                  float *Z, int zs, int col, float *scr, int stride)
 {
-    // scratch (global workspace, 6 n floats): u0, u1, u2, multipliers, swaps, x
-    float *u0 = scr, *u1 = scr + n, *u2 = scr + 2 * n, *ml = scr + 3 * n, *sw = scr + 4 * n, *x = scr + 5 * n;
+    auto at = [&](int a, int i) -> float & { return scr[(size_t)(a * n + i) * stride]; };
     float p0 = d[0] - sigma, p1 = n > 1 ? e[0] : 0.0f, p2 = 0.0f;
+    float c = p1, dn = n > 1 ? d[1] : 0.0f;
     for (int i = 0; i + 1 < n; ++i) {
-        const float c = e[i];                       // sub-diagonal of row i + 1
-        const float a1 = d[i + 1] - sigma;
+        // c = e[i]: sub-diagonal of row i + 1 (operands read a step ahead of the stores)
+        const float a1 = dn - sigma;
         const float b1 = (i + 2 < n) ? e[i + 1] : 0.0f;
-        if (fabsf(c) > fabsf(p0)) {
-            // pivot on row i + 1
-            const float mlt = p0 / c;
-            u0[i] = c; u1[i] = a1; u2[i] = b1; ml[i] = mlt; sw[i] = 1.0f;
-            p0 = p1 - mlt * a1;
-            p1 = p2 - mlt * b1;
-            p2 = 0.0f;
-        } else {
-            const float piv = fabsf(p0) < tiny ? (p0 < 0.0f ? -tiny : tiny) : p0;
-            const float mlt = c / piv;
-            u0[i] = piv; u1[i] = p1; u2[i] = p2; ml[i] = mlt; sw[i] = 0.0f;
-            p0 = a1 - mlt * p1;
-            p1 = b1 - mlt * p2;
-            p2 = 0.0f;
-        }
+        dn = (i + 2 < n) ? d[i + 2] : 0.0f;
+        const bool swap = fabsf(c) > fabsf(p0);  // pivot on row i + 1
+        const float piv = swap ? c : (fabsf(p0) < tiny ? (p0 < 0.0f ? -tiny : tiny) : p0);
+        const float r = 1.0f / piv;
+        const float mlt = (swap ? p0 : c) * r;
+        at(0, i) = r;
+        at(1, i) = swap ? a1 : p1;
+        at(2, i) = swap ? b1 : p2;
+        at(3, i) = mlt;
+        at(4, i) = swap ? 1.0f : 0.0f;
+        const float n0 = swap ? fmaf(-mlt, a1, p1) : fmaf(-mlt, p1, a1);
+        p1 = swap ? fmaf(-mlt, b1, p2) : fmaf(-mlt, p2, b1);
+        p0 = n0;
+        p2 = 0.0f;
+        c = b1;
     }
-    u0[n - 1] = fabsf(p0) < tiny ? (p0 < 0.0f ? -tiny : tiny) : p0;
-    u1[n - 1] = 0.0f;
-    u2[n - 1] = 0.0f;
+    at(0, n - 1) = 1.0f / (fabsf(p0) < tiny ? (p0 < 0.0f ? -tiny : tiny) : p0);
+    at(1, n - 1) = 0.0f;
+    at(2, n - 1) = 0.0f;
     unsigned h = 0x9E3779B9u * (unsigned)(seed + 1);
     for (int i = 0; i < n; ++i) {
         h = h * 1664525u + 1013904223u;
-        x[i] = 1.0f + 0.25f * ((float)(h >> 8) * (1.0f / 16777216.0f) - 0.5f);
+        at(5, i) = 1.0f + 0.25f * ((float)(h >> 8) * (1.0f / 16777216.0f) - 0.5f);
     }
+    float s2 = 0.0f, inv = 1.0f;  // inv: the last solve's normalisation, applied on the next read
     for (int it = 0; it < 3; ++it) {
         // forward: apply the row swaps and multipliers to the right-hand side
+        // (each step's operands are read before the last one's result is stored)
+        float x0 = at(5, 0) * inv;
+        float nx = n > 1 ? at(5, 1) : 0.0f, nm = at(3, 0), nsw = at(4, 0);
+#pragma unroll 4
         for (int i = 0; i + 1 < n; ++i) {
-            if (sw[i] != 0.0f) {
-                const float t = x[i];
-                x[i] = x[i + 1];
-                x[i + 1] = t - ml[i] * x[i];
-            } else {
-                x[i + 1] -= ml[i] * x[i];
+            const float x1 = nx * inv, ml = nm;
+            const bool swap = nsw != 0.0f;
+            if (i + 2 < n) {
+                nx = at(5, i + 2);
+                nm = at(3, i + 1);
+                nsw = at(4, i + 1);
             }
+            at(5, i) = swap ? x1 : x0;
+            x0 = swap ? fmaf(-ml, x1, x0) : fmaf(-ml, x0, x1);
         }
         // back substitution
-        x[n - 1] = x[n - 1] / u0[n - 1];
-        if (n > 1) x[n - 2] = (x[n - 2] - u1[n - 2] * x[n - 1]) / u0[n - 2];
-        for (int i = n - 3; i >= 0; --i) x[i] = (x[i] - u1[i] * x[i + 1] - u2[i] * x[i + 2]) / u0[i];
-        float mx = 0.0f;
-        for (int i = 0; i < n; ++i) mx = fmaxf(mx, fabsf(x[i]));
-        const float inv = mx > 0.0f ? 1.0f / mx : 1.0f;
-        for (int i = 0; i < n; ++i) x[i] *= inv;
+        float x1 = x0 * at(0, n - 1), x2 = 0.0f, mx = fabsf(x1);
+        at(5, n - 1) = x1;
+        float b0 = 0.0f, b1 = 0.0f, b2 = 0.0f, b5 = 0.0f;
+        auto fetch = [&](int i) {
+            b0 = at(0, i);
+            b1 = at(1, i);
+            b2 = at(2, i);
+            b5 = at(5, i);
+        };
+        if (n > 1) fetch(n - 2);
+#pragma unroll 4
+        for (int i = n - 2; i >= 0; --i) {
+            const float x = fmaf(-b1, x1, fmaf(-b2, x2, b5)) * b0;
+            if (i > 0) fetch(i - 1);
+            at(5, i) = x;
+            mx = fmaxf(mx, fabsf(x));
+            x2 = x1;
+            x1 = x;
+        }
+        inv = mx > 0.0f ? 1.0f / mx : 1.0f;
     }
-    float s2 = 0.0f;
-    for (int i = 0; i < n; ++i) s2 += x[i] * x[i];
-    const float inv = rsqrtf(s2);
-    for (int i = 0; i < n; ++i) Z[i * zs + col] = x[i] * inv;
+    for (int i = 0; i < n; ++i) {
+        const float x = at(5, i) * inv;
+        s2 = fmaf(x, x, s2);
+    }
+    inv *= rsqrtf(s2);
+    for (int i = 0; i < n; ++i) Z[i * zs + col] = at(5, i) * inv;
+}
+
+// Householder tridiagonalisation of the packed lower triangle Ap (F x F,
+// complex Hermitian): d, the complex off-diagonal ec, the reflectors hv with
+// their tau.  Per step: the reflector v from the new column and its norm, p =
+// tau A v, K = tau / 2 Re v^H p, w = p - K v, A -= v w^H + w v^H.
+//
+// tridiagonalise_blocks: a matrix in shared memory (F <= 220), issue-bound on
+// its one SM, so the work goes by 32 x 32 blocks with no index arithmetic or
+// sum over the lanes inside: A v with a lane per row (below the diagonal the
+// lane walks its stored row, beyond it the stored rows of the column block,
+// conjugated), up to four warps a row block; the update with a lane per
+// column, one 16-byte broadcast (v_i, w_i) a row.  The first column of the new
+// trailing matrix comes out of the update.  Former versions: warp
+// per row with nine barriers a step 1.5 ms at 200 frames (3.0M cycles), two
+// barriers and v, w in registers 2.6M cycles (30k instructions a step).
+constexpr int kPartStride = 224;
+struct EigShared {
+    float2 *part;     // up to four partial sums of A v, kPartStride apart
+    float4 *vw;       // (v_i, w_i)
+};
+
+__device__ __forceinline__ float warp_sum(float x)
+{
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// the reflector of the column x[0 .. m): every warp sums its squared norm, a
+// lane's few values first and then the lanes (the error of the norm is the
+// reflector's departure from a unitary matrix: sums of 32 in a row raised the
+// error of the filtered IQ by half at 160 frames)
+__device__ __forceinline__ void reflector(const float2 *x, int m, int lane, float &tau, float2 &v0, float2 &beta)
+{
+    float a2 = 0.0f;
+    for (int i = lane; i < m; i += 32) a2 = fmaf(x[i].x, x[i].x, fmaf(x[i].y, x[i].y, a2));
+    a2 = warp_sum(a2);
+    const float2 x0 = x[0];
+    const float ax0 = sqrtf(fmaf(x0.x, x0.x, x0.y * x0.y));
+    const float alpha = sqrtf(a2);
+    tau = 0.0f;
+    v0 = beta = make_float2(0, 0);
+    if (alpha > 1e-30f) {
+        const float2 th = ax0 > 0.0f ? make_float2(x0.x / ax0, x0.y / ax0) : make_float2(1.0f, 0.0f);
+        beta = make_float2(-th.x * alpha, -th.y * alpha);  // -theta alpha
+        v0 = make_float2(th.x * (ax0 + alpha), th.y * (ax0 + alpha));
+        tau = 1.0f / (alpha * (alpha + ax0));
+    }
+}
+
+__device__ __forceinline__ float2 rank2(float2 c, float2 vi, float2 wi, float2 x, float2 y)  // c - vi conj(y) - wi conj(x)
+{
+    c.x = fmaf(-vi.x, y.x, fmaf(-vi.y, y.y, fmaf(-wi.x, x.x, fmaf(-wi.y, x.y, c.x))));
+    c.y = fmaf(-vi.y, y.x, fmaf(vi.x, y.y, fmaf(-wi.y, x.x, fmaf(wi.x, x.y, c.y))));
+    return c;
+}
+
+__device__ __forceinline__ void tridiagonalise_blocks(float2 *Ap, int F, float *d, float2 *ec, float2 *vvA, float2 *vvB,
+                                                      const EigShared &es, float2 *__restrict__ hv,
+                                                      float *__restrict__ tau_g, int k1, int lane, int wid, int nw)
+{
+    for (int i = 1 + wid * 32 + lane; i < F; i += 32 * nw) vvA[i - 1] = Ap[pidx(i, 0)];  // column 0
+    __syncthreads();
+    for (int k = 0; k < k1; ++k) {
+        const int m = F - k - 1;  // length of the column below the diagonal
+        const int nb = (m + 31) >> 5;
+        float2 *vv = (k & 1) ? vvB : vvA, *vnext = (k & 1) ? vvA : vvB;
+        // ---- the reflector
+        float tau;
+        float2 v0, beta;
+        reflector(vv, m, lane, tau, v0, beta);
+        __syncthreads();
+        for (int i = wid * 32 + lane; i < 32 * nb; i += 32 * nw) {  // zeros past m
+            const float2 v = i == 0 ? v0 : (i < m && tau != 0.0f ? vv[i] : make_float2(0, 0));
+            vv[i] = v;
+            if (i < m) hv[(size_t)k * F + k + 1 + i] = v;
+        }
+        if (wid == nw - 1 && lane == 0) {
+            d[k] = Ap[pidx(k, k)].x;
+            ec[k] = beta;
+            tau_g[k] = tau;
+        }
+        __syncthreads();
+        // ---- partial sums of A v: W warps a row block, column blocks ws, ws + W, ..
+        const int W = min(4, nw / nb);
+        if (wid < W * nb) {
+            const int rb = wid / W, ws = wid - rb * W;
+            const int i = 32 * rb + lane, ic = min(i, m - 1);
+            float2 s = make_float2(0, 0), t = make_float2(0, 0);  // two chains
+            for (int cb = ws; cb < nb; cb += W) {
+                const float2 *v = vv + 32 * cb;
+                if (cb < rb) {
+                    const float2 *a = Ap + pidx(k + 1 + ic, k + 1 + 32 * cb);
+#pragma unroll 8
+                    for (int j = 0; j < 32; j += 2) {
+                        const float2 a0 = a[j], a1 = a[j + 1], x0 = v[j], x1 = v[j + 1];
+                        s.x = fmaf(a0.x, x0.x, fmaf(-a0.y, x0.y, s.x));
+                        s.y = fmaf(a0.x, x0.y, fmaf(a0.y, x0.x, s.y));
+                        t.x = fmaf(a1.x, x1.x, fmaf(-a1.y, x1.y, t.x));
+                        t.y = fmaf(a1.x, x1.y, fmaf(a1.y, x1.x, t.y));
+                    }
+                } else if (cb > rb) {
+                    const int n = min(32, m - 32 * cb);
+                    int o = pidx(k + 1 + 32 * cb, k + 1 + i), st = k + 2 + 32 * cb;  // row 32 cb + j: o += its length
+#pragma unroll 8
+                    for (int j = 0; j < n; ++j) {
+                        const float2 a0 = Ap[o], x0 = v[j];
+                        o += st++;
+                        s.x = fmaf(a0.x, x0.x, fmaf(a0.y, x0.y, s.x));
+                        s.y = fmaf(a0.x, x0.y, fmaf(-a0.y, x0.x, s.y));
+                    }
+                } else {
+                    const int n = min(32, m - 32 * cb);
+                    const int own = pidx(k + 1 + ic, k + 1 + 32 * cb);
+#pragma unroll 4
+                    for (int j = 0; j < n; ++j) {
+                        const bool low = j <= ic - 32 * cb;
+                        const float2 a0 = Ap[low ? own + j : pidx(k + 1 + 32 * cb + j, k + 1 + ic)], x0 = v[j];
+                        const float ay = low ? a0.y : -a0.y;
+                        s.x = fmaf(a0.x, x0.x, fmaf(-ay, x0.y, s.x));
+                        s.y = fmaf(a0.x, x0.y, fmaf(ay, x0.x, s.y));
+                    }
+                }
+            }
+            if (i < m) es.part[ws * kPartStride + i] = make_float2(s.x + t.x, s.y + t.y);
+        }
+        __syncthreads();
+        // ---- p, K (every warp), w
+        float vhp = 0.0f;
+        float2 pq = make_float2(0, 0), vq = make_float2(0, 0);  // of the warp's own block
+        for (int q = 0; q < nb; ++q) {
+            const int i = 32 * q + lane;
+            float2 p = make_float2(0, 0), v = make_float2(0, 0);
+            if (i < m) {
+                const int Wp = min(W, nb);
+                for (int h = 0; h < Wp; ++h) {
+                    const float2 x = es.part[h * kPartStride + i];
+                    p.x += x.x;
+                    p.y += x.y;
+                }
+                p = make_float2(tau * p.x, tau * p.y);
+                v = vv[i];
+                vhp = fmaf(v.x, p.x, fmaf(v.y, p.y, vhp));
+            }
+            if (q == wid) {
+                pq = p;
+                vq = v;
+            }
+        }
+        const float K = 0.5f * tau * warp_sum(vhp);
+        if (wid < nb) es.vw[32 * wid + lane] = make_float4(vq.x, vq.y, fmaf(-K, vq.x, pq.x), fmaf(-K, vq.y, pq.y));
+        __syncthreads();
+        // ---- A -= v w^H + w v^H by lower blocks, numbered along the block rows
+        for (int t = wid, rb = 0; ; t += nw) {
+            // block t of the triangle (from the last one found on)
+            while (rb < nb && (rb + 1) * (rb + 2) / 2 <= t) ++rb;
+            if (rb >= nb) break;
+            const int cb = t - rb * (rb + 1) / 2;
+            const int j = 32 * cb + lane;
+            const float4 y = es.vw[j];
+            const int n = min(32, m - 32 * rb);
+            int o = pidx(k + 1 + 32 * rb, k + 1 + j), st = k + 2 + 32 * rb;
+            for (int r = 0; r < n; r += 4) {
+                float2 a[4];
+                int oo[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    oo[u] = o;
+                    const bool on = r + u < n && j <= 32 * rb + r + u;
+                    a[u] = on ? Ap[o] : make_float2(0, 0);
+                    o += st++;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int i = 32 * rb + r + u;
+                    const float4 x = es.vw[min(i, 32 * nb - 1)];
+                    a[u] = rank2(a[u], make_float2(x.x, x.y), make_float2(x.z, x.w), make_float2(y.x, y.y),
+                                 make_float2(y.z, y.w));
+                    if (r + u < n && j <= i) Ap[oo[u]] = a[u];
+                    if (j == 0 && i > 0 && r + u < n) vnext[i - 1] = a[u];  // the new trailing matrix's first column
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// The last 128 columns (or all of a smaller matrix): warp per row, two rows
+// together, v and w of the lane's 32-column blocks in registers, two barriers a
+// step.  With few blocks left, tridiagonalise_blocks keeps few warps busy (all
+// of 100 frames: 635k cycles by blocks, 543k by rows; 48: 242k and 174k).
+template <int NQ>
+__device__ __forceinline__ void tridiagonalise_lanes(float2 *Ap, int F, int k0, float *d, float2 *ec, float2 *vvA, float2 *vvB,
+                                               float2 *pv, float *redq, float2 *__restrict__ hv,
+                                               float *__restrict__ tau_g, int lane, int wid, int nw)
+{
+    for (int k = k0; k + 2 < F; ++k) {
+        const int m = F - k - 1;  // length of the column below the diagonal
+        float2 *vv = (k & 1) ? vvB : vvA, *vnext = (k & 1) ? vvA : vvB;
+        // ---- (B)
+        float tau;
+        float2 v0, beta;
+        reflector(vv, m, lane, tau, v0, beta);
+        auto vat = [&](int i) { return i == 0 ? v0 : (tau != 0.0f ? vv[i] : make_float2(0, 0)); };
+        if (wid == nw - 1 && lane == 0) {
+            d[k] = Ap[pidx(k, k)].x;
+            ec[k] = beta;
+            tau_g[k] = tau;
+        }
+        for (int i = wid * 32 + lane; i < m; i += 32 * nw) hv[(size_t)k * F + k + 1 + i] = vat(i);
+        float2 v[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) v[q] = lane + 32 * q < m ? vat(lane + 32 * q) : make_float2(0, 0);
+        int cb[NQ];  // first word of the lane's columns below the diagonal
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) cb[q] = pidx(k + 1 + lane + 32 * q, 0);
+        float vhp = 0.0f;
+        for (int i = wid; i < m; i += 2 * nw) {
+            const int i2 = i + nw;
+            const bool two = i2 < m;
+            const int iz = two ? i2 : i;
+            const int g1 = k + 1 + i, g2 = k + 1 + iz;
+            const int r1 = pidx(g1, k + 1), r2 = pidx(g2, k + 1);
+            // s += A(i, j) v_j for the lane's columns j = 32 q + lane: the stored row up
+            // to the diagonal, the conjugate of the column beyond it
+            auto mac = [](float2 &s, float2 a, float2 x) {
+                s.x = fmaf(a.x, x.x, fmaf(-a.y, x.y, s.x));
+                s.y = fmaf(a.x, x.y, fmaf(a.y, x.x, s.y));
+            };
+            auto macc = [](float2 &s, float2 a, float2 x) {  // conj(a) x
+                s.x = fmaf(a.x, x.x, fmaf(a.y, x.y, s.x));
+                s.y = fmaf(a.x, x.y, fmaf(-a.y, x.x, s.y));
+            };
+            float2 s1 = make_float2(0, 0), s2 = make_float2(0, 0);
+            // both rows' loads before their sums (columns past m: the row's last
+            // value times v = 0)
+            float2 a[NQ], b[NQ];
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+                if (32 * q < m) {
+                    const int j = lane + 32 * q;
+                    const bool in = j < m;
+                    a[q] = Ap[j <= i || !in ? r1 + min(j, i) : cb[q] + g1];
+                    b[q] = Ap[j <= iz || !in ? r2 + min(j, iz) : cb[q] + g2];
+                }
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+                if (32 * q < m) {
+                    const int j = lane + 32 * q;
+                    if (32 * q + 31 <= i) mac(s1, a[q], v[q]);
+                    else if (32 * q > i) macc(s1, a[q], v[q]);
+                    else mac(s1, make_float2(a[q].x, j <= i ? a[q].y : -a[q].y), v[q]);
+                    if (32 * q + 31 <= iz) mac(s2, b[q], v[q]);
+                    else if (32 * q > iz) macc(s2, b[q], v[q]);
+                    else mac(s2, make_float2(b[q].x, j <= iz ? b[q].y : -b[q].y), v[q]);
+                }
+            // four sums over the lanes in six exchanges: s1.x, s1.y, s2.x, s2.y end in
+            // lanes 0, 8, 16, 24 (and the seven after each)
+            const bool h16 = lane & 16, h8 = lane & 8;
+            const float ax = (h16 ? s2.x : s1.x) + __shfl_xor_sync(0xffffffffu, h16 ? s1.x : s2.x, 16);
+            const float ay = (h16 ? s2.y : s1.y) + __shfl_xor_sync(0xffffffffu, h16 ? s1.y : s2.y, 16);
+            float t = (h8 ? ay : ax) + __shfl_xor_sync(0xffffffffu, h8 ? ax : ay, 8);
+            t += __shfl_xor_sync(0xffffffffu, t, 4);
+            t += __shfl_xor_sync(0xffffffffu, t, 2);
+            t += __shfl_xor_sync(0xffffffffu, t, 1);
+            if ((lane & 7) == 0 && (two || !h16)) {
+                const int row = h16 ? i2 : i;
+                const float pc = tau * t;
+                const float2 x = vat(row);
+                reinterpret_cast<float *>(pv)[2 * row + (h8 ? 1 : 0)] = pc;
+                vhp = fmaf(h8 ? x.y : x.x, pc, vhp);
+            }
+        }
+        vhp = warp_sum(vhp);
+        if (lane == 0) redq[wid] = vhp;
+        __syncthreads();
+        // ---- (A)
+        const float K = 0.5f * tau * warp_sum(lane < nw ? redq[lane] : 0.0f);
+        auto wat = [&](int i) {
+            const float2 x = vat(i), p = pv[i];
+            return make_float2(fmaf(-K, x.x, p.x), fmaf(-K, x.y, p.y));
+        };
+        float2 w[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) w[q] = lane + 32 * q < m ? wat(lane + 32 * q) : make_float2(0, 0);
+        for (int i = wid; i < m; i += 2 * nw) {
+            const int i2 = i + nw;
+            const bool two = i2 < m;
+            const int r1 = pidx(k + 1 + i, k + 1), r2 = two ? pidx(k + 1 + i2, k + 1) : r1;
+            const float2 vi1 = vat(i), wi1 = wat(i), vi2 = two ? vat(i2) : vi1, wi2 = two ? wat(i2) : wi1;
+            auto first = [&](int row, float2 c) {  // the first column of the new trailing matrix
+                if (lane == 0 && row > 0) vnext[row - 1] = c;
+            };
+            const int e2 = two ? i2 : -1;  // last columns of the two rows: i, e2
+            // both rows loaded before anything is stored: the compiler cannot
+            // move a load over a store to the same matrix
+            float2 a[NQ], b[NQ];
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int j = lane + 32 * q;
+                if (32 * q <= i && j <= i) a[q] = Ap[r1 + j];
+                if (32 * q <= e2 && j <= e2) b[q] = Ap[r2 + j];
+            }
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int j = lane + 32 * q;
+                if (32 * q <= i) {
+                    a[q] = rank2(a[q], vi1, wi1, v[q], w[q]);
+                    if (j <= i) Ap[r1 + j] = a[q];
+                }
+                if (32 * q <= e2) {
+                    b[q] = rank2(b[q], vi2, wi2, v[q], w[q]);
+                    if (j <= e2) Ap[r2 + j] = b[q];
+                }
+            }
+            first(i, a[0]);
+            if (two) first(i2, b[0]);
+        }
+        __syncthreads();
+    }
+}
+
+// A matrix in global memory (F > 220): warp per row, two barriers a step.
+__device__ __forceinline__ void tridiagonalise_rows(float2 *Ap, int F, float *d, float2 *ec, float2 *vvA, float2 *vvB,
+                                                    float2 *pv, float *redq, float2 *__restrict__ hv,
+                                                    float *__restrict__ tau_g, int lane, int wid, int nw)
+{
+    for (int i = 1 + wid * 32 + lane; i < F; i += 32 * nw) vvA[i - 1] = Ap[pidx(i, 0)];  // column 0
+    __syncthreads();
+    for (int k = 0; k + 2 < F; ++k) {
+        const int m = F - k - 1;  // length of the column below the diagonal
+        float2 *vv = (k & 1) ? vvB : vvA, *vnext = (k & 1) ? vvA : vvB;
+        float tau;
+        float2 v0, beta;
+        reflector(vv, m, lane, tau, v0, beta);
+        auto vat = [&](int i) { return i == 0 ? v0 : (tau != 0.0f ? vv[i] : make_float2(0, 0)); };
+        if (wid == nw - 1 && lane == 0) {
+            d[k] = Ap[pidx(k, k)].x;
+            ec[k] = beta;
+            tau_g[k] = tau;
+        }
+        for (int i = wid * 32 + lane; i < m; i += 32 * nw) hv[(size_t)k * F + k + 1 + i] = vat(i);
+        float vhp = 0.0f;
+        for (int i = wid; i < m; i += nw) {
+            const int gi = k + 1 + i;
+            float2 s = make_float2(0, 0);
+#pragma unroll 4
+            for (int j = lane; j < m; j += 32) {
+                const float2 a = Ap[j <= i ? pidx(gi, k + 1 + j) : pidx(k + 1 + j, gi)], x = vat(j);
+                const float ay = j <= i ? a.y : -a.y;
+                s.x = fmaf(a.x, x.x, fmaf(-ay, x.y, s.x));
+                s.y = fmaf(a.x, x.y, fmaf(ay, x.x, s.y));
+            }
+            s.x = warp_sum(s.x);
+            s.y = warp_sum(s.y);
+            if (lane == 0) {
+                const float2 p = make_float2(tau * s.x, tau * s.y), x = vat(i);
+                pv[i] = p;
+                vhp = fmaf(x.x, p.x, fmaf(x.y, p.y, vhp));
+            }
+        }
+        if (lane == 0) redq[wid] = vhp;
+        __syncthreads();
+        const float K = 0.5f * tau * warp_sum(lane < nw ? redq[lane] : 0.0f);
+        auto wat = [&](int i) {
+            const float2 x = vat(i), p = pv[i];
+            return make_float2(fmaf(-K, x.x, p.x), fmaf(-K, x.y, p.y));
+        };
+        for (int i = wid; i < m; i += nw) {
+            const int r = pidx(k + 1 + i, k + 1);
+            const float2 vi = vat(i), wi = wat(i);
+#pragma unroll 4
+            for (int j = lane; j <= i; j += 32) {
+                const float2 c = rank2(Ap[r + j], vi, wi, vat(j), wat(j));
+                Ap[r + j] = c;
+                if (j == 0 && i > 0) vnext[i - 1] = c;  // the first column of the new trailing matrix
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// One step of subspace iteration with the matrix itself: V <- orth(G V) for the
+// k <= kRefineMaxK vectors, where lambda_j is well above the rounding of G.
+// It takes the rounding of the F reflectors out of the filter's subspace (a
+// factor lambda_{k+1} / lambda_k of it stays): error of the filtered IQ against
+// 64 bits at 200 / 160 / 100 / 60 frames 1.8 / 4.6 / 1.8 / 3.3e-6 without it (the
+// former, slower tridiagonalisation 1.4 / 3.4 / 1.8 / 3.6e-6), 0.46 / 1.3 / 0.51 /
+// 1.1e-6 with it, for 0.03 ms at 200 frames.
+// Y: k F values of scratch.
+constexpr int kRefineMaxK = 8;
+__device__ __forceinline__ void refine_vectors(const float2 *__restrict__ G, int F, int k, const float *lam, float2 *Y,
+                                               float2 *V, float2 *Vt, int lane, int wid, int nw)
+{
+    __syncthreads();
+    for (int i = wid; i < F; i += nw)
+        for (int j0 = 0; j0 < k; j0 += 4) {  // four columns together: their sums over the lanes overlap
+            float2 s[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s[u] = make_float2(0, 0);
+            for (int f = lane; f < F; f += 32) {
+                const float2 g = G[(size_t)i * F + f];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (j0 + u < k) {
+                        const float2 t = cmul(g, Vt[(size_t)(j0 + u) * F + f]);
+                        s[u].x += t.x;
+                        s[u].y += t.y;
+                    }
+            }
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    s[u].x += __shfl_xor_sync(0xffffffffu, s[u].x, o);
+                    s[u].y += __shfl_xor_sync(0xffffffffu, s[u].y, o);
+                }
+            if (lane == 0)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (j0 + u < k)
+                        Y[(size_t)(j0 + u) * F + i] =
+                            lam[j0 + u] > 2.44140625e-4f * lam[0] ? s[u] : Vt[(size_t)(j0 + u) * F + i];
+        }
+    __syncthreads();
+    if (wid == 0) {  // modified Gram-Schmidt in the order of the eigenvalues
+        for (int j = 0; j < k; ++j) {
+            float2 *y = Y + (size_t)j * F;
+            for (int pass = 0; pass <= j; ++pass) {
+                float n2 = 0.0f;
+                for (int f = lane; f < F; f += 32) n2 = fmaf(y[f].x, y[f].x, fmaf(y[f].y, y[f].y, n2));
+                const float inv = rsqrtf(fmaxf(warp_sum(n2), FLT_MIN));  // unit length first: no overflow below
+                for (int f = lane; f < F; f += 32) y[f] = make_float2(y[f].x * inv, y[f].y * inv);
+                __syncwarp();
+                if (pass == j) break;
+                const float2 *x = Y + (size_t)pass * F;
+                float2 c = make_float2(0, 0);
+                for (int f = lane; f < F; f += 32) cmac(c, x[f].x, x[f].y, y[f].x, y[f].y);
+                c.x = warp_sum(c.x);
+                c.y = warp_sum(c.y);
+                for (int f = lane; f < F; f += 32) {
+                    const float2 t = cmul(x[f], c);
+                    y[f] = make_float2(y[f].x - t.x, y[f].y - t.y);
+                }
+                __syncwarp();
+            }
+            for (int f = lane; f < F; f += 32) {
+                Vt[(size_t)j * F + f] = y[f];
+                if (V) V[(size_t)f * F + j] = y[f];
+            }
+        }
+    }
 }
 
 // Householder tridiagonalisation of the Hermitian G (lower triangle used),
@@ -438,10 +980,14 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
     float2 *Ap = big ? big : dyn;                 // packed lower triangle, later Z (real, stride F+1)
     float *Z = reinterpret_cast<float *>(Ap);
     __shared__ float red[33];
-    __shared__ float d[512], e[512], rc[512], rs[512];
-    __shared__ float2 ec[512], vv[512], pv[512], delta[512];
+    __shared__ float d[512], e[512], redq[32];
+    __shared__ float2 ec[512], vv[512], rcs[512];
+    __shared__ float2 eigw[1536];  // the partial sums of the tridiagonalisation; p; then the three below
+    float2 *pv = eigw, *delta = eigw + 512;
+    float *spare = reinterpret_cast<float *>(eigw + 1024);  // e^2 and the eigenvalues
+    float *rc = reinterpret_cast<float *>(rcs), *rs = rc + 512;  // QL rotations (tridiagonalisation: a second vv)
     __shared__ int perm[512];
-    __shared__ float s_tau, s_scale;
+    __shared__ float s_scale;
     __shared__ int s_m, s_nrot, s_done, s_fail;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
 
@@ -470,80 +1016,16 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
         }
     __syncthreads();
 
-    // ---- tridiagonalisation
-    for (int k = 0; k + 2 < F; ++k) {
-        const int m = F - k - 1;  // length of the column below the diagonal
-        float part = 0.0f;
-        for (int i = tid; i < m; i += blockDim.x) {
-            float2 x = Ap[pidx(k + 1 + i, k)];
-            part += x.x * x.x + x.y * x.y;
-        }
-        float a2 = block_sum(part, red);
-        if (tid == 0) {
-            d[k] = Ap[pidx(k, k)].x;
-            float2 x0 = Ap[pidx(k + 1, k)];
-            float ax0 = sqrtf(x0.x * x0.x + x0.y * x0.y);
-            float alpha = sqrtf(a2);
-            if (alpha <= 1e-30f) {
-                s_tau = 0.0f;
-                ec[k] = make_float2(0, 0);
-                vv[0] = make_float2(0, 0);
-            } else {
-                float2 th = ax0 > 0.0f ? make_float2(x0.x / ax0, x0.y / ax0) : make_float2(1.0f, 0.0f);
-                ec[k] = make_float2(-th.x * alpha, -th.y * alpha);   // beta = -theta alpha
-                vv[0] = make_float2(th.x * (ax0 + alpha), th.y * (ax0 + alpha));
-                s_tau = 1.0f / (alpha * (alpha + ax0));
-            }
-        }
-        __syncthreads();
-        const float tau = s_tau;
-        for (int i = 1 + tid; i < m; i += blockDim.x) vv[i] = tau != 0.0f ? Ap[pidx(k + 1 + i, k)] : make_float2(0, 0);
-        __syncthreads();
-        for (int i = tid; i < m; i += blockDim.x) hv[(size_t)k * F + k + 1 + i] = vv[i];
-        if (tid == 0) tau_g[k] = tau;
-        if (tau == 0.0f) {
-            __syncthreads();
-            continue;
-        }
-        // p = tau A22 v (warp per row)
-        for (int i = wid; i < m; i += nw) {
-            float2 s = make_float2(0, 0);
-            const int gi = k + 1 + i;
-            for (int j = lane; j < m; j += 32) {
-                const int gj = k + 1 + j;
-                float2 a = gj <= gi ? Ap[pidx(gi, gj)] : cconj(Ap[pidx(gj, gi)]);
-                float2 t = cmul(a, vv[j]);
-                s.x += t.x;
-                s.y += t.y;
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-                s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
-            }
-            if (lane == 0) pv[i] = make_float2(tau * s.x, tau * s.y);
-        }
-        __syncthreads();
-        // K = tau / 2 * Re(v^H p)
-        float q = 0.0f;
-        for (int i = tid; i < m; i += blockDim.x) q += vv[i].x * pv[i].x + vv[i].y * pv[i].y;
-        float vhp = block_sum(q, red);
-        const float K = 0.5f * tau * vhp;
-        // w = p - K v (in place in pv)
-        for (int i = tid; i < m; i += blockDim.x) pv[i] = make_float2(pv[i].x - K * vv[i].x, pv[i].y - K * vv[i].y);
-        __syncthreads();
-        // A22 -= v w^H + w v^H (lower triangle)
-        for (int i = wid; i < m; i += nw) {
-            const float2 vi = vv[i], wi = pv[i];
-            for (int j = lane; j <= i; j += 32) {
-                float2 a = Ap[pidx(k + 1 + i, k + 1 + j)];
-                float2 t1 = cmul(vi, cconj(pv[j]));
-                float2 t2 = cmul(wi, cconj(vv[j]));
-                a.x -= t1.x + t2.x;
-                a.y -= t1.y + t2.y;
-                Ap[pidx(k + 1 + i, k + 1 + j)] = a;
-            }
-        }
-        __syncthreads();
+    // (a matrix in shared memory, F <= 220, goes by `dyn` itself, so that it is
+    // addressed as such)
+    __shared__ float4 vw[224];
+    if (big) {
+        tridiagonalise_rows(big, F, d, ec, vv, rcs, pv, redq, hv, tau_g, lane, wid, nw);
+    } else {
+        const EigShared es = {eigw, vw};
+        const int k1 = max(0, F - 129);  // blocks while more than 128 rows remain
+        tridiagonalise_blocks(dyn, F, d, ec, vv, rcs, es, hv, tau_g, k1, lane, wid, nw);
+        tridiagonalise_lanes<4>(dyn, F, k1, d, ec, vv, rcs, pv, redq, hv, tau_g, lane, wid, nw);
     }
     if (tid == 0) {
         if (F >= 2) {
@@ -551,43 +1033,58 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
             ec[F - 2] = Ap[pidx(F - 1, F - 2)];
         }
         d[F - 1] = Ap[pidx(F - 1, F - 1)].x;
-        // diagonal unitary scaling making the off-diagonal real and >= 0
-        delta[0] = make_float2(1.0f, 0.0f);
-        for (int k = 0; k + 1 < F; ++k) {
-            float2 x = ec[k];
-            float ax = sqrtf(x.x * x.x + x.y * x.y);
-            e[k] = ax;
-            delta[k + 1] = ax > 0.0f ? cmul(delta[k], make_float2(x.x / ax, x.y / ax)) : delta[k];
-        }
-        e[F - 1] = 0.0f;
         s_fail = 0;
+    }
+    __syncthreads();
+    // diagonal unitary scaling making the off-diagonal real and >= 0: the phases
+    // side by side, then their running product
+    for (int k = tid; k < F; k += blockDim.x) {
+        const float2 x = k + 1 < F ? ec[k] : make_float2(0, 0);
+        const float ax = sqrtf(x.x * x.x + x.y * x.y);
+        e[k] = ax;
+        vv[k] = ax > 0.0f ? make_float2(x.x / ax, x.y / ax) : make_float2(1.0f, 0.0f);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        float2 dl = make_float2(1.0f, 0.0f);
+        delta[0] = dl;
+#pragma unroll 4
+        for (int k = 0; k + 1 < F; ++k) {
+            dl = cmul(dl, vv[k]);
+            delta[k + 1] = dl;
+        }
     }
     __syncthreads();
     const int zs = F + 1;
     if (topk_only) {
         // ---- all eigenvalues by bisection (one thread each), top-k vectors by
         // inverse iteration; the QL path below is the fallback for large k
-        __shared__ float e2[512], lamd[512];
-        __shared__ float s_lo, s_hi, s_piv, s_tnorm;
+        float *e2 = spare, *lamd = spare + 512;
+        __shared__ float s_lo, s_hi, s_tnorm;
         __shared__ int s_k;
-        for (int i = tid; i < F; i += blockDim.x) e2[i] = e[i] * e[i];
-        if (tid == 0) {
+        for (int i = tid; i < F; i += blockDim.x) e2[i] = fmaxf(e[i] * e[i], 4.0f * FLT_MIN);  // > 0
+        if (wid == 0) {
             float lo = 1e30f, hi = -1e30f, tn = 0.0f;
-            for (int i = 0; i < F; ++i) {
+            for (int i = lane; i < F; i += 32) {
                 const float r = (i > 0 ? e[i - 1] : 0.0f) + e[i];
                 lo = fminf(lo, d[i] - r);
                 hi = fmaxf(hi, d[i] + r);
                 tn = fmaxf(tn, fabsf(d[i]) + r);
             }
-            const float pad = 4.0f * FLT_EPSILON * fmaxf(tn, 1e-30f);
-            s_lo = lo - pad;
-            s_hi = hi + pad;
-            s_tnorm = tn;
-            s_piv = fmaxf(1e-30f, FLT_MIN * 4.0f);
+            for (int o = 16; o > 0; o >>= 1) {
+                lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+                tn = fmaxf(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+            }
+            if (lane == 0) {
+                const float pad = 4.0f * FLT_EPSILON * fmaxf(tn, 1e-30f);
+                s_lo = lo - pad;
+                s_hi = hi + pad;
+                s_tnorm = tn;
+            }
         }
         __syncthreads();
-        for (int j = tid; j < F; j += blockDim.x)
-            lamd[j] = bisect_eig(d, e2, F, F - 1 - j, s_lo, s_hi, s_piv);  // descending order
+        multisect(d, e2, F, s_lo, s_hi, s_tnorm, lamd);  // descending order
         __syncthreads();
         for (int j = tid; j < F; j += blockDim.x) lam_out[j] = (double)lamd[j] * (double)gscale;
         if (tid == 0) {
@@ -607,9 +1104,20 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
         __syncthreads();
         const int k = s_k;
         if (k <= kFastMaxK && ii_scr) {
+            int zk;
             const float tiny = FLT_EPSILON * fmaxf(s_tnorm, 1e-30f);
-            for (int j = tid; j < k; j += blockDim.x)
-                inverse_iteration(d, e, F, lamd[j], tiny, j, Z, zs, j, ii_scr + (size_t)j * 6 * F);
+            // vectors (stride zk) and, where they fit behind them, the solves' scratch
+            // in the packed matrix's storage
+            zk = k | 1;
+            const bool in_z = !big && (size_t)F * zk + (size_t)6 * k * F <= (size_t)F * (F + 1);
+            for (int j = tid; j < k; j += blockDim.x) {
+                if (in_z) {
+                    float *z = reinterpret_cast<float *>(dyn);
+                    inverse_iteration(d, e, F, lamd[j], tiny, j, z, zk, j, z + (size_t)F * zk + j, k);
+                } else {
+                    inverse_iteration(d, e, F, lamd[j], tiny, j, Z, zk, j, ii_scr + (size_t)j * 6 * F, 1);
+                }
+            }
             __syncthreads();
             // re-orthogonalise vectors of close eigenvalues (modified Gram-Schmidt, warp 0)
             if (wid == 0) {
@@ -620,24 +1128,32 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
                         if (fabsf(lamd[i] - lamd[j]) > gap) continue;
                         any = true;
                         float dot = 0.0f;
-                        for (int r = lane; r < F; r += 32) dot += Z[r * zs + i] * Z[r * zs + j];
+                        for (int r = lane; r < F; r += 32) dot += Z[r * zk + i] * Z[r * zk + j];
                         for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-                        for (int r = lane; r < F; r += 32) Z[r * zs + j] -= dot * Z[r * zs + i];
+                        for (int r = lane; r < F; r += 32) Z[r * zk + j] -= dot * Z[r * zk + i];
                         __syncwarp();
                     }
                     if (any) {
                         float n2 = 0.0f;
-                        for (int r = lane; r < F; r += 32) n2 += Z[r * zs + j] * Z[r * zs + j];
+                        for (int r = lane; r < F; r += 32) n2 += Z[r * zk + j] * Z[r * zk + j];
                         for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
                         const float inv = rsqrtf(n2);
-                        for (int r = lane; r < F; r += 32) Z[r * zs + j] *= inv;
+                        for (int r = lane; r < F; r += 32) Z[r * zk + j] *= inv;
                         __syncwarp();
                     }
                 }
             }
             for (int j = tid; j < F; j += blockDim.x) perm[j] = j;
             __syncthreads();
-            back_transform(F, k, Z, zs, perm, delta, hv, tau_g, V, Vt, lane, wid, nw);
+            // reflectors staged behind the k vectors (2 nbuf F complex values)
+            const int nbuf = min(16, (F - zk) / 4);
+            if (!big && nbuf > 0)
+                back_transform(F, k, reinterpret_cast<float *>(dyn), zk, perm, delta, hv, tau_g, V, Vt,
+                               dyn + (F * zk + 1) / 2, nbuf, lane, wid, nw);
+            else
+                back_transform(F, k, Z, zk, perm, delta, hv, tau_g, V, Vt, nullptr, 0, lane, wid, nw);
+            if (k <= kRefineMaxK && k < F)
+                refine_vectors(G, F, k, lamd, big || 2 * k > F + 1 ? reinterpret_cast<float2 *>(ii_scr) : dyn, V, Vt, lane, wid, nw);
             return;
         }
     }
@@ -762,10 +1278,11 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
         if (k_out) *k_out = k;
         if (status && s_fail) *status = FQ_ERR_NUMERICAL;
     }
-    back_transform(F, F, Z, zs, perm, delta, hv, tau_g, V, Vt, lane, wid, nw);
+    back_transform(F, F, Z, zs, perm, delta, hv, tau_g, V, Vt, nullptr, 0, lane, wid, nw);
 }
 
-__global__ void __launch_bounds__(kEigThreads) eig_kernel(const float2 *__restrict__ G, int F, float2 *__restrict__ big,
+template <int NT>
+__global__ void __launch_bounds__(NT) eig_kernel(const float2 *__restrict__ G, int F, float2 *__restrict__ big,
                                                           float2 *__restrict__ hv, float *__restrict__ tau_g,
                                                           double *__restrict__ lam_out, float2 *__restrict__ V,
                                                           float2 *__restrict__ Vt, int k_cut, double thresh,
@@ -776,14 +1293,14 @@ __global__ void __launch_bounds__(kEigThreads) eig_kernel(const float2 *__restri
 }
 
 // One CTA per ensemble of a wave; the packed matrix always in the workspace.
-__global__ void __launch_bounds__(kEigThreads) eig_batched_kernel(const fqb::EnsDev *__restrict__ ens,
+__global__ void __launch_bounds__(kTopThreads) eig_batched_kernel(const fqb::EnsDev *__restrict__ ens,
                                                                   const int *__restrict__ members)
 {
     const fqb::EnsDev &e = ens[members[blockIdx.x]];
     char *ws = e.cws;
     double *lam = e.eigvals ? e.eigvals : (double *)(ws + e.cl_lam);
     int *kk = e.k_used ? e.k_used : (int *)(ws + e.cl_k);
-    eig_body((const float2 *)(ws + e.cl_G), e.F, (float2 *)(ws + e.cl_big), (float2 *)(ws + e.cl_hv),
+    eig_body((const float2 *)(ws + e.cl_G), e.F, eig_in_smem(e.F) ? nullptr : (float2 *)(ws + e.cl_big), (float2 *)(ws + e.cl_hv),
              (float *)(ws + e.cl_tau), lam, (float2 *)(ws + e.cl_V), (float2 *)(ws + e.cl_Vt), e.k_cut,
              e.energy_thresh, kk, e.status, 1, (float *)(ws + e.cl_ii));
 }
@@ -904,7 +1421,7 @@ fq_status launch_project(const void *S, int64_t P, int F, const float2 *Vt, cons
 
 // ------------------------------------------------------------- batched --
 template <typename T>
-__global__ void __launch_bounds__(kGramThreads, 2) gram_batched_kernel(const fqb::EnsDev *__restrict__ ens, const fqb::StageQueue q)
+__global__ void __launch_bounds__(kGramThreads, kGramCtas) gram_batched_kernel(const fqb::EnsDev *__restrict__ ens, const fqb::StageQueue q)
 {
     extern __shared__ float4 panel[];
     __shared__ int s_buf[2];
@@ -1005,15 +1522,16 @@ fq_status launch_eig(const float2 *G, int F, float2 *big, float2 *hv, float *tau
                      float *ii_scr = nullptr)
 {
     size_t smem = big ? 0 : sizeof(float2) * (size_t)F * (F + 1) / 2;
+    auto kern = topk_only ? eig_kernel<kTopThreads> : eig_kernel<kEigThreads>;
     if (smem > 0) {
         // the kernel's static arrays count against the same 48 KB default,
         // so the opt-in is needed for much smaller packed matrices too
-        fq_status s = fqi::cuda_check(cudaFuncSetAttribute(eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           (int)smem), "eig: smem attribute");
+        fq_status s = fqi::cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                                      "eig: smem attribute");
         if (s) return s;
     }
-    eig_kernel<<<1, kEigThreads, smem, st>>>(G, F, big, hv, tau, lam, V, Vt, k_cut, thresh, k_out, status,
-                                             topk_only, ii_scr);
+    kern<<<1, topk_only ? kTopThreads : kEigThreads, smem, st>>>(G, F, big, hv, tau, lam, V, Vt, k_cut, thresh, k_out,
+                                                                status, topk_only, ii_scr);
     return fqi::launch_check("fq_hermitian_eig");
 }
 
@@ -1351,9 +1869,14 @@ fq_status batched_gram_reduce(const fqb::EnsDev *ens, const fqb::StageQueue &q, 
     return launch_check("batched Gram reduce");
 }
 
-fq_status batched_eig(const fqb::EnsDev *ens, const int *members, int n, cudaStream_t st)
+fq_status batched_eig(const fqb::EnsDev *ens, const int *members, int n, int F_max, cudaStream_t st)
 {
-    eig_batched_kernel<<<n, kEigThreads, 0, st>>>(ens, members);
+    while (!eig_in_smem(F_max)) --F_max;  // larger members keep their matrix in the workspace
+    const size_t smem = sizeof(float2) * (size_t)F_max * (F_max + 1) / 2;
+    fq_status s = cuda_check(cudaFuncSetAttribute(eig_batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)smem), "batched eig: smem attribute");
+    if (s) return s;
+    eig_batched_kernel<<<n, kTopThreads, smem, st>>>(ens, members);
     return launch_check("batched eig");
 }
 

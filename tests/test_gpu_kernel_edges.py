@@ -1,7 +1,7 @@
 """The hot kernels at the edges of their layouts: angle blocks and record
 segments of the RF kernel, pixel panels and column blocks of the FP32 Gram,
-frame groups and voxel pairs of the 16-bit delay-and-sum, accumulator runs
-of the convolution."""
+register blocks of the tridiagonalisation, frame groups and voxel pairs of
+the 16-bit delay-and-sum, accumulator runs of the convolution."""
 import numpy as np
 import pytest
 import torch
@@ -61,6 +61,29 @@ def test_gram_panels(F, P, dt):
     mag = (S.double().abs().sum(2)).mT @ S.double().abs().sum(2)
     err = (G - s.mH @ s).abs()
     assert bool((err <= 2.0 ** -24 * (2 * P + 16) * mag).all())
+
+
+# register blocks of 32 columns, the shared-memory limit (220) and beyond;
+# eigenvalues within 2 F 2^-24 of the largest, and with them the filtered
+# energy of the pixels
+@pytest.mark.parametrize("F", [2, 3, 5, 32, 33, 65, 128, 129, 200, 221, 300])
+def test_eigen_blocks(F):
+    g = torch.Generator(device="cuda").manual_seed(F)
+    P, k = 700, min(3, F - 1)
+    lev = torch.tensor([100.0, 40.0, 20.0], device="cuda")[:k]
+    U = torch.randn((P, k), generator=g, device="cuda", dtype=torch.complex64)
+    V = torch.linalg.qr(torch.randn((F, k), generator=g, device="cuda", dtype=torch.complex64))[0]
+    s = (U * lev) @ V.mH + 0.3 * torch.randn((P, F), generator=g, device="cuda", dtype=torch.complex64)
+    pd, ev = torch.empty(P, device="cuda"), torch.empty(F, dtype=torch.float64, device="cuda")
+    S = torch.view_as_real(s).contiguous()
+    fq.fq_clutter_svd(S, k_cut=k, want_iq_f=False, pd=pd, eigvals=ev)
+    s64 = s.to(torch.complex128)
+    lam, vec = torch.linalg.eigh(s64.mH @ s64)
+    lam, vec = lam.flip(0), vec.flip(1)[:, :k]
+    assert float((ev - lam).abs().max()) <= (2 * F * 2.0 ** -24 + 2.0 ** -22) * float(lam[0])
+    sf = s64 - (s64 @ vec) @ vec.mH
+    want = (sf.real ** 2 + sf.imag ** 2).mean(1)
+    assert rel_l2(pd.double().cpu().numpy(), want.cpu().numpy()) <= 1e-3
 
 
 # 16-bit channel data against the FP32 kernel on the same values: the
