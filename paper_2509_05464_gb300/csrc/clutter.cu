@@ -265,7 +265,11 @@ __global__ void __launch_bounds__(kGramThreads) gram_reduce_kernel(const float2 
 
 // ------------------------------------------------------------ eigen (1 CTA) --
 constexpr int kEigThreads = 1024;  // all eigenvectors (QL)
-constexpr int kTopThreads = 512;   // eigenvalues and the first vectors
+constexpr int kTopThreads = 512;   // eigenvalues and the first vectors, the matrix in shared memory
+// The first vectors of a matrix in global memory (F > 220) take 1024 threads:
+// the rows wait on the L2 cache (240 / 300 frames, k = 2: 2.85 / 5.32 ms at 512
+// threads, 2.55 / 4.34 at 1024).
+inline int top_threads(int F) { return eig_in_smem(F) ? kTopThreads : kEigThreads; }
 
 __device__ __forceinline__ int pidx(int i, int j) { return i * (i + 1) / 2 + j; }  // i >= j
 
@@ -284,7 +288,7 @@ __device__ __forceinline__ void back_transform_nq(int F, int ncol, const float *
     auto stage = [&](int c) {
         float2 *b = buf + (size_t)(c & 1) * nbuf * F;
         const int r0 = c * nbuf, cnt = min(nbuf, n - r0);
-        for (int t = threadIdx.x; t < cnt * F; t += blockDim.x) {
+        for (int t = threadIdx.x; t < cnt * F; t += 32 * nw) {
             const int r = t / F, i = t - r * F, k = n - 1 - (r0 + r);
             if (i > k) fqi::cp_async<8>(b + t, hv + (size_t)k * F + i);
             else b[t] = make_float2(0, 0);
@@ -391,11 +395,11 @@ __device__ __forceinline__ void sturm_below(const float *d, const float *e2, int
 // under the latency of the pivot recurrences), until the bracket is below 2^-31 of
 // the largest row sum -- a hundredth of the tridiagonalisation's rounding --
 // or holds no other number.
-__device__ void multisect(const float *d, const float *e2, int n, float lo0, float hi0, float tnorm, float *lam)
+__device__ void multisect(const float *d, const float *e2, int n, float lo0, float hi0, float tnorm, float *lam, int nt)
 {
     int np = 1;
-    while (np < 32 && 2 * np * n <= (int)blockDim.x / 2) np *= 2;
-    const int per = blockDim.x / np;  // eigenvalues of a pass
+    while (np < 32 && 2 * np * n <= nt / 2) np *= 2;
+    const int per = nt / np;  // eigenvalues of a pass
     const int lane = threadIdx.x & 31, p = threadIdx.x % np;
     const unsigned grp = (np == 32 ? 0xffffffffu : (1u << np) - 1u) << (lane - p);
     const float width = tnorm * 4.6566129e-10f;
@@ -974,7 +978,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
                                          double *__restrict__ lam_out, float2 *__restrict__ V,
                                          float2 *__restrict__ Vt, int k_cut, double thresh,
                                          int *__restrict__ k_out, int *__restrict__ status,
-                                         int topk_only, float *__restrict__ ii_scr)
+                                         int topk_only, float *__restrict__ ii_scr, int nt)
 {
     extern __shared__ float2 dyn[];
     float2 *Ap = big ? big : dyn;                 // packed lower triangle, later Z (real, stride F+1)
@@ -989,7 +993,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
     __shared__ int perm[512];
     __shared__ float s_scale;
     __shared__ int s_m, s_nrot, s_done, s_fail;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
 
     // scale to max |G_ij| <= 1 (eigenvectors unchanged, eigenvalues rescaled at the end)
     float amax = 0.0f;
@@ -1038,7 +1042,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
     __syncthreads();
     // diagonal unitary scaling making the off-diagonal real and >= 0: the phases
     // side by side, then their running product
-    for (int k = tid; k < F; k += blockDim.x) {
+    for (int k = tid; k < F; k += nt) {
         const float2 x = k + 1 < F ? ec[k] : make_float2(0, 0);
         const float ax = sqrtf(x.x * x.x + x.y * x.y);
         e[k] = ax;
@@ -1062,7 +1066,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
         float *e2 = spare, *lamd = spare + 512;
         __shared__ float s_lo, s_hi, s_tnorm;
         __shared__ int s_k;
-        for (int i = tid; i < F; i += blockDim.x) e2[i] = fmaxf(e[i] * e[i], 4.0f * FLT_MIN);  // > 0
+        for (int i = tid; i < F; i += nt) e2[i] = fmaxf(e[i] * e[i], 4.0f * FLT_MIN);  // > 0
         if (wid == 0) {
             float lo = 1e30f, hi = -1e30f, tn = 0.0f;
             for (int i = lane; i < F; i += 32) {
@@ -1084,9 +1088,9 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
             }
         }
         __syncthreads();
-        multisect(d, e2, F, s_lo, s_hi, s_tnorm, lamd);  // descending order
+        multisect(d, e2, F, s_lo, s_hi, s_tnorm, lamd, nt);  // descending order
         __syncthreads();
-        for (int j = tid; j < F; j += blockDim.x) lam_out[j] = (double)lamd[j] * (double)gscale;
+        for (int j = tid; j < F; j += nt) lam_out[j] = (double)lamd[j] * (double)gscale;
         if (tid == 0) {
             int k = k_cut;
             if (k < 0) {
@@ -1110,12 +1114,12 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
             // in the packed matrix's storage
             zk = k | 1;
             const bool in_z = !big && (size_t)F * zk + (size_t)6 * k * F <= (size_t)F * (F + 1);
-            for (int j = tid; j < k; j += blockDim.x) {
+            for (int j = tid; j < k; j += nt) {
                 if (in_z) {
                     float *z = reinterpret_cast<float *>(dyn);
                     inverse_iteration(d, e, F, lamd[j], tiny, j, z, zk, j, z + (size_t)F * zk + j, k);
                 } else {
-                    inverse_iteration(d, e, F, lamd[j], tiny, j, Z, zk, j, ii_scr + (size_t)j * 6 * F, 1);
+                    inverse_iteration(d, e, F, lamd[j], tiny, j, Z, zk, j, ii_scr + j, k);
                 }
             }
             __syncthreads();
@@ -1143,7 +1147,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
                     }
                 }
             }
-            for (int j = tid; j < F; j += blockDim.x) perm[j] = j;
+            for (int j = tid; j < F; j += nt) perm[j] = j;
             __syncthreads();
             // reflectors staged behind the k vectors (2 nbuf F complex values)
             const int nbuf = min(16, (F - zk) / 4);
@@ -1158,7 +1162,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
         }
     }
     // Z = identity (stride F+1), reusing the packed-matrix storage
-    for (int i = tid; i < F * zs; i += blockDim.x) Z[i] = ((i / zs) == (i % zs)) ? 1.0f : 0.0f;
+    for (int i = tid; i < F * zs; i += nt) Z[i] = ((i / zs) == (i % zs)) ? 1.0f : 0.0f;
     __syncthreads();
 
     // ---- implicit QL; thread 0 runs the scalar recurrence, everybody applies the rotations
@@ -1232,7 +1236,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
             const int done = s_done, nrot = s_nrot, mm = s_m, fail = s_fail;
             if (!done) {
                 // rotation r acts on columns (i, i+1) with i = m - 1 - r
-                for (int row = tid; row < F; row += blockDim.x) {
+                for (int row = tid; row < F; row += nt) {
                     float *zr = Z + row * zs;
                     for (int r = 0; r < nrot; ++r) {
                         int i = mm - 1 - r;
@@ -1253,7 +1257,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
     }
     __syncthreads();
     // ---- sort descending (rank by value, ties by index)
-    for (int i = tid; i < F; i += blockDim.x) {
+    for (int i = tid; i < F; i += nt) {
         float di = d[i];
         int rank = 0;
         for (int j = 0; j < F; ++j) {
@@ -1263,7 +1267,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
         perm[rank] = i;
     }
     __syncthreads();
-    for (int j = tid; j < F; j += blockDim.x) lam_out[j] = (double)d[perm[j]] * (double)gscale;
+    for (int j = tid; j < F; j += nt) lam_out[j] = (double)d[perm[j]] * (double)gscale;
     if (tid == 0) {
         int k = k_cut;
         if (k < 0) {
@@ -1289,20 +1293,25 @@ __global__ void __launch_bounds__(NT) eig_kernel(const float2 *__restrict__ G, i
                                                           int *__restrict__ k_out, int *__restrict__ status,
                                                           int topk_only, float *__restrict__ ii_scr)
 {
-    eig_body(G, F, big, hv, tau_g, lam_out, V, Vt, k_cut, thresh, k_out, status, topk_only, ii_scr);
+    eig_body(G, F, big, hv, tau_g, lam_out, V, Vt, k_cut, thresh, k_out, status, topk_only, ii_scr, NT);
 }
 
-// One CTA per ensemble of a wave; the packed matrix always in the workspace.
-__global__ void __launch_bounds__(kTopThreads) eig_batched_kernel(const fqb::EnsDev *__restrict__ ens,
-                                                                  const int *__restrict__ members)
+// One CTA per ensemble of a wave.  In a wave with a matrix too large for shared
+// memory (NT = 1024) the other members leave with the threads that a single call
+// would not have, so that their sums are the same.
+template <int NT>
+__global__ void __launch_bounds__(NT) eig_batched_kernel(const fqb::EnsDev *__restrict__ ens,
+                                                         const int *__restrict__ members)
 {
     const fqb::EnsDev &e = ens[members[blockIdx.x]];
+    const int nt = eig_in_smem(e.F) ? kTopThreads : NT;
+    if (threadIdx.x >= nt) return;
     char *ws = e.cws;
     double *lam = e.eigvals ? e.eigvals : (double *)(ws + e.cl_lam);
     int *kk = e.k_used ? e.k_used : (int *)(ws + e.cl_k);
     eig_body((const float2 *)(ws + e.cl_G), e.F, eig_in_smem(e.F) ? nullptr : (float2 *)(ws + e.cl_big), (float2 *)(ws + e.cl_hv),
              (float *)(ws + e.cl_tau), lam, (float2 *)(ws + e.cl_V), (float2 *)(ws + e.cl_Vt), e.k_cut,
-             e.energy_thresh, kk, e.status, 1, (float *)(ws + e.cl_ii));
+             e.energy_thresh, kk, e.status, 1, (float *)(ws + e.cl_ii), nt);
 }
 
 // ------------------------------------------------ projection + power Doppler --
@@ -1522,7 +1531,8 @@ fq_status launch_eig(const float2 *G, int F, float2 *big, float2 *hv, float *tau
                      float *ii_scr = nullptr)
 {
     size_t smem = big ? 0 : sizeof(float2) * (size_t)F * (F + 1) / 2;
-    auto kern = topk_only ? eig_kernel<kTopThreads> : eig_kernel<kEigThreads>;
+    const int nt = topk_only ? top_threads(F) : kEigThreads;
+    auto kern = nt == kTopThreads ? eig_kernel<kTopThreads> : eig_kernel<kEigThreads>;
     if (smem > 0) {
         // the kernel's static arrays count against the same 48 KB default,
         // so the opt-in is needed for much smaller packed matrices too
@@ -1530,7 +1540,7 @@ fq_status launch_eig(const float2 *G, int F, float2 *big, float2 *hv, float *tau
                                       "eig: smem attribute");
         if (s) return s;
     }
-    kern<<<1, topk_only ? kTopThreads : kEigThreads, smem, st>>>(G, F, big, hv, tau, lam, V, Vt, k_cut, thresh, k_out,
+    kern<<<1, nt, smem, st>>>(G, F, big, hv, tau, lam, V, Vt, k_cut, thresh, k_out,
                                                                 status, topk_only, ii_scr);
     return fqi::launch_check("fq_hermitian_eig");
 }
@@ -1871,12 +1881,14 @@ fq_status batched_gram_reduce(const fqb::EnsDev *ens, const fqb::StageQueue &q, 
 
 fq_status batched_eig(const fqb::EnsDev *ens, const int *members, int n, int F_max, cudaStream_t st)
 {
+    const int nt = top_threads(F_max);
     while (!eig_in_smem(F_max)) --F_max;  // larger members keep their matrix in the workspace
     const size_t smem = sizeof(float2) * (size_t)F_max * (F_max + 1) / 2;
-    fq_status s = cuda_check(cudaFuncSetAttribute(eig_batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    auto kern = nt == kTopThreads ? eig_batched_kernel<kTopThreads> : eig_batched_kernel<kEigThreads>;
+    fq_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)smem), "batched eig: smem attribute");
     if (s) return s;
-    eig_batched_kernel<<<n, kTopThreads, smem, st>>>(ens, members);
+    kern<<<n, nt, smem, st>>>(ens, members);
     return launch_check("batched eig");
 }
 

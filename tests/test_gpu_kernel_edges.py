@@ -11,6 +11,7 @@ from oracle import cnn as ocnn
 from paper_2509_05464_gb300 import build as fqbuild
 from paper_2509_05464_gb300 import fq
 from paper_2509_05464_gb300 import workload as W
+from paper_2509_05464_gb300.pipeline import Pipeline
 
 pytestmark = pytest.mark.gpu
 
@@ -128,3 +129,23 @@ def test_conv_frame_runs(shape):
     assert int(net.status.item()) == 0
     # FP32 sums of at most 1440 exact products of BF16 values
     assert np.abs(out.double().cpu().numpy() - ref).max() <= 1e-5 * np.abs(ref).max()
+
+
+def test_batch_of_small_and_large_eigen_problems():
+    """Members on both sides of the shared-memory limit of the eigen step in one
+    wave: each gives exactly what its single call gives."""
+    ms = [w for i, F in enumerate((240, 100, 222, 40))
+          for w in W.config4(seed=80 + i, n=1, s_range=(300, 800), f_range=(F, F), grids=((16, 1, 24),))]
+    b = fq.Batch(ms)
+    b.launch()
+    b.status()
+    torch.cuda.synchronize()
+    for i, w in enumerate(ms):
+        pl = Pipeline(w)
+        pl.upload()
+        pl.step()
+        fq.fq_clutter_status(pl.ws_svd)
+        torch.cuda.synchronize()
+        assert int(b.k_used[i].cpu()[0]) == int(pl.k_used.cpu()[0]), i
+        assert torch.equal(b.eigvals[i], pl.eigvals), i
+        assert torch.equal(b.pd[i], pl.pd), i
