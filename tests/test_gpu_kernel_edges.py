@@ -149,3 +149,29 @@ def test_batch_of_small_and_large_eigen_problems():
         assert int(b.k_used[i].cpu()[0]) == int(pl.k_used.cpu()[0]), i
         assert torch.equal(b.eigvals[i], pl.eigvals), i
         assert torch.equal(b.pd[i], pl.pd), i
+
+
+@pytest.mark.parametrize("F,Z,X", [(1, 1, 1), (15, 3, 5), (16, 5, 7), (33, 2, 33), (48, 9, 29), (65, 4, 16)])
+@pytest.mark.parametrize("remove_mean", [True, False])
+def test_filter_volume_frame_batches(F, Z, X, remove_mean):
+    """The learned filter's volume, target and power Doppler for frame counts
+    around the batches of loads: elementwise FP32 sums against FP64."""
+    g = torch.Generator(device="cuda").manual_seed(F)
+    iq = torch.randn((Z * X, F, 2), generator=g, device="cuda") + 0.5
+    vol = torch.full((F, Z, X, 32), 7.0, device="cuda", dtype=torch.bfloat16)
+    tgt = torch.empty((F, Z, X, 2), device="cuda")
+    _, _, sc = fq.fq_cnn_from_casorati(iq, F, Z, X, remove_mean, gain=2.0, vol=vol, target=tgt)
+    d = iq.double()
+    d = d - d.mean(1, keepdim=True) if remove_mean else d
+    sc_ref = 1.0 / d.square().mean().sqrt() if (F > 1 or not remove_mean) else sc.double()
+    eps = 2.0 ** -23
+    assert torch.allclose(sc.double().reshape(()), sc_ref.reshape(()), rtol=(F + 8) * eps, atol=0)
+    ref = (d * sc.double() * 2.0).permute(1, 0, 2).reshape(F, Z, X, 2)
+    # the mean of F values of size <= 6 and three roundings of the product
+    tol = ((F + 4) * eps * 6 * 2.0 * sc.double()).item()
+    assert (tgt.double() - ref).abs().max().item() <= tol
+    assert torch.equal(vol[..., :2], tgt.to(torch.bfloat16)) and not vol[..., 2:].any()
+    y = torch.randn((F, Z, X, 32), generator=g, device="cuda")
+    pd = fq.fq_cnn_power_doppler(y, 0.5)
+    pd_ref = y[..., :2].double().square().sum(-1).mean(0) / 0.25
+    assert ((pd.double().reshape(Z, X) - pd_ref).abs() <= (F + 6) * eps * pd_ref).all()
