@@ -1464,10 +1464,28 @@ __global__ void __launch_bounds__(NT, MINB) rf_synth_quad_kernel(const RfParams 
     rf_quad_tile<NT, OutT>(p, blockIdx.x, blockIdx.y, blockIdx.z, pos, amp, rf_base, rf, tile, sh);
 }
 
+// Words that the pass over the taps may address in records too short for
+// echoes clear of both ends (qn = 0).  Its lanes without such an echo add zeros
+// at samples 1 .. 2 dmax + 8, dmax = qlo + jmin: two whole delay offsets and the
+// taps around them.  Past the records those are words that nothing reads, but
+// they have to be the CTA's own.
+size_t quad_idle_words(const RfParams &p)
+{
+    if (p.qn > 0) return 0;
+    const size_t last = 2 * (size_t)(p.qlo + p.jmin);
+    size_t words = 0;
+    for (QuadBlock b(p.ag, p.pr.ns);; b.next(p.ag, p.pr.ns)) {
+        const size_t rows = b.guard ? b.guard + b.seg + 8 : last + 9;  // (segments: sample k is row k mod seg)
+        words = std::max(words, b.base + 32 * rows + (b.guard ? 4 * b.nb * (last / b.seg + 1) : 0));
+        if (b.b0 + b.nb >= p.ag) return words;
+    }
+}
+
 size_t quad_smem(const RfParams &p)
 {
     // the records and, before them, the pass-1 bins (2 x (Ns + 2 win) per angle)
-    return sizeof(int) * std::max<size_t>(quad_words(p.ag, p.pr.ns), 2 * (size_t)p.ag * (p.pr.ns + 2 * p.win));
+    const size_t words = std::max<size_t>(quad_words(p.ag, p.pr.ns), 2 * (size_t)p.ag * (p.pr.ns + 2 * p.win));
+    return sizeof(int) * std::max(words, quad_idle_words(p));
 }
 
 template <typename OutT>

@@ -175,3 +175,32 @@ def test_filter_volume_frame_batches(F, Z, X, remove_mean):
     pd = fq.fq_cnn_power_doppler(y, 0.5)
     pd_ref = y[..., :2].double().square().sum(-1).mean(0) / 0.25
     assert ((pd.double().reshape(Z, X) - pd_ref).abs() <= (F + 6) * eps * pd_ref).all()
+
+
+# records too short for echoes clear of both ends (at most 2 dmax + 9 samples,
+# dmax = ceil(3 pitch fs / c) + 2: 39 at 0.1 mm, 257 at 1 mm) up to the first
+# length that has them, in blocks of 1, 4 + 1, 8 and 8 + 1 angles.  FP32 bar:
+# 5e-6 and the phase of four roundings (of the difference of squares, the
+# root, the reciprocal, the product) of an element's delay offset from its
+# quad's first, at most 3 pitches
+@pytest.mark.parametrize("A", [1, 5, 8, 9])
+@pytest.mark.parametrize("ns,pitch", [(9, 0.1e-3), (16, 0.1e-3), (38, 0.1e-3), (39, 0.1e-3), (40, 0.1e-3),
+                                      (128, 1e-3), (256, 1e-3), (257, 1e-3), (258, 1e-3)])
+@pytest.mark.parametrize("dt", ["f32", "bf16", "f16"])
+def test_rf_short_records(A, ns, pitch, dt):
+    p = W.Probe(8, 1, pitch, pitch, 0.1e-3, 0.1e-3, 15.6e6, 62.5e6, 1540.0, 0.5, 2, ns)
+    rng = np.random.default_rng(100 * A + ns)
+    S, z1 = 517, 1.15 * ns * 1540.0 / 62.5e6 / 2
+    pos = np.stack([rng.uniform(-5 * pitch, 5 * pitch, S), np.zeros(S), rng.uniform(0.02e-3, z1, S)]).astype(np.float32)
+    amp = 1e-3 * rng.standard_normal(S).astype(np.float32)  # (1 / r is up to 5e4 here)
+    tx = list(np.radians(np.linspace(-6.0, 6.0, A))) if A > 1 else [0.0]
+    base = rng.standard_normal((A, 8, ns)).astype(np.float32)
+    t = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}[dt]
+    for b in (None, base):
+        got = fq.fq_simulate_rf(p, tx, [0.0] * A, torch.from_numpy(pos[None]).cuda(), torch.from_numpy(amp).cuda(), 1,
+                                rf_base=None if b is None else torch.from_numpy(b).cuda(), out_dtype=t)
+        want = oracle.simulate_rf(p, tx, [0.0] * A, pos, amp, rf=None if b is None else b.astype(np.float64),
+                                  accumulate=b is not None)
+        err = rel_l2(got[0].float().cpu().numpy().astype(np.float64), want)
+        f32 = 5e-6 + 2 * np.pi * p.f0 * 3 * pitch / p.c * 2.0 ** -22
+        assert err <= {"f32": f32, "bf16": 1e-2, "f16": 1e-3}[dt], (b is None, err)
