@@ -905,10 +905,14 @@ __device__ __forceinline__ void tridiagonalise_rows(float2 *Ap, int F, float *d,
 // 64 bits at 200 / 160 / 100 / 60 frames 1.8 / 4.6 / 1.8 / 3.3e-6 without it (the
 // former, slower tridiagonalisation 1.4 / 3.4 / 1.8 / 3.6e-6), 0.46 / 1.3 / 0.51 /
 // 1.1e-6 with it, for 0.03 ms at 200 frames.
+// G is scaled as in the decomposition (ginv: the power of two, exact), so that
+// the norms of the new vectors, about lambda_j, lie within 2^-12 / F and F at any
+// amplitude of the IQ (unscaled, their squares left binary32 beyond lambda 1.8e19
+// and below 1.1e-19, and the filter removed nothing).
 // Y: k F values of scratch.
 constexpr int kRefineMaxK = 8;
-__device__ __forceinline__ void refine_vectors(const float2 *__restrict__ G, int F, int k, const float *lam, float2 *Y,
-                                               float2 *V, float2 *Vt, int lane, int wid, int nw)
+__device__ __forceinline__ void refine_vectors(const float2 *__restrict__ G, float ginv, int F, int k, const float *lam,
+                                               float2 *Y, float2 *V, float2 *Vt, int lane, int wid, int nw)
 {
     __syncthreads();
     for (int i = wid; i < F; i += nw)
@@ -917,7 +921,8 @@ __device__ __forceinline__ void refine_vectors(const float2 *__restrict__ G, int
 #pragma unroll
             for (int u = 0; u < 4; ++u) s[u] = make_float2(0, 0);
             for (int f = lane; f < F; f += 32) {
-                const float2 g = G[(size_t)i * F + f];
+                float2 g = G[(size_t)i * F + f];
+                g = make_float2(g.x * ginv, g.y * ginv);
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     if (j0 + u < k) {
@@ -946,7 +951,7 @@ __device__ __forceinline__ void refine_vectors(const float2 *__restrict__ G, int
             for (int pass = 0; pass <= j; ++pass) {
                 float n2 = 0.0f;
                 for (int f = lane; f < F; f += 32) n2 = fmaf(y[f].x, y[f].x, fmaf(y[f].y, y[f].y, n2));
-                const float inv = rsqrtf(fmaxf(warp_sum(n2), FLT_MIN));  // unit length first: no overflow below
+                const float inv = rsqrtf(fmaxf(warp_sum(n2), FLT_MIN));
                 for (int f = lane; f < F; f += 32) y[f] = make_float2(y[f].x * inv, y[f].y * inv);
                 __syncwarp();
                 if (pass == j) break;
@@ -1157,7 +1162,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
             else
                 back_transform(F, k, Z, zk, perm, delta, hv, tau_g, V, Vt, nullptr, 0, lane, wid, nw);
             if (k <= kRefineMaxK && k < F)
-                refine_vectors(G, F, k, lamd, big || 2 * k > F + 1 ? reinterpret_cast<float2 *>(ii_scr) : dyn, V, Vt, lane, wid, nw);
+                refine_vectors(G, ginv, F, k, lamd, big || 2 * k > F + 1 ? reinterpret_cast<float2 *>(ii_scr) : dyn, V, Vt, lane, wid, nw);
             return;
         }
     }

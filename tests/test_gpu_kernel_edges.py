@@ -204,3 +204,46 @@ def test_rf_short_records(A, ns, pitch, dt):
         err = rel_l2(got[0].float().cpu().numpy().astype(np.float64), want)
         f32 = 5e-6 + 2 * np.pi * p.f0 * 3 * pitch / p.c * 2.0 ** -22
         assert err <= {"f32": f32, "bf16": 1e-2, "f16": 1e-3}[dt], (b is None, err)
+
+
+# every step of the filter scales by powers of two exactly, so an ensemble times
+# 2^n gives the same result times 2^n, bit for bit (eigenvalues and power
+# Doppler times 4^n); at 2^40 the largest eigenvalue is ~5e31
+@pytest.mark.parametrize("F,k", [(100, 1), (100, 2), (100, 8), (240, 2)])
+@pytest.mark.parametrize("form", ["f32", "bf16", "tf32 gram", "bf16 gram", "noalloc"])
+def test_clutter_filter_at_any_amplitude(F, k, form):
+    g = torch.Generator(device="cuda").manual_seed(F + k)
+    lev = 100.0 * 0.8 ** torch.arange(k, device="cuda")
+    U = torch.randn((4096, k), generator=g, device="cuda", dtype=torch.complex64)
+    V = torch.linalg.qr(torch.randn((F, k), generator=g, device="cuda", dtype=torch.complex64))[0]
+    s = (U * lev) @ V.mH + 0.3 * torch.randn((4096, F), generator=g, device="cuda", dtype=torch.complex64)
+    S = torch.view_as_real(s).to(torch.bfloat16 if form == "bf16" else torch.float32).contiguous()
+    mode = {"tf32 gram": fq.FQ_GRAM_TF32, "bf16 gram": fq.FQ_GRAM_BF16}.get(form, fq.FQ_GRAM_F32)
+
+    def run(n):
+        x = S * 2.0 ** n
+        o = fq.fq_clutter_svd_noalloc(x, k) if form == "noalloc" else fq.fq_clutter_svd(x, k, gram_mode=mode)
+        return o["iq_f"].double() * 2.0 ** -n, o["pd"].double() * 4.0 ** -n, o["eigvals"] * 4.0 ** -n
+
+    want = run(0)
+    assert float(want[1].mean()) < 2.0 * 2 * 0.3 ** 2  # the components are gone, the noise is left
+    for n in (-40, -20, 20, 40):
+        for a, b in zip(run(n), want):
+            assert torch.equal(a, b), n
+
+
+def test_batch_at_any_amplitude():
+    ms = W.config4(seed=90, n=2, s_range=(300, 800), f_range=(60, 80), grids=((32, 1, 48),))
+    out = []
+    for n in (0, -40, 24):
+        for w in ms:
+            w.amp = (w.amp * np.float32(2.0 ** n)).astype(np.float32)
+        b = fq.Batch(ms)
+        b.launch()
+        b.status()
+        out.append([p.double() * 4.0 ** -n for p in b.pd])
+        for w in ms:
+            w.amp = (w.amp * np.float32(2.0 ** -n)).astype(np.float32)
+    for o in out[1:]:
+        for a, b in zip(o, out[0]):
+            assert torch.equal(a, b)
