@@ -36,6 +36,11 @@ __host__ __device__ inline int gram_cols(int F) { return (F + 3) / 4; }
 __host__ __device__ inline int gram_blocks(int F) { return gram_cols(F) * (gram_cols(F) + 1) / 2; }
 __host__ __device__ inline int gram_parts(int F) { return (gram_blocks(F) + kGramThreads - 1) / kGramThreads; }
 size_t gram_smem(int F) { return 2 * (size_t)kGramPx * 2 * gram_cols(F) * sizeof(float4); }
+// Dynamic shared memory the kernels are opted in to: the most of any call, not
+// the call's own, which another thread's smaller call could take back between
+// this thread's opt-in and its launch.
+constexpr int kMaxF = 512;
+constexpr size_t kEigSmemMax = 190 * 1024;
 constexpr int kFastMaxK = 48;  // top-k eigenvectors by inverse iteration up to this k
 
 inline size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -50,7 +55,7 @@ int gram_chunks(int64_t P, int F)
     return want;
 }
 
-__host__ __device__ inline bool eig_in_smem(int F) { return (size_t)F * (F + 1) / 2 * sizeof(float2) <= 190 * 1024; }
+__host__ __device__ inline bool eig_in_smem(int F) { return (size_t)F * (F + 1) / 2 * sizeof(float2) <= kEigSmemMax; }
 
 // Operand bytes of the tensor-core Gram modes (0 = CUDA-core FP32 Gram).
 int tc_esz(int gram_mode) { return gram_mode == FQ_GRAM_BF16 ? 2 : (gram_mode == FQ_GRAM_TF32 ? 4 : 0); }
@@ -1513,7 +1518,7 @@ fq_status launch_gram(const void *S, int64_t P, int F, const ClutterLayout &L, c
     float2 *part = (float2 *)(ws + L.part);
     const size_t smem = gram_smem(F);
     fq_status s = fqi::cuda_check(cudaFuncSetAttribute(gram_partial_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)smem), "fq_casorati_gram: smem attribute");
+                                                       (int)gram_smem(kMaxF)), "fq_casorati_gram: smem attribute");
     if (s) return s;
     dim3 grid(gram_parts(F), L.n_chunks);
     gram_partial_kernel<T><<<grid, kGramThreads, smem, st>>>((const T *)S, P, F, L.chunk_len, part);
@@ -1541,8 +1546,8 @@ fq_status launch_eig(const float2 *G, int F, float2 *big, float2 *hv, float *tau
     if (smem > 0) {
         // the kernel's static arrays count against the same 48 KB default,
         // so the opt-in is needed for much smaller packed matrices too
-        fq_status s = fqi::cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                                      "eig: smem attribute");
+        fq_status s = fqi::cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)kEigSmemMax), "eig: smem attribute");
         if (s) return s;
     }
     kern<<<1, nt, smem, st>>>(G, F, big, hv, tau, lam, V, Vt, k_cut, thresh, k_out,
@@ -1858,8 +1863,8 @@ fq_status launch_gram_batched(const fqb::EnsDev *ens, const fqb::StageQueue &q, 
 {
     const size_t smem = gram_smem(F_max);
     auto kern = gram_batched_kernel<T>;
-    fq_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                             "batched Gram: smem attribute");
+    fq_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)gram_smem(kMaxF)), "batched Gram: smem attribute");
     if (s) return s;
     kern<<<fqb::persistent_grid(kern, kGramThreads, smem, items), kGramThreads, smem, st>>>(ens, q);
     return launch_check("batched Gram");
@@ -1891,7 +1896,7 @@ fq_status batched_eig(const fqb::EnsDev *ens, const int *members, int n, int F_m
     const size_t smem = sizeof(float2) * (size_t)F_max * (F_max + 1) / 2;
     auto kern = nt == kTopThreads ? eig_batched_kernel<kTopThreads> : eig_batched_kernel<kEigThreads>;
     fq_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem), "batched eig: smem attribute");
+                                                  (int)kEigSmemMax), "batched eig: smem attribute");
     if (s) return s;
     kern<<<n, nt, smem, st>>>(ens, members);
     return launch_check("batched eig");

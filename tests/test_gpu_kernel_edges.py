@@ -2,6 +2,8 @@
 segments of the RF kernel, pixel panels and column blocks of the FP32 Gram,
 register blocks of the tridiagonalisation, frame groups and voxel pairs of
 the 16-bit delay-and-sum, accumulator runs of the convolution."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -247,3 +249,31 @@ def test_batch_at_any_amplitude():
     for o in out[1:]:
         for a, b in zip(o, out[0]):
             assert torch.equal(a, b)
+
+
+def test_threads_with_different_frame_counts():
+    """Gram matrices of 40 and 200 frames (less and more than 48 KB of shared
+    memory) from threads on their own streams: no call takes back what
+    another is about to launch with (a race: seen in one of 40000 launches)."""
+    errors = []
+
+    def work(F):
+        try:
+            g = torch.Generator(device="cuda").manual_seed(F)
+            S = torch.randn((8, F, 2), generator=g, device="cuda")
+            want, G = fq.fq_casorati_gram(S), torch.empty((F, F, 2), device="cuda")
+            torch.cuda.synchronize()
+            ws, st = fq.workspace(fq.fq_gram_workspace_size(8, F)), torch.cuda.Stream()
+            for _ in range(20000):
+                fq.fq_casorati_gram(S, G=G, ws=ws, stream=st)
+            st.synchronize()
+            assert torch.equal(G, want), F
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    ts = [threading.Thread(target=work, args=(F,)) for F in (40, 200, 40, 200, 40)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not errors, errors
