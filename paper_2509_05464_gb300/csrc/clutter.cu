@@ -348,9 +348,17 @@ __device__ __forceinline__ void back_transform_nq(int F, int ncol, const float *
         } else if (on) {
             for (int k = n - 1; k >= 0; --k) apply(hv + (size_t)k * F, k, false);
         }
+        // unit length again: the reflectors are unitary to their rounding only, and
+        // what is missing of the largest components stays in the filtered IQ
+        float n2 = 0.0f;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) n2 = fmaf(y[q].x, y[q].x, fmaf(y[q].y, y[q].y, n2));
+        for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        const float unit = fmaf(-0.5f, n2, 1.5f);  // 1 / sqrt(n2) for n2 = 1 + 1e-5
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
             const int i = lane + 32 * q;
+            y[q] = make_float2(y[q].x * unit, y[q].y * unit);
             if (on && i < F) {
                 if (V) V[(size_t)i * F + j] = y[q];
                 Vt[(size_t)j * F + i] = y[q];
@@ -534,7 +542,10 @@ __device__ __forceinline__ void inverse_iteration(const float *d, const float *e
 // lane walks its stored row, beyond it the stored rows of the column block,
 // conjugated), up to four warps a row block; the update with a lane per
 // column, one 16-byte broadcast (v_i, w_i) a row.  The first column of the new
-// trailing matrix comes out of the update.  Former versions: warp
+// trailing matrix comes out of the update.  A block's part of A v is summed in
+// four chains of eight before it joins the row's sum (one or two chains over
+// all blocks: eigenvalues 1.5 times as far off at 200 frames, the same time).
+// Former versions: warp
 // per row with nine barriers a step 1.5 ms at 200 frames (3.0M cycles), two
 // barriers and v, w in registers 2.6M cycles (30k instructions a step).
 constexpr int kPartStride = 224;
@@ -571,11 +582,12 @@ __device__ __forceinline__ void reflector(const float2 *x, int m, int lane, floa
     }
 }
 
-__device__ __forceinline__ float2 rank2(float2 c, float2 vi, float2 wi, float2 x, float2 y)  // c - vi conj(y) - wi conj(x)
+// c - (vi conj(y) + wi conj(x)): the small correction first, so that c is rounded once
+__device__ __forceinline__ float2 rank2(float2 c, float2 vi, float2 wi, float2 x, float2 y)
 {
-    c.x = fmaf(-vi.x, y.x, fmaf(-vi.y, y.y, fmaf(-wi.x, x.x, fmaf(-wi.y, x.y, c.x))));
-    c.y = fmaf(-vi.y, y.x, fmaf(vi.x, y.y, fmaf(-wi.y, x.x, fmaf(wi.x, x.y, c.y))));
-    return c;
+    const float u = fmaf(vi.x, y.x, fmaf(vi.y, y.y, fmaf(wi.x, x.x, wi.y * x.y)));
+    const float v = fmaf(vi.y, y.x, fmaf(-vi.x, y.y, fmaf(wi.y, x.x, -wi.x * x.y)));
+    return make_float2(c.x - u, c.y - v);
 }
 
 __device__ __forceinline__ void tridiagonalise_blocks(float2 *Ap, int F, float *d, float2 *ec, float2 *vvA, float2 *vvB,
@@ -609,43 +621,52 @@ __device__ __forceinline__ void tridiagonalise_blocks(float2 *Ap, int F, float *
         if (wid < W * nb) {
             const int rb = wid / W, ws = wid - rb * W;
             const int i = 32 * rb + lane, ic = min(i, m - 1);
-            float2 s = make_float2(0, 0), t = make_float2(0, 0);  // two chains
+            float2 s = make_float2(0, 0);
             for (int cb = ws; cb < nb; cb += W) {
                 const float2 *v = vv + 32 * cb;
+                float2 c[4];  // the block's sum in four chains of eight, then added to s
+#pragma unroll
+                for (int u = 0; u < 4; ++u) c[u] = make_float2(0, 0);
                 if (cb < rb) {
                     const float2 *a = Ap + pidx(k + 1 + ic, k + 1 + 32 * cb);
-#pragma unroll 8
-                    for (int j = 0; j < 32; j += 2) {
-                        const float2 a0 = a[j], a1 = a[j + 1], x0 = v[j], x1 = v[j + 1];
-                        s.x = fmaf(a0.x, x0.x, fmaf(-a0.y, x0.y, s.x));
-                        s.y = fmaf(a0.x, x0.y, fmaf(a0.y, x0.x, s.y));
-                        t.x = fmaf(a1.x, x1.x, fmaf(-a1.y, x1.y, t.x));
-                        t.y = fmaf(a1.x, x1.y, fmaf(a1.y, x1.x, t.y));
-                    }
+#pragma unroll 2
+                    for (int j = 0; j < 32; j += 4)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const float2 a0 = a[j + u], x0 = v[j + u];
+                            c[u].x = fmaf(a0.x, x0.x, fmaf(-a0.y, x0.y, c[u].x));
+                            c[u].y = fmaf(a0.x, x0.y, fmaf(a0.y, x0.x, c[u].y));
+                        }
                 } else if (cb > rb) {
                     const int n = min(32, m - 32 * cb);
                     int o = pidx(k + 1 + 32 * cb, k + 1 + i), st = k + 2 + 32 * cb;  // row 32 cb + j: o += its length
-#pragma unroll 8
-                    for (int j = 0; j < n; ++j) {
-                        const float2 a0 = Ap[o], x0 = v[j];
-                        o += st++;
-                        s.x = fmaf(a0.x, x0.x, fmaf(a0.y, x0.y, s.x));
-                        s.y = fmaf(a0.x, x0.y, fmaf(-a0.y, x0.x, s.y));
-                    }
+#pragma unroll 2
+                    for (int j = 0; j < n; j += 4)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const float2 a0 = Ap[j + u < n ? o : 0], x0 = v[j + u];  // (v = 0 past the end)
+                            o += st++;
+                            c[u].x = fmaf(a0.x, x0.x, fmaf(a0.y, x0.y, c[u].x));
+                            c[u].y = fmaf(a0.x, x0.y, fmaf(-a0.y, x0.x, c[u].y));
+                        }
                 } else {
                     const int n = min(32, m - 32 * cb);
                     const int own = pidx(k + 1 + ic, k + 1 + 32 * cb);
-#pragma unroll 4
-                    for (int j = 0; j < n; ++j) {
-                        const bool low = j <= ic - 32 * cb;
-                        const float2 a0 = Ap[low ? own + j : pidx(k + 1 + 32 * cb + j, k + 1 + ic)], x0 = v[j];
-                        const float ay = low ? a0.y : -a0.y;
-                        s.x = fmaf(a0.x, x0.x, fmaf(-ay, x0.y, s.x));
-                        s.y = fmaf(a0.x, x0.y, fmaf(ay, x0.x, s.y));
-                    }
+                    for (int j = 0; j < n; j += 4)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int jc = min(j + u, n - 1);
+                            const bool low = jc <= ic - 32 * cb;
+                            const float2 a0 = Ap[low ? own + jc : pidx(k + 1 + 32 * cb + jc, k + 1 + ic)], x0 = v[j + u];
+                            const float ay = low ? a0.y : -a0.y;
+                            c[u].x = fmaf(a0.x, x0.x, fmaf(-ay, x0.y, c[u].x));
+                            c[u].y = fmaf(a0.x, x0.y, fmaf(ay, x0.x, c[u].y));
+                        }
                 }
+                s.x += (c[0].x + c[1].x) + (c[2].x + c[3].x);
+                s.y += (c[0].y + c[1].y) + (c[2].y + c[3].y);
             }
-            if (i < m) es.part[ws * kPartStride + i] = make_float2(s.x + t.x, s.y + t.y);
+            if (i < m) es.part[ws * kPartStride + i] = s;
         }
         __syncthreads();
         // ---- p, K (every warp), w
@@ -907,9 +928,8 @@ __device__ __forceinline__ void tridiagonalise_rows(float2 *Ap, int F, float *d,
 // k <= kRefineMaxK vectors, where lambda_j is well above the rounding of G.
 // It takes the rounding of the F reflectors out of the filter's subspace (a
 // factor lambda_{k+1} / lambda_k of it stays): error of the filtered IQ against
-// 64 bits at 200 / 160 / 100 / 60 frames 1.8 / 4.6 / 1.8 / 3.3e-6 without it (the
-// former, slower tridiagonalisation 1.4 / 3.4 / 1.8 / 3.6e-6), 0.46 / 1.3 / 0.51 /
-// 1.1e-6 with it, for 0.03 ms at 200 frames.
+// 64 bits, components 1.4 dB apart, 200 frames: 0.46e-6 for k = 8 with it, 1.33e-6
+// for k = 9 without, for 0.03 ms.
 // G is scaled as in the decomposition (ginv: the power of two, exact), so that
 // the norms of the new vectors, about lambda_j, lie within 2^-12 / F and F at any
 // amplitude of the IQ (unscaled, their squares left binary32 beyond lambda 1.8e19

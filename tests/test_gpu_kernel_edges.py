@@ -277,3 +277,39 @@ def test_threads_with_different_frame_counts():
     for t in ts:
         t.join()
     assert not errors, errors
+
+
+# F reflectors, each unitary to its rounding, and unit vectors at the end: V^H V
+# within (F + 8) 2^-24 of the identity
+@pytest.mark.parametrize("F", [2, 3, 5, 40, 100, 128, 160, 220, 221, 300])
+def test_eigenvectors_are_orthonormal(F):
+    g = torch.Generator(device="cuda").manual_seed(F)
+    A = torch.randn((2 * F, F), generator=g, device="cuda", dtype=torch.complex128)
+    G = torch.view_as_real((A.mH @ A).to(torch.complex64)).contiguous()
+    lam, V, ws = fq.fq_hermitian_eig(G)
+    fq.fq_clutter_status(ws)
+    V = torch.view_as_complex(V.double())
+    G64 = torch.view_as_complex(G.double())
+    assert float((V.mH @ V - torch.eye(F, device="cuda")).abs().max()) <= (F + 8) * 2.0 ** -24
+    assert float((G64 @ V - V * lam).norm()) <= 2 * F * 2.0 ** -24 * float(G64.norm())
+
+
+# components removed without the subspace step (more than 8), with the solves'
+# scratch in and beyond the matrix's storage; eigenvalues within 2 F 2^-24 of
+# the largest turn the subspace by that over the gap
+@pytest.mark.parametrize("F", [60, 130, 160, 220, 240])
+@pytest.mark.parametrize("k", [0, 1, 8, 9, 24, 48])
+def test_filtered_iq_of_many_components(F, k):
+    g = torch.Generator(device="cuda").manual_seed(1000 * k + F)
+    lev = torch.linspace(100.0, 50.0, max(k, 1), device="cuda")[:k]
+    U = torch.randn((4096, k), generator=g, device="cuda", dtype=torch.complex64)
+    V = torch.linalg.qr(torch.randn((F, max(k, 1)), generator=g, device="cuda", dtype=torch.complex64))[0][:, :k]
+    s = (U * lev) @ V.mH + 0.3 * torch.randn((4096, F), generator=g, device="cuda", dtype=torch.complex64)
+    S = torch.view_as_real(s).contiguous()
+    got = torch.view_as_complex(fq.fq_clutter_svd(S, k)["iq_f"].double())
+    s64 = torch.view_as_complex(S.double())
+    lam, vec = torch.linalg.eigh(s64.mH @ s64)
+    lam, vec = lam.flip(0), vec.flip(1)[:, :k]
+    want = s64 - (s64 @ vec) @ vec.mH
+    turn = (2 * F * 2.0 ** -24 + 2.0 ** -22) * float(lam[0] / (lam[k - 1] - lam[k])) if k else 0.0
+    assert float((got - want).norm()) <= (turn + (F + 8) * 2.0 ** -24) * float(s64.norm())
