@@ -1195,7 +1195,12 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
     for (int i = tid; i < F * zs; i += nt) Z[i] = ((i / zs) == (i % zs)) ? 1.0f : 0.0f;
     __syncthreads();
 
-    // ---- implicit QL; thread 0 runs the scalar recurrence, everybody applies the rotations
+    // ---- implicit QL; thread 0 runs the scalar recurrence, everybody applies the
+    // rotations.  An off-diagonal counts as zero below the rounding of its
+    // neighbours or a thousandth of that of the whole matrix; where ten sweeps (two or
+    // three are usual) have not come to that, the sweeps' own rounding keeps it
+    // above, and the rounding of the whole matrix is what can be had (without this
+    // 1 of 8 matrices of 100 frames and half of those of 300 did not converge)
     float tnorm = 0.0f;
     if (tid == 0) {
         for (int i = 0; i < F; ++i) tnorm = fmaxf(tnorm, fabsf(d[i]) + fabsf(e[i]));
@@ -1208,7 +1213,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
                 int m = l;
                 for (; m < F - 1; ++m) {
                     float dd = fabsf(d[m]) + fabsf(d[m + 1]);
-                    if (fabsf(e[m]) <= FLT_EPSILON * dd || fabsf(e[m]) <= 1e-3f * FLT_EPSILON * tnorm) break;
+                    if (fabsf(e[m]) <= FLT_EPSILON * dd || fabsf(e[m]) <= (iter < 10 ? 1e-3f : 1.0f) * FLT_EPSILON * tnorm) break;
                 }
                 s_done = (m == l);
                 s_nrot = 0;

@@ -313,3 +313,31 @@ def test_filtered_iq_of_many_components(F, k):
     want = s64 - (s64 @ vec) @ vec.mH
     turn = (2 * F * 2.0 ** -24 + 2.0 ** -22) * float(lam[0] / (lam[k - 1] - lam[k])) if k else 0.0
     assert float((got - want).norm()) <= (turn + (F + 8) * 2.0 ** -24) * float(s64.norm())
+
+
+# matrices of a few large eigenvalues over many near the rounding of the largest
+# (slowly turning clutter, blood, noise 46 dB below), all vectors: converges,
+# and the eigenvalues are within 2 F 2^-24 of the largest
+@pytest.mark.parametrize("F", [100, 160, 220, 300])
+def test_all_eigenvectors_of_clutter(F):
+    t = torch.arange(F, device="cuda", dtype=torch.float32)[None]
+    for seed in range(8):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+
+        def randn(*n):
+            return torch.randn(n, generator=g, device="cuda", dtype=torch.complex64)
+
+        s = 0.05 * randn(4096, F)
+        for j, (lev, w) in enumerate(((10.0, 0.004), (5.0, 0.09), (2.0, -0.17))):
+            s = s + lev * randn(4096, 1) * torch.polar(1.0 + 0.05 * torch.sin(0.03 * (j + 1) * t),
+                                                       w * t + 0.4 * torch.sin(0.02 * (j + 1) * t))
+        shift = 0.3 + 1.2 * torch.rand((4096, 1), generator=g, device="cuda")
+        s = s + randn(4096, 1) * torch.polar(torch.ones_like(shift * t), shift * t)
+        G = torch.view_as_real((s.to(torch.complex128).mH @ s.to(torch.complex128)).to(torch.complex64)).contiguous()
+        lam, V, ws = fq.fq_hermitian_eig(G)
+        fq.fq_clutter_status(ws)
+        G64 = torch.view_as_complex(G.double())
+        want = torch.linalg.eigvalsh(torch.tril(G64) + torch.tril(G64, -1).mH).flip(0)
+        assert float((lam - want).abs().max()) <= (2 * F * 2.0 ** -24 + 2.0 ** -22) * float(want[0]), seed
+        o = fq.fq_clutter_svd(torch.view_as_real(s).contiguous(), 50, want_iq_f=False)
+        fq.fq_clutter_status(o["ws"])
