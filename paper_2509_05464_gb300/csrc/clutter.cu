@@ -402,44 +402,49 @@ __device__ __forceinline__ void sturm_below(const float *d, const float *e2, int
     cb = c1;
 }
 
+// binary32 as integers of the same order (and back)
+__device__ __forceinline__ int ordered_bits(int b) { return b ^ ((b >> 31) & 0x7fffffff); }
+
 // The eigenvalues in descending order by multisection on [lo, hi]: np threads
 // (a power of two that divides the warp) per eigenvalue evaluate two points of
-// its bracket each a round (np = 2 at 200 frames, where 13 warps still fit
-// under the latency of the pivot recurrences), until the bracket is below 2^-31 of
-// the largest row sum -- a hundredth of the tridiagonalisation's rounding --
-// or holds no other number.
-__device__ void multisect(const float *d, const float *e2, int n, float lo0, float hi0, float tnorm, float *lam, int nt)
+// its bracket each a round, until the bracket holds no other number.  The points
+// divide the numbers of the bracket evenly, not its length, so that an eigenvalue
+// takes log_(2 np + 1) 2^32 rounds whatever its size (20 for np = 1), and small
+// ones of a graded matrix are good to their last bits (halving the length to
+// 2^-31 of the largest row sum took as long).
+__device__ void multisect(const float *d, const float *e2, int n, float lo0, float hi0, float *lam, int nt)
 {
     int np = 1;
     while (np < 32 && 2 * np * n <= nt / 2) np *= 2;
     const int per = nt / np;  // eigenvalues of a pass
     const int lane = threadIdx.x & 31, p = threadIdx.x % np;
     const unsigned grp = (np == 32 ? 0xffffffffu : (1u << np) - 1u) << (lane - p);
-    const float width = tnorm * 4.6566129e-10f;
+    const unsigned part = 0xffffffffu / (unsigned)(2 * np + 1) + 1u;
     for (int j0 = 0; j0 < n; j0 += per) {
         const int j = j0 + (int)threadIdx.x / np;
         const int m = n - 1 - j;  // m-th smallest
-        float lo = lo0, hi = hi0;
-        bool act = j < n;
-        for (int it = 0; it < 80; ++it) {
-            const float mid = 0.5f * (lo + hi);
-            act = act && mid > lo && mid < hi && hi - lo > width;
+        int lo = ordered_bits(__float_as_int(lo0)), hi = ordered_bits(__float_as_int(hi0));
+        bool act = j < n && lo < hi;
+        for (int it = 0; it < 40; ++it) {
+            const unsigned gap = (unsigned)hi - (unsigned)lo;
+            act = act && gap > 1u;
             if (!__any_sync(0xffffffffu, act)) break;
             // the 2 np points, computed alike by every thread of the group
-            const float h = hi - lo, inv = 1.0f / (float)(2 * np + 1);
-            auto point = [&](int i) { return fminf(fmaxf(fmaf(h, (float)(i + 1) * inv, lo), lo), hi); };
+            auto point = [&](int i) { return (int)((unsigned)lo + __umulhi(gap, (unsigned)(i + 1) * part)); };
+            auto value = [&](int i) { return __int_as_float(ordered_bits(point(i))); };
             int ca = 0, cb = 0;
-            if (act) sturm_below(d, e2, n, point(2 * p), point(2 * p + 1), ca, cb);
+            if (act) sturm_below(d, e2, n, value(2 * p), value(2 * p + 1), ca, cb);
             const unsigned ba = __ballot_sync(0xffffffffu, act && ca < m + 1) & grp;
             const unsigned bb = __ballot_sync(0xffffffffu, act && cb < m + 1) & grp;
             const int c = __popc(ba) + __popc(bb);  // points below the eigenvalue
             if (act) {
-                const float nlo = c > 0 ? point(c - 1) : lo, nhi = c < 2 * np ? point(c) : hi;
+                const int nlo = c > 0 ? point(c - 1) : lo, nhi = c < 2 * np ? point(c) : hi;
                 lo = nlo;
                 hi = nhi;
             }
         }
-        if (j < n && p == 0) lam[j] = 0.5f * (lo + hi);
+        if (j < n && p == 0)
+            lam[j] = 0.5f * (__int_as_float(ordered_bits(lo)) + __int_as_float(ordered_bits(hi)));
     }
 }
 
@@ -1091,8 +1096,8 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
     __syncthreads();
     const int zs = F + 1;
     if (topk_only) {
-        // ---- all eigenvalues by bisection (one thread each), top-k vectors by
-        // inverse iteration; the QL path below is the fallback for large k
+        // ---- all eigenvalues by multisection, top-k vectors by inverse iteration;
+        // the QL path below is the fallback for large k
         float *e2 = spare, *lamd = spare + 512;
         __shared__ float s_lo, s_hi, s_tnorm;
         __shared__ int s_k;
@@ -1118,7 +1123,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
             }
         }
         __syncthreads();
-        multisect(d, e2, F, s_lo, s_hi, s_tnorm, lamd, nt);  // descending order
+        multisect(d, e2, F, s_lo, s_hi, lamd, nt);  // descending order
         __syncthreads();
         for (int j = tid; j < F; j += nt) lam_out[j] = (double)lamd[j] * (double)gscale;
         if (tid == 0) {

@@ -341,3 +341,15 @@ def test_all_eigenvectors_of_clutter(F):
         assert float((lam - want).abs().max()) <= (2 * F * 2.0 ** -24 + 2.0 ** -22) * float(want[0]), seed
         o = fq.fq_clutter_svd(torch.view_as_real(s).contiguous(), 50, want_iq_f=False)
         fq.fq_clutter_status(o["ws"])
+
+
+# the Gram matrix of orthogonal frames is diagonal, exactly: its eigenvalues, over
+# nine decades, to the last bits of binary32
+@pytest.mark.parametrize("F", [2, 10, 40, 100, 200, 260])
+def test_eigenvalues_of_graded_frames(F):
+    a = torch.tensor([10.0 ** (-4.5 * i / (F - 1)) for i in range(F)], device="cuda")
+    S = torch.zeros((F, F, 2), device="cuda")
+    S[torch.arange(F), torch.arange(F).flip(0), 0] = a
+    lam = fq.fq_clutter_svd(S, 1)["eigvals"]
+    want = (a * a).double()
+    assert float(((lam - want).abs() / want).max()) <= 4 * 2.0 ** -24
