@@ -553,13 +553,19 @@ __global__ void sum_parts_kernel(const double *__restrict__ part, int n, int64_t
 // free under the swizzle.  A CTA writes one partial (kWgVals floats); the
 // partials are summed in order by wgrad_reduce_kernel.
 //
+// The tensor core's accumulation truncates, a bias that grows with the steps
+// of a running sum (1.2e-6 of the gradients at 1.7k voxels a CTA, 1.5e-4 at
+// 86k), so an accumulator runs over the 32 voxels of a row only, from zero, and
+// is added to the running sum in FP32: 5.4e-8 and 7.9e-8, for 0.03 ms of a
+// training step (every 16 voxels: 5.6e-8, 0.07 ms).
+//
 // Why: one thread per four results on the CUDA cores with a shared-memory
 // step of 64 voxels re-read x and dy for each of the 45 taps (3.3 ms a
 // layer), and its reduction summed db in one CTA (1.5 ms).  Four layers of a
-// training step of 4 volumes of 64 x 32 x 32 voxels: 19.1 -> 0.24 ms
-// (step 20.4 -> 1.57 ms); bound by the mma.sync rate (24 per 16 voxels and
-// warp).  tcgen05 would need 4 taps per M = 128 operand at unequal row
-// offsets, which its descriptors cannot express.
+// training step of 4 volumes of 64 x 32 x 32 voxels: 19.1 -> 0.29 ms; bound by
+// the mma.sync rate (24 per 16 voxels and warp) and the additions.  tcgen05
+// would need 4 taps per M = 128 operand at unequal row offsets, which its
+// descriptors cannot express.
 constexpr int kHaloX = TILE_X + 2, kHaloZ = TILE_Z + 2;
 constexpr int kWgWarps = 15;                    // (dt, dz)
 constexpr int kWgThreads = 32 * (kWgWarps + 1);  // and the TMA warp
@@ -579,13 +585,23 @@ __device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4])
                  : "memory");
 }
 
-__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+// t += A B
+__device__ __forceinline__ void mma16816(float (&t)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
         "{%0, %1, %2, %3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "+f"(t[0]), "+f"(t[1]), "+f"(t[2]), "+f"(t[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// t = A B
+__device__ __forceinline__ void mma16816z(float (&t)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%10, %10, %10, %10};"
+        : "=f"(t[0]), "=f"(t[1]), "=f"(t[2]), "=f"(t[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
 }
 
 // byte offset of 16-byte chunk c of 64-byte row q under the 64-byte swizzle
@@ -683,32 +699,40 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                     if (!warp_wait(&g_full[sg], (uint32_t)(jg / kWgDySlots) & 1u)) { ok = false; break; }
                     const uint32_t xb = smem_u32(xs + s * kWgXSlotB), gb = smem_u32(gs + sg * kWgDyB);
 #pragma unroll 1
-                    for (int ks = 0; ks < TILE_M / 16; ++ks) {
-                        uint32_t b[(NT + 1) / 2][4];
+                    for (int ks = 0; ks < TILE_M / 16; ks += 2) {  // the 32 pixels of a row
+                        uint32_t b[2][(NT + 1) / 2][4];
 #pragma unroll
-                        for (int n = 0; n < (NT + 1) / 2; ++n)
-                            ldsm4t(gb + sw64_off(16 * ks + b_row, 2 * n + b_ch), b[n]);
-                        const int q0 = ((ks >> 1) + dzi) * kHaloX + 16 * (ks & 1) + a_row;
+                        for (int q = 0; q < 2; ++q)
+#pragma unroll
+                            for (int n = 0; n < (NT + 1) / 2; ++n)
+                                ldsm4t(gb + sw64_off(16 * (ks + q) + b_row, 2 * n + b_ch), b[q][n]);
+                        const int q0 = ((ks >> 1) + dzi) * kHaloX + a_row;
 #pragma unroll
                         for (int dx = 0; dx < 3; ++dx) {
 #pragma unroll
                             for (int m = 0; m < 2; ++m) {
-                                uint32_t a[4];
-                                ldsm4t(xb + sw64_off(q0 + dx, 2 * m + a_ch), a);
+                                uint32_t a0[4], a1[4];
+                                ldsm4t(xb + sw64_off(q0 + dx, 2 * m + a_ch), a0);
+                                ldsm4t(xb + sw64_off(q0 + 16 + dx, 2 * m + a_ch), a1);
 #pragma unroll
-                                for (int n = 0; n < NT; ++n)
-                                    mma16816(acc[dx][m][n], a, b[n / 2][2 * (n & 1)], b[n / 2][2 * (n & 1) + 1]);
+                                for (int n = 0; n < NT; ++n) {
+                                    float t[4];
+                                    mma16816z(t, a0, b[0][n / 2][2 * (n & 1)], b[0][n / 2][2 * (n & 1) + 1]);
+                                    mma16816(t, a1, b[1][n / 2][2 * (n & 1)], b[1][n / 2][2 * (n & 1) + 1]);
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) acc[dx][m][n][i] += t[i];
+                                }
                             }
                         }
                         if (warp == 0) {
 #pragma unroll
-                            for (int n = 0; n < NT; ++n) {
-                                const float2 u = __bfloat1622float2(
-                                    *reinterpret_cast<const __nv_bfloat162 *>(&b[n / 2][2 * (n & 1)]));
-                                const float2 v = __bfloat1622float2(
-                                    *reinterpret_cast<const __nv_bfloat162 *>(&b[n / 2][2 * (n & 1) + 1]));
-                                db[n] += (u.x + u.y) + (v.x + v.y);
-                            }
+                            for (int n = 0; n < NT; ++n)
+#pragma unroll
+                                for (int q = 0; q < 2; ++q) {
+                                    const float2 u = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&b[q][n / 2][2 * (n & 1)]));
+                                    const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&b[q][n / 2][2 * (n & 1) + 1]));
+                                    db[n] += (u.x + u.y) + (v.x + v.y);
+                                }
                         }
                     }
                     __syncwarp();

@@ -353,3 +353,41 @@ def test_eigenvalues_of_graded_frames(F):
     lam = fq.fq_clutter_svd(S, 1)["eigvals"]
     want = (a * a).double()
     assert float(((lam - want).abs() / want).max()) <= 4 * 2.0 ** -24
+
+
+def test_weight_gradient_sums_over_many_voxels():
+    """Weight gradients of the last two layers over 2^20 voxels against 64 bits
+    on the same BF16 operands: a running sum of n = V / (152 x 32) rounded
+    additions per CTA, so sqrt(n) 2^-24 of them and a few for the products and
+    the sum of the CTAs."""
+    n, F, Z, X = 1, 64, 128, 128
+    V = n * F * Z * X
+    g = torch.Generator(device="cuda").manual_seed(4)
+    rng = np.random.default_rng(4)
+    net = fq.CNN(4)
+    net.set_weights([(rng.standard_normal((45, a, b)) * np.sqrt(2.0 / (45 * a)), 0.05 * rng.standard_normal(b))
+                     for a, b in ((2, 32), (32, 32), (32, 32), (32, 2))])
+    x = torch.zeros((n, F, Z, X, 32), dtype=torch.bfloat16, device="cuda")
+    x[..., :2] = torch.randn((n, F, Z, X, 2), generator=g, device="cuda").bfloat16()
+    tgt = torch.randn((n, F, Z, X, 2), generator=g, device="cuda")
+    acts = fq.fq_cnn_forward(net, x)
+    y = fq.cnn_output(acts, n, F, Z, X)
+    dy3 = torch.zeros_like(x)
+    dy3[..., :2] = (2.0 * (y[..., :2] - tgt) * (1.0 / (2 * V))).bfloat16()
+    hid = [fq.cnn_hidden(acts, k, n, F, Z, X).clone() for k in (1, 2)]
+    dy2 = torch.empty_like(x)
+    fq.fq_cnn_conv(fq.CNN_MODE_MASK, dy3, net, 3, 1, dy2, mask=hid[1])
+    grads, _ = fq.fq_cnn_backward(net, x, tgt, acts)
+    torch.cuda.synchronize()
+    assert int(net.status.item()) == 0
+    for layer, a, d in ((3, hid[1], dy3), (2, hid[0], dy2)):
+        o = fq.lib().fq_cnn_param_offset(0, layer) // 4
+        gw = grads[o:o + 45 * 1024].view(45, 32, 32).double()
+        pad = torch.nn.functional.pad(a[0].double(), (0, 0, 1, 1, 1, 1, 2, 2))
+        num = den = 0.0
+        for t in (0, 13, 22, 44):
+            dt, dz, dx = t // 9, t // 3 % 3, t % 3
+            want = pad[dt:dt + F, dz:dz + Z, dx:dx + X].reshape(-1, 32).T @ d[0].double().reshape(-1, 32)
+            num += float(((gw[t] - want) ** 2).sum())
+            den += float((want ** 2).sum())
+        assert (num / den) ** 0.5 <= ((V / (152 * 32)) ** 0.5 + 4) * 2.0 ** -24, layer
