@@ -7,7 +7,9 @@
 // the k largest components is S_f = S - (S V_k) V_k^H and the power Doppler
 // is the mean of |S_f|^2 over frames.  With k << F this is O(P F k) and
 // bound by the single read of S.
+#include <algorithm>
 #include <cfloat>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -60,14 +62,14 @@ __host__ __device__ inline bool eig_in_smem(int F) { return (size_t)F * (F + 1) 
 // Operand bytes of the tensor-core Gram modes (0 = CUDA-core FP32 Gram).
 int tc_esz(int gram_mode) { return gram_mode == FQ_GRAM_BF16 ? 2 : (gram_mode == FQ_GRAM_TF32 ? 4 : 0); }
 
-ClutterLayout layout(int64_t P, int F, int gram_mode = FQ_GRAM_F32, bool force_big = false)
+ClutterLayout layout(int64_t P, int F, int gram_mode = FQ_GRAM_F32, bool force_big = false, int max_chunks = INT_MAX)
 {
     ClutterLayout L;
     size_t o = 0;
     const int esz = tc_esz(gram_mode);
     L.status = o; o += 256;
     L.G = o; o += al256(sizeof(float2) * F * F);
-    L.n_chunks = gram_chunks(P, F);
+    L.n_chunks = std::min(gram_chunks(P, F), max_chunks);
     int64_t per = (P + L.n_chunks - 1) / L.n_chunks;
     L.chunk_len = (per + kGramRound - 1) / kGramRound * kGramRound;
     L.part = o; o += esz ? 0 : al256(sizeof(float2) * (size_t)L.n_chunks * F * F);
@@ -1591,34 +1593,25 @@ fq_status launch_eig(const float2 *G, int F, float2 *big, float2 *hv, float *tau
 // device address that cudaGetSymbolAddress returns for the current device.
 constexpr size_t kNoallocBytes = (size_t)12 << 20;
 constexpr int kNoallocMaxF = 256;
-constexpr int kNoallocMaxChunks = 16;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 
-// The workspace layout of the clutter filter with at most max_chunks Gram
-// partial sums (fewer pixel chunks, each longer), so that its size depends
-// on F only.
-ClutterLayout layout_capped(int64_t P, int F, int max_chunks)
+// The workspace layout of the clutter filter with the Gram partial sums (pixel
+// chunks) that the array holds: at most 151 of the 228 that a workspace has at
+// 100 frames, 34 of 91 at 200, 18 of 50 at 256; of those the count whose CTAs
+// load the SMs most evenly (18 chunks of 9 parts at 256 frames would leave most SMs
+// one CTA and a few two: 16).  2^21 x 100: 4.13 ms (16 chunks at any F: 18.5;
+// with a workspace 3.86); 65536 x 200: 1.66 (1.95).
+ClutterLayout layout_noalloc(int64_t P, int F)
 {
-    ClutterLayout L = layout(P, F);
-    if (L.n_chunks <= max_chunks) return L;
-    size_t o = 0;
-    L.status = o; o += 256;
-    L.G = o; o += al256(sizeof(float2) * F * F);
-    L.n_chunks = max_chunks;
-    int64_t per = (P + L.n_chunks - 1) / L.n_chunks;
-    L.chunk_len = (per + kGramRound - 1) / kGramRound * kGramRound;
-    L.part = o; o += al256(sizeof(float2) * (size_t)L.n_chunks * F * F);
-    L.V = o; o += al256(sizeof(float2) * F * F);
-    L.Vt = o; o += al256(sizeof(float2) * F * F);
-    L.lam = o; o += al256(sizeof(double) * F);
-    L.k = o; o += 256;
-    L.hv = o; o += al256(sizeof(float2) * F * F);
-    L.tau = o; o += al256(sizeof(float) * F);
-    L.big = o; o += eig_in_smem(F) ? 0 : al256(sizeof(float2) * (size_t)F * (F + 1) / 2);
-    L.ii = o; o += al256(sizeof(float) * 6 * (size_t)kFastMaxK * F);
-    L.tc = o;
-    L.total = o;
-    return L;
+    const ClutterLayout one = layout(P, F, FQ_GRAM_F32, false, 1);
+    if (one.total > kNoallocBytes) return one;  // (the caller refuses it)
+    const int most = 1 + (int)std::min<size_t>((kNoallocBytes - one.total) / (sizeof(float2) * F * F), 1 << 20);
+    const int cap = std::min(most, gram_chunks(P, F)), parts = gram_parts(F);
+    auto cost = [&](int n) { return (double)((n * parts + 151) / 152) / n; };  // CTAs of an SM x pixels of each
+    int best = cap;
+    for (int n = cap; n >= 1; --n)
+        if (cost(n) < 0.97 * cost(best)) best = n;
+    return layout(P, F, FQ_GRAM_F32, false, best);
 }
 
 // Unique ID of the calling thread's current CUDA context (0 if none), from
@@ -1850,7 +1843,7 @@ fq_status fq_clutter_svd_noalloc(const void *iq, int32_t dtype, int64_t P, int32
                "fq_clutter_svd_noalloc: energy_thresh must be in (0, 1] when k_cut < 0");
     FQ_REQUIRE(dtype == FQ_F32 || dtype == FQ_BF16, FQ_ERR_UNSUPPORTED, "fq_clutter_svd_noalloc: dtype");
     FQ_REQUIRE(fqi::aligned(iq, 8) && fqi::aligned(iq_f, 8), FQ_ERR_ALIGN, "fq_clutter_svd_noalloc: alignment");
-    ClutterLayout L = layout_capped(P, F, kNoallocMaxChunks);
+    ClutterLayout L = layout_noalloc(P, F);
     FQ_REQUIRE(L.total <= kNoallocBytes, FQ_ERR_SHAPE,
                "fq_clutter_svd_noalloc: needs %zu scratch bytes, the built-in array has %zu", L.total, kNoallocBytes);
     char *ws = nullptr;
