@@ -28,8 +28,9 @@ struct ClutterLayout {
     int64_t chunk_len;
 };
 
+constexpr int kMaxF = 512;      // frames
 constexpr int kGramThreads = 256;
-constexpr int kGramPx = 16;     // pixels per shared-memory panel of the Gram kernel
+constexpr int kGramWideF = 272; // the most frames with panels of 16 pixels, beyond it 8
 constexpr int kGramCtas = 3;    // CTAs of the Gram kernel per SM
 constexpr int kGramRound = 32;  // pixel chunks are multiples of this
 
@@ -37,11 +38,15 @@ constexpr int kGramRound = 32;  // pixel chunks are multiples of this
 __host__ __device__ inline int gram_cols(int F) { return (F + 3) / 4; }
 __host__ __device__ inline int gram_blocks(int F) { return gram_cols(F) * (gram_cols(F) + 1) / 2; }
 __host__ __device__ inline int gram_parts(int F) { return (gram_blocks(F) + kGramThreads - 1) / kGramThreads; }
-size_t gram_smem(int F) { return 2 * (size_t)kGramPx * 2 * gram_cols(F) * sizeof(float4); }
+__host__ __device__ inline int gram_px(int F) { return F <= kGramWideF ? 16 : 8; }  // pixels per shared-memory panel
+// 16-byte units from plane to plane of a panel: half of the banks on, so that the
+// copies of a row, which alternate between the planes, meet no other's bank
+__host__ __device__ inline int gram_plane(int F) { return (gram_cols(F) + 3) / 8 * 8 + 4; }
+size_t gram_smem(int F) { return 2 * (size_t)gram_px(F) * 2 * gram_plane(F) * sizeof(float4); }
+size_t gram_smem_upto(int F) { return std::max(gram_smem(F), gram_smem(std::min(F, kGramWideF))); }
 // Dynamic shared memory the kernels are opted in to: the most of any call, not
 // the call's own, which another thread's smaller call could take back between
 // this thread's opt-in and its launch.
-constexpr int kMaxF = 512;
 constexpr size_t kEigSmemMax = 190 * 1024;
 constexpr int kFastMaxK = 48;  // top-k eigenvectors by inverse iteration up to this k
 
@@ -110,42 +115,173 @@ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y
 // 51% busy, the rest issue: four loads, the panels' copies and barriers).  A panel row is two planes, columns
 // (4b, 4b + 1) and (4b + 2, 4b + 3), so that the 16-byte loads of 32
 // consecutive blocks are contiguous.
-__device__ __forceinline__ void gram_stage(const float *__restrict__ S, int64_t p0, int64_t pend, int F, int nb, float4 *buf)
-{
-    const int n = (int)min((int64_t)kGramPx, pend - p0);
-    if ((F & 1) == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0) {  // rows of whole 16-byte units
-        const int U = F >> 1;
-        const float *src = S + p0 * F * 2;
-        // (pixel, unit) of this thread's next copy by steps of 256 units
-        const int dp = kGramThreads / U, du = kGramThreads - dp * U;
-        int px = threadIdx.x / U, u = threadIdx.x - px * U;
-        for (int i = threadIdx.x; i < n * U; i += kGramThreads) {
-            fqi::cp_async<16>(buf + px * 2 * nb + (u & 1) * nb + (u >> 1), src + (size_t)i * 4);
-            px += dp;
-            u += du;
-            if (u >= U) {
-                u -= U;
-                ++px;
+//
+// Panels of more than 272 frames hold 8 pixels, so that three CTAs fit as well
+// (16 pixels: two, and one from 448 frames on).  There a copy comes with every 64
+// FMAs, and its instructions count: a row of the next panel is copied with each
+// pixel's sums, one unit a thread from a running address.  65536 x 512: 3.57 ->
+// 2.48 ms, x 300: 0.79 -> 0.75 (the same in narrower panels, where few threads
+// have a unit of a row, 2^21 x 100: 2.8 -> 3.1).
+// BF16 input has to be widened: a thread holds its part of the next panel (at
+// most 18 values) in registers while it computes, and writes it out after;
+// waiting for the loads first left the SMs idle: 65536 x 220 0.49 -> 0.37 ms, x
+// 512 13.6 -> 2.18.
+constexpr int kGramHold = 18;
+static_assert(16 * kGramWideF <= kGramThreads * kGramHold && 8 * kMaxF <= kGramThreads * kGramHold, "panel values per thread");
+static_assert(kMaxF <= 2 * kGramThreads, "two columns of a row per thread");
+
+template <int PX, typename T>
+struct GramStage;
+
+// The walk of a thread over the units (two columns, one 16-byte store) of a
+// panel by steps of 256, by shared-memory address.
+struct GramWalk {
+    int U, du, u;
+    unsigned row, drow, rowb, plane;  // shared-memory byte addresses
+    __device__ __forceinline__ GramWalk(int units, int ps, const float4 *buf) : U(units)
+    {
+        const int dp = kGramThreads / U, px = threadIdx.x / U;
+        du = kGramThreads - dp * U;
+        u = threadIdx.x - px * U;
+        rowb = 32u * ps;
+        plane = 16u * ps - 8u;
+        drow = dp * rowb;
+        row = (unsigned)__cvta_generic_to_shared(buf) + px * rowb;
+    }
+    __device__ __forceinline__ unsigned at() const { return row + 8u * u + (u & 1) * plane; }
+    __device__ __forceinline__ void next()
+    {
+        row += drow;
+        u += du;
+        if (u >= U) {
+            u -= U;
+            row += rowb;
+        }
+    }
+};
+
+template <int PX>
+struct GramStage<PX, float> {
+    // wide panels: a row of the next with each pixel's sums; else all copies at once
+    static constexpr bool kRows = PX == 8;
+    const float *S;
+    int F, ps;  // frames, plane stride
+    bool wide;  // rows of whole 16-byte units
+    const float *src;
+    unsigned dst;
+    __device__ __forceinline__ GramStage(const float *s, int f, int p) : S(s), F(f), ps(p)
+    {
+        wide = (F & 1) == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0;
+    }
+    // start the copy of pixels p0 .. p0 + n - 1 into buf (kRows: by the calls of row() that follow)
+    __device__ __forceinline__ void fetch(int64_t p0, int n, float4 *buf)
+    {
+        const int t = threadIdx.x;
+        src = S + (p0 * F + (wide ? 2 * t : t)) * 2;
+        const unsigned b = (unsigned)__cvta_generic_to_shared(buf);
+        if constexpr (kRows) {
+            dst = b + (wide ? 16u * ((t & 1) * ps + (t >> 1)) : 16u * (((t >> 1) & 1) * ps + (t >> 2)) + 8u * (t & 1));
+        } else if (wide) {
+            // (pixel, unit) of this thread's next copy by steps of 256 units
+            const int U = F >> 1, dp = kGramThreads / U, du = kGramThreads - dp * U;
+            int px = t / U, u = t - px * U;
+            for (int i = t; i < n * U; i += kGramThreads) {
+                fqi::cp_async<16>(buf + px * 2 * ps + (u & 1) * ps + (u >> 1), S + p0 * F * 2 + (size_t)i * 4);
+                px += dp;
+                u += du;
+                if (u >= U) {
+                    u -= U;
+                    ++px;
+                }
+            }
+        } else {
+            for (int i = t; i < n * F; i += kGramThreads, src += 2 * kGramThreads) {
+                const int px = i / F, c = i - px * F;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                                 b + 16u * (px * 2 * ps + ((c >> 1) & 1) * ps + (c >> 2)) + 8u * (c & 1)),
+                             "l"(src)
+                             : "memory");
             }
         }
-    } else {
-        const float *src = S + p0 * F * 2;
-        for (int i = threadIdx.x; i < n * F; i += kGramThreads) {
-            const int px = i / F, c = i - px * F;
-            float2 *d = reinterpret_cast<float2 *>(buf + px * 2 * nb + ((c >> 1) & 1) * nb + (c >> 2)) + (c & 1);
-            fqi::cp_async<8>(d, src + (size_t)i * 2);
+    }
+    __device__ __forceinline__ void row()  // at most 256 units (F <= 512)
+    {
+        if constexpr (kRows) {
+            if (wide) {
+                if (2 * (int)threadIdx.x < F) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if ((int)threadIdx.x + h * kGramThreads < F)
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + h * 4u * kGramThreads),
+                                     "l"(src + h * 2 * kGramThreads)
+                                     : "memory");
+            }
+            src += 2 * F;
+            dst += 32u * ps;
         }
     }
-}
-__device__ __forceinline__ void gram_stage(const __nv_bfloat16 *__restrict__ S, int64_t p0, int64_t pend, int F, int nb, float4 *buf)
-{
-    const int n = (int)min((int64_t)kGramPx, pend - p0);
-    for (int i = threadIdx.x; i < n * F; i += kGramThreads) {
-        const int px = i / F, c = i - px * F;
-        float2 *d = reinterpret_cast<float2 *>(buf + px * 2 * nb + ((c >> 1) & 1) * nb + (c >> 2)) + (c & 1);
-        *d = fqi::load_c(S, p0 * F + i);
+    __device__ __forceinline__ void put(int, float4 *) const {}
+};
+
+template <int PX>
+struct GramStage<PX, __nv_bfloat16> {
+    static constexpr bool kRows = false;
+    const __nv_bfloat16 *S;
+    int F, ps;
+    uint32_t hold[kGramHold];
+    __device__ __forceinline__ GramStage(const __nv_bfloat16 *s, int f, int p) : S(s), F(f), ps(p) {}
+    __device__ __forceinline__ void row() const {}
+    __device__ __forceinline__ void fetch(int64_t p0, int n, float4 *)
+    {
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(S + p0 * F * 2);
+        if ((F & 1) == 0) {  // two columns at once (S is 8-byte aligned)
+            const uint2 *s2 = reinterpret_cast<const uint2 *>(src) + threadIdx.x;
+#pragma unroll
+            for (int q = 0; q < kGramHold / 2; ++q)
+                if ((int)threadIdx.x + q * kGramThreads < n * (F >> 1)) {
+                    const uint2 v = s2[q * kGramThreads];
+                    hold[2 * q] = v.x;
+                    hold[2 * q + 1] = v.y;
+                }
+        } else {
+#pragma unroll
+            for (int q = 0; q < kGramHold; ++q)
+                if ((int)threadIdx.x + q * kGramThreads < n * F) hold[q] = src[threadIdx.x + q * kGramThreads];
+        }
     }
-}
+    // the values that fetch has loaded, into buf
+    __device__ __forceinline__ void put(int n, float4 *buf) const
+    {
+        if ((F & 1) == 0) {
+            GramWalk w(F >> 1, ps, buf);
+#pragma unroll
+            for (int q = 0; q < kGramHold / 2; ++q) {
+                if ((int)threadIdx.x + q * kGramThreads >= n * w.U) break;
+                const uint32_t a = hold[2 * q], b = hold[2 * q + 1];
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(w.at()), "r"(a << 16), "r"(a & 0xffff0000u),
+                             "r"(b << 16), "r"(b & 0xffff0000u)
+                             : "memory");
+                w.next();
+            }
+        } else {
+            const int dp = kGramThreads / F, dc = kGramThreads - dp * F;
+            int px = threadIdx.x / F, c = threadIdx.x - px * F;
+#pragma unroll
+            for (int q = 0; q < kGramHold; ++q) {
+                if ((int)threadIdx.x + q * kGramThreads >= n * F) break;
+                float2 *d = reinterpret_cast<float2 *>(buf + px * 2 * ps + ((c >> 1) & 1) * ps + (c >> 2)) + (c & 1);
+                *d = make_float2(__uint_as_float(hold[q] << 16), __uint_as_float(hold[q] & 0xffff0000u));
+                px += dp;
+                c += dc;
+                if (c >= F) {
+                    c -= F;
+                    ++px;
+                }
+            }
+        }
+    }
+};
 
 __device__ __forceinline__ void cmac(float2 &s, float ax, float ay, float bx, float by)  // s += conj(a) b
 {
@@ -155,7 +291,7 @@ __device__ __forceinline__ void cmac(float2 &s, float ax, float ay, float bx, fl
     s.y = fmaf(-ay, bx, s.y);
 }
 
-template <typename T>
+template <int PX, typename T>
 __device__ __forceinline__ void gram_part(const T *__restrict__ S, int64_t P, int F, int64_t chunk_len,
                                           float2 *__restrict__ part, int which, int c, float4 *panel)
 {
@@ -171,42 +307,69 @@ __device__ __forceinline__ void gram_part(const T *__restrict__ S, int64_t P, in
         while (t >= nb - bi) { t -= nb - bi; ++bi; }
         bj = bi + t;
     }
-    const int psz = kGramPx * 2 * nb;  // units of a panel
+    const int ps = gram_plane(F), psz = PX * 2 * ps;  // units of a plane and of a panel
     __syncthreads();  // the previous item of a persistent CTA still reads the panels
     // columns past F stay zero (every panel writes the same places)
     if (F & 3)
-        for (int i = threadIdx.x; i < 2 * kGramPx; i += kGramThreads)
-            panel[i * 2 * nb + nb - 1] = panel[i * 2 * nb + 2 * nb - 1] = make_float4(0, 0, 0, 0);
+        for (int i = threadIdx.x; i < 2 * PX; i += kGramThreads)
+            panel[i * 2 * ps + nb - 1] = panel[i * 2 * ps + ps + nb - 1] = make_float4(0, 0, 0, 0);
     __syncthreads();
     float2 acc[4][4];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[r][q] = make_float2(0, 0);
-    if (pbeg < pend) gram_stage(S, pbeg, pend, F, nb, panel);
+    GramStage<PX, T> stage(S, F, ps);
+    constexpr bool kRows = GramStage<PX, T>::kRows;
+    int n = (int)max((int64_t)0, min((int64_t)PX, pend - pbeg));  // pixels of this panel, then of the next
+    if (n > 0) {
+        stage.fetch(pbeg, n, panel);
+        for (int px = 0; px < n; ++px) stage.row();
+        stage.put(n, panel);
+    }
     fqi::cp_async_commit();
     int cur = 0;
-    for (int64_t p0 = pbeg; p0 < pend; p0 += kGramPx) {
-        if (p0 + kGramPx < pend) gram_stage(S, p0 + kGramPx, pend, F, nb, panel + (cur ^ 1) * psz);
-        fqi::cp_async_commit();
-        fqi::cp_async_wait<1>();
+    for (int64_t p0 = pbeg; p0 < pend; p0 += PX) {
+        const int next = (int)max((int64_t)0, min((int64_t)PX, pend - p0 - PX));
+        if (!kRows) {
+            if (next > 0) stage.fetch(p0 + PX, next, panel + (cur ^ 1) * psz);
+            fqi::cp_async_commit();
+        }
+        fqi::cp_async_wait<kRows ? 0 : 1>();
         __syncthreads();
-        if (on) {
-            const int n = (int)min((int64_t)kGramPx, pend - p0);
-            const float4 *row = panel + cur * psz;
+        if (kRows && next > 0) stage.fetch(p0 + PX, next, panel + (cur ^ 1) * psz);
+        const float4 *row = panel + cur * psz;
+        auto sums = [&](const float4 *row) {
+            const float4 a0 = row[bi], a1 = row[ps + bi], b0 = row[bj], b1 = row[ps + bj];
+            const float ax[4] = {a0.x, a0.z, a1.x, a1.z}, ay[4] = {a0.y, a0.w, a1.y, a1.w};
+            const float bx[4] = {b0.x, b0.z, b1.x, b1.z}, by[4] = {b0.y, b0.w, b1.y, b1.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) cmac(acc[r][q], ax[r], ay[r], bx[q], by[q]);
+        };
+        if constexpr (PX == 16 && sizeof(T) == 4) {
+            if (on) {
 #pragma unroll 2
-            for (int px = 0; px < n; ++px, row += 2 * nb) {
-                const float4 a0 = row[bi], a1 = row[nb + bi], b0 = row[bj], b1 = row[nb + bj];
-                const float ax[4] = {a0.x, a0.z, a1.x, a1.z}, ay[4] = {a0.y, a0.w, a1.y, a1.w};
-                const float bx[4] = {b0.x, b0.z, b1.x, b1.z}, by[4] = {b0.y, b0.w, b1.y, b1.w};
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) cmac(acc[r][q], ax[r], ay[r], bx[q], by[q]);
+                for (int px = 0; px < n; ++px, row += 2 * ps) sums(row);
+            }
+        } else {
+            // (the same loop for every panel: 8% faster here, 10% slower above)
+#pragma unroll 2
+            for (int px = 0; px < PX; ++px, row += 2 * ps) {
+                if (kRows) {  // two rows of the next panel with each of the first pixels
+                    if (2 * px < next) stage.row();
+                    if (2 * px + 1 < next) stage.row();
+                }
+                if (on && px < n) sums(row);
             }
         }
+        // (the other panel was last read before the barrier at the end of the last round)
+        if (next > 0) stage.put(next, panel + (cur ^ 1) * psz);
+        if (kRows) fqi::cp_async_commit();
         __syncthreads();
         cur ^= 1;
+        n = next;
     }
     fqi::cp_async_wait<0>();
     if (on) {
@@ -221,12 +384,12 @@ __device__ __forceinline__ void gram_part(const T *__restrict__ S, int64_t P, in
     }
 }
 
-template <typename T>
+template <int PX, typename T>
 __global__ void __launch_bounds__(kGramThreads, kGramCtas) gram_partial_kernel(const T *__restrict__ S, int64_t P, int F,
                                                                        int64_t chunk_len, float2 *__restrict__ part)
 {
     extern __shared__ float4 panel[];
-    gram_part<T>(S, P, F, chunk_len, part, blockIdx.x, blockIdx.y, panel);
+    gram_part<PX, T>(S, P, F, chunk_len, part, blockIdx.x, blockIdx.y, panel);
 }
 
 // 32 entries of G from the partial sums: eight threads per entry take every
@@ -1479,7 +1642,9 @@ __global__ void __launch_bounds__(kGramThreads, kGramCtas) gram_batched_kernel(c
     fqb::Item it;
     while (fqb::next_item(q, ens, fqb::ST_GRAM, s_buf, it)) {
         const fqb::EnsDev &e = ens[it.e];
-        gram_part<T>((const T *)e.iq, e.P, e.F, e.chunk_len, (float2 *)(e.cws + e.cl_part), it.x, it.y, panel);
+        float2 *part = (float2 *)(e.cws + e.cl_part);
+        if (gram_px(e.F) == 16) gram_part<16, T>((const T *)e.iq, e.P, e.F, e.chunk_len, part, it.x, it.y, panel);
+        else gram_part<8, T>((const T *)e.iq, e.P, e.F, e.chunk_len, part, it.x, it.y, panel);
     }
 }
 
@@ -1549,11 +1714,12 @@ fq_status launch_gram(const void *S, int64_t P, int F, const ClutterLayout &L, c
 {
     float2 *part = (float2 *)(ws + L.part);
     const size_t smem = gram_smem(F);
-    fq_status s = fqi::cuda_check(cudaFuncSetAttribute(gram_partial_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)gram_smem(kMaxF)), "fq_casorati_gram: smem attribute");
+    auto kern = gram_px(F) == 16 ? gram_partial_kernel<16, T> : gram_partial_kernel<8, T>;
+    fq_status s = fqi::cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)gram_smem_upto(kMaxF)), "fq_casorati_gram: smem attribute");
     if (s) return s;
     dim3 grid(gram_parts(F), L.n_chunks);
-    gram_partial_kernel<T><<<grid, kGramThreads, smem, st>>>((const T *)S, P, F, L.chunk_len, part);
+    kern<<<grid, kGramThreads, smem, st>>>((const T *)S, P, F, L.chunk_len, part);
     gram_reduce_kernel<<<(F * F + kReduceItem - 1) / kReduceItem, kGramThreads, 0, st>>>(part, L.n_chunks, F, G);
     return fqi::launch_check("fq_casorati_gram");
 }
@@ -1884,10 +2050,10 @@ void clutter_layout_batched(int64_t P, int F, size_t off[10], int *n_chunks, int
 template <typename T>
 fq_status launch_gram_batched(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int F_max, cudaStream_t st)
 {
-    const size_t smem = gram_smem(F_max);
+    const size_t smem = gram_smem_upto(F_max);
     auto kern = gram_batched_kernel<T>;
     fq_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)gram_smem(kMaxF)), "batched Gram: smem attribute");
+                                                  (int)gram_smem_upto(kMaxF)), "batched Gram: smem attribute");
     if (s) return s;
     kern<<<fqb::persistent_grid(kern, kGramThreads, smem, items), kGramThreads, smem, st>>>(ens, q);
     return launch_check("batched Gram");

@@ -391,3 +391,20 @@ def test_weight_gradient_sums_over_many_voxels():
             num += float(((gw[t] - want) ** 2).sum())
             den += float((want ** 2).sum())
         assert (num / den) ** 0.5 <= ((V / (152 * 32)) ** 0.5 + 4) * 2.0 ** -24, layer
+
+
+# panels of 16 and 8 pixels at their limit (272 frames) and the most frames, even
+# and odd counts, whole panels and remainders, rows of whole and of half 16-byte
+# units; the bar of test_gram_panels
+@pytest.mark.parametrize("F", [271, 272, 273, 300, 385, 511, 512])
+@pytest.mark.parametrize("P", [1, 7, 8, 33, 1001])
+@pytest.mark.parametrize("dt,shift", [("f32", 0), ("f32", 2), ("bf16", 0), ("bf16", 4)])
+def test_gram_wide_panels(F, P, dt, shift):
+    g = torch.Generator(device="cuda").manual_seed(F * 1000 + P)
+    buf = torch.randn(2 * P * F + shift, generator=g, device="cuda").to(torch.float32 if dt == "f32" else torch.bfloat16)
+    S = buf[shift:].view(P, F, 2)
+    G = torch.view_as_complex(fq.fq_casorati_gram(S).double().contiguous())
+    s = torch.view_as_complex(S.double().contiguous())
+    mag = (S.double().abs().sum(2)).mT @ S.double().abs().sum(2)
+    err = (G - s.mH @ s).abs()
+    assert bool((err <= 2.0 ** -24 * (2 * P + 16) * mag).all())
