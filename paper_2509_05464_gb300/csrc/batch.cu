@@ -292,7 +292,11 @@ fq_status launch_stage(fq_batch *b, char *arena, int w, int s, cudaStream_t st)
     case fqb::ST_GRAM: return fqi::batched_gram(ens, q, q.total, b->iq_dtype, b->F_max, st);
     case fqb::ST_GRAM_REDUCE: return fqi::batched_gram_reduce(ens, q, q.total, st);
     case fqb::ST_EIG:
-        return fqi::batched_eig(ens, reinterpret_cast<const int *>(arena + wv.members_off), q.n, b->F_max, st);
+    {
+        std::vector<int> F;  // of the members, largest first
+        for (int i : wv.order[fqb::ST_EIG]) F.push_back(b->e[i].F);
+        return fqi::batched_eig(ens, reinterpret_cast<const int *>(arena + wv.members_off), F.data(), q.n, st);
+    }
     case fqb::ST_PROJECT: return fqi::batched_project(ens, q, q.total, b->iq_dtype, st);
     default: return fqi::set_error(FQ_ERR_INVALID_ARG, "batch: stage %d", s);
     }

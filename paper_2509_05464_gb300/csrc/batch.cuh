@@ -159,7 +159,8 @@ fq_status batched_das(const fqb::EnsDev *ens, const fqb::StageQueue &q, int item
 fq_status batched_gram(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int iq_dtype, int F_max, cudaStream_t st);
 void gram_item_counts(int F, int *parts, int *reduce_items);  // CTAs per pixel chunk; reduction items
 fq_status batched_gram_reduce(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, cudaStream_t st);
-fq_status batched_eig(const fqb::EnsDev *ens, const int *members, int n, int F_max, cudaStream_t st);
+// members and their frame counts F (host), largest first
+fq_status batched_eig(const fqb::EnsDev *ens, const int *members, const int *F, int n, cudaStream_t st);
 fq_status batched_project(const fqb::EnsDev *ens, const fqb::StageQueue &q, int items, int iq_dtype,
                           cudaStream_t st);
 

@@ -1501,22 +1501,21 @@ __global__ void __launch_bounds__(NT) eig_kernel(const float2 *__restrict__ G, i
     eig_body(G, F, big, hv, tau_g, lam_out, V, Vt, k_cut, thresh, k_out, status, topk_only, ii_scr, NT);
 }
 
-// One CTA per ensemble of a wave.  In a wave with a matrix too large for shared
-// memory (NT = 1024) the other members leave with the threads that a single call
-// would not have, so that their sums are the same.
+// One CTA per member, each with the threads of its single call, so that its sums
+// are the same.
 template <int NT>
 __global__ void __launch_bounds__(NT) eig_batched_kernel(const fqb::EnsDev *__restrict__ ens,
                                                          const int *__restrict__ members)
 {
+    if (NT == kEigThreads) asm volatile("griddepcontrol.launch_dependents;");  // (see batched_eig)
     const fqb::EnsDev &e = ens[members[blockIdx.x]];
-    const int nt = eig_in_smem(e.F) ? kTopThreads : NT;
-    if (threadIdx.x >= nt) return;
     char *ws = e.cws;
     double *lam = e.eigvals ? e.eigvals : (double *)(ws + e.cl_lam);
     int *kk = e.k_used ? e.k_used : (int *)(ws + e.cl_k);
     eig_body((const float2 *)(ws + e.cl_G), e.F, eig_in_smem(e.F) ? nullptr : (float2 *)(ws + e.cl_big), (float2 *)(ws + e.cl_hv),
              (float *)(ws + e.cl_tau), lam, (float2 *)(ws + e.cl_V), (float2 *)(ws + e.cl_Vt), e.k_cut,
-             e.energy_thresh, kk, e.status, 1, (float *)(ws + e.cl_ii), nt);
+             e.energy_thresh, kk, e.status, 1, (float *)(ws + e.cl_ii), NT);
+    if (NT == kTopThreads) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ------------------------------------------------ projection + power Doppler --
@@ -2078,16 +2077,36 @@ fq_status batched_gram_reduce(const fqb::EnsDev *ens, const fqb::StageQueue &q, 
     return launch_check("batched Gram reduce");
 }
 
-fq_status batched_eig(const fqb::EnsDev *ens, const int *members, int n, int F_max, cudaStream_t st)
+// Matrices too large for shared memory in a launch of their own without any: they
+// live in the L1 cache as far as they fit, and shared memory for the other
+// members' matrices took it from them (6 members of 240 frames 3.8 -> 2.64 ms, of
+// 400 14.4 -> 9.4).  The other members' launch starts as soon as
+// all CTAs of the first run (programmatic launch; it reads nothing of theirs) and
+// ends after them, so that the stages that follow see both (6 members of 50 to 300
+// frames: 3.97 ms, one after the other 5.33, in one launch 5.5).
+fq_status batched_eig(const fqb::EnsDev *ens, const int *members, const int *F, int n, cudaStream_t st)
 {
-    const int nt = top_threads(F_max);
-    while (!eig_in_smem(F_max)) --F_max;  // larger members keep their matrix in the workspace
-    const size_t smem = sizeof(float2) * (size_t)F_max * (F_max + 1) / 2;
-    auto kern = nt == kTopThreads ? eig_batched_kernel<kTopThreads> : eig_batched_kernel<kEigThreads>;
-    fq_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)kEigSmemMax), "batched eig: smem attribute");
-    if (s) return s;
-    kern<<<n, nt, smem, st>>>(ens, members);
+    int big = 0;
+    while (big < n && !eig_in_smem(F[big])) ++big;
+    if (big > 0) eig_batched_kernel<kEigThreads><<<big, kEigThreads, 0, st>>>(ens, members);
+    if (big < n) {
+        auto kern = eig_batched_kernel<kTopThreads>;
+        fq_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      (int)kEigSmemMax), "batched eig: smem attribute");
+        if (s) return s;
+        cudaLaunchAttribute early;
+        early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        early.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(n - big);
+        cfg.blockDim = dim3(kTopThreads);
+        cfg.dynamicSmemBytes = sizeof(float2) * (size_t)F[big] * (F[big] + 1) / 2;
+        cfg.stream = st;
+        cfg.attrs = &early;
+        cfg.numAttrs = big > 0 ? 1 : 0;
+        s = cuda_check(cudaLaunchKernelEx(&cfg, kern, ens, members + big), "batched eig");
+        if (s) return s;
+    }
     return launch_check("batched eig");
 }
 

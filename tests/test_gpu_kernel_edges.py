@@ -408,3 +408,23 @@ def test_gram_wide_panels(F, P, dt, shift):
     mag = (S.double().abs().sum(2)).mT @ S.double().abs().sum(2)
     err = (G - s.mH @ s).abs()
     assert bool((err <= 2.0 ** -24 * (2 * P + 16) * mag).all())
+
+
+def test_graph_of_small_and_large_eigen_problems():
+    """As above by a replayed graph, with more members: the two kinds run in
+    launches that overlap, and the stages after them see both."""
+    ms = [w for i, F in enumerate((230, 60, 222, 200, 41, 256, 100, 225, 220, 221))
+          for w in W.config4(seed=120 + i, n=1, s_range=(300, 800), f_range=(F, F), grids=((16, 1, 24),))]
+    b = fq.Batch(ms)
+    b.capture()
+    for _ in range(3):
+        b.graph_launch()
+    b.status()
+    torch.cuda.synchronize()
+    for i, w in enumerate(ms):
+        pl = Pipeline(w)
+        pl.upload()
+        pl.step()
+        torch.cuda.synchronize()
+        assert torch.equal(b.eigvals[i], pl.eigvals), i
+        assert torch.equal(b.pd[i], pl.pd), i
