@@ -167,7 +167,10 @@ int32_t fq_version(void);
  *   seg_id    device int32 [S]     segment index or -1
  *   flow_coord device float [3][S] (q, xi1, xi2) rows, read for blood only
  *   pos_out   device float [n_frames][3][S]
- * Arithmetic is FP64 (wrap decisions bit-identical to IEEE double).
+ * Wrap decisions are those of IEEE double, bit for bit.  Positions are
+ * float pairs (~48 bits) rounded once to binary32; beyond 4096 wraps the
+ * path coordinate is IEEE double, with a rigid rotation (omega != 0)
+ * everything is.
  * Errors: FQ_ERR_INVALID_ARG (null pointer, S < 0, n_frames < 1, seg_id
  * outside [-1, n_seg) is not checked on the device: such scatterers are
  * treated as tissue), FQ_ERR_SHAPE (n_seg or n_terms above the maximum). */

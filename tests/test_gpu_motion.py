@@ -54,3 +54,24 @@ def test_trajectories(medium, kind, S, F, dt, sign):
         assert np.all(diff <= ulp), (f, float((diff / ulp).max()))
         same += np.mean(diff == 0) / len(frames)
     assert same > 0.999
+
+
+@pytest.mark.parametrize("medium", ["tree", "arcs"])
+@pytest.mark.parametrize("t0", [1e3, 1e5, 1e6, 1e7])
+def test_trajectories_after_many_wraps(medium, t0):
+    """10^4 to 10^8 wraps: the path coordinate of IEEE double, the bars above."""
+    F, dt = 5, 1e-3
+    w = W.config3(seed=6, n_scat=20_000, n_frames=F) if medium == "tree" else W.config2(seed=6, n_scat=20_000, n_frames=F)
+    m = motion("rigid")
+    d = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (w.p0, w.seg, w.flow)]
+    pos = fq.fq_advect_scatterers(*d, w.segments, m, t0, dt, F).cpu().numpy()
+    st, mt = W.segment_table(w), W.motion_table(m)
+    blood = w.seg >= 0
+    same = 0
+    for f in range(F):
+        want = oracle.advect(w.p0, w.seg, w.flow, st, mt, t0 + f * dt)
+        ulp = np.spacing(np.abs(want).astype(np.float32))
+        diff = np.abs(pos[f].astype(np.float64) - want.astype(np.float64))
+        assert np.all(diff <= ulp), (f, float((diff / ulp).max()))
+        same += np.mean(diff[:, blood] == 0) / F
+    assert same > 0.999
