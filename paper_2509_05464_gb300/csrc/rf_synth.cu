@@ -1384,6 +1384,7 @@ __device__ __forceinline__ void rf_quad_tile(const RfParams &p, int bx, int ag, 
                              k[0] = r0 + kofs;
                              k[1] = r1 + kofs;
                              pulse.taps(p, PH, [&](auto j, f2 t) {
+                                 if constexpr (FFD && decltype(j)::value == 4) t = fqi::f2_fma(fqi::f2_dup(p.dc_corr), pulse.A, t);
                                  float t0, t1;
                                  fqi::f2_split(t, t0, t1);
                                  put(0, decltype(j)::value, t0);
