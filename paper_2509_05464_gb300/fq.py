@@ -265,11 +265,12 @@ def make_grid(g) -> Grid:
 class _FlowHolder:
     def __init__(self, segments):
         n = len(segments)
-        flat = []
+        flat, whole = [], n > 0
         for s in segments:
             flat += (int(s.kind), *s.p0, *s.a1, *s.a2, *s.a3, s.length, s.radius, s.vmax, s.arc_radius, s.phi1,
                      *s.arc_end)
-        if n and len(flat) == 20 * n:
+            whole = whole and len(s.p0) == len(s.a1) == len(s.a2) == len(s.a3) == 3 and len(s.arc_end) == 2
+        if whole:
             # all segments in one pack: setting the structs' fields one by one
             # took 0.25 ms for the 63 vessels of the 3D workload's tree
             self.arr = (Segment * n).from_buffer_copy(struct.pack("=" + "i4x19d" * n, *flat))

@@ -75,3 +75,22 @@ def test_binding_fails_loudly_without_library(monkeypatch):
     monkeypatch.setattr(fq, "LIB_PATH", "/nonexistent/libfq.so")
     with pytest.raises(fq.FqError):
         fq.lib()
+
+
+def test_vessels_are_packed_field_by_field():
+    """Vessel vectors of the wrong length are not taken for one another: too
+    many values are an error, missing ones are 0, also where the counts of a
+    vessel add up."""
+    class Seg:
+        kind, length, radius, vmax, arc_radius, phi1 = 1, 2.0, 3.0, 4.0, 5.0, 6.0
+        p0, a1, a2, a3, arc_end = (1.0, 2.0, 3.0), (4.0, 5.0, 6.0), (7.0, 8.0, 9.0), (10.0, 11.0, 12.0), (13.0, 14.0)
+
+    ok, long_, short = Seg(), Seg(), Seg()
+    st = fq._FlowHolder([ok, ok]).arr[1]
+    assert (list(st.p0), list(st.a1), list(st.a3), st.phi1, list(st.arc_end)) == (
+        [1.0, 2.0, 3.0], [4.0, 5.0, 6.0], [10.0, 11.0, 12.0], 6.0, [13.0, 14.0])
+    long_.p0, long_.a1 = (1.0, 2.0, 3.0, 3.5), (4.0, 5.0)
+    with pytest.raises(IndexError):
+        fq._FlowHolder([ok, long_])
+    short.a2 = (7.0, 8.0)
+    assert list(fq._FlowHolder([short, ok]).arr[0].a2) == [7.0, 8.0, 0.0]
