@@ -1175,8 +1175,15 @@ fq_status fq_cnn_backward(const void *params, const void *vol, const float *targ
     for (int l = 3; l >= 0; --l) {
         // weight and bias gradients of layer l from its input and output gradient
         float *part = (float *)(ab + A.part);
-        if (l == 3) s = launch_wgrad<1>(act_in[l], dy[cur], d, A.wg_parts, part, grads + L.w[l], grads + L.b[l], status, st);
-        else s = launch_wgrad<4>(act_in[l], dy[cur], d, A.wg_parts, part, grads + L.w[l], grads + L.b[l], status, st);
+        const __nv_bfloat16 *x = act_in[l];
+        if (!fqi::aligned(x, 16)) {  // the caller's volume, whose copy can use the other gradient buffer now
+            s = fqi::cuda_check(cudaMemcpyAsync(dy[cur ^ 1], x, (size_t)V * C * 2, cudaMemcpyDeviceToDevice, st),
+                                "fq_cnn_backward: volume");
+            if (s) return s;
+            x = dy[cur ^ 1];
+        }
+        if (l == 3) s = launch_wgrad<1>(x, dy[cur], d, A.wg_parts, part, grads + L.w[l], grads + L.b[l], status, st);
+        else s = launch_wgrad<4>(x, dy[cur], d, A.wg_parts, part, grads + L.w[l], grads + L.b[l], status, st);
         if (s) return s;
         if (l == 0) break;
         // data gradient through layer l, masked by the ReLU of layer l - 1

@@ -447,3 +447,19 @@ def test_rf_echoes_near_the_record_end(dt):
         out.append(fq.fq_simulate_rf(p, [0.0], [0.0], torch.from_numpy(pos[None]).cuda(), amp, 1, out_dtype=t)[..., :300])
     assert float(out[0].float().abs().max()) > 0
     assert torch.equal(out[0], out[1])
+
+
+def test_weight_gradients_of_an_unaligned_volume():
+    """The backward pass takes a volume at any element's address."""
+    n, F, Z, X = 2, 5, 8, 32
+    g = torch.Generator(device="cuda").manual_seed(9)
+    net = fq.CNN(9, zero_last=False)
+    buf = torch.zeros(n * F * Z * X * 32 + 1, dtype=torch.bfloat16, device="cuda")
+    x = buf[1:].view(n, F, Z, X, 32)
+    x[..., :2] = torch.randn((n, F, Z, X, 2), generator=g, device="cuda").bfloat16()
+    tgt = torch.randn((n, F, Z, X, 2), generator=g, device="cuda")
+    aligned = x.clone()
+    acts = fq.fq_cnn_forward(net, aligned)
+    want, loss = fq.fq_cnn_backward(net, aligned, tgt, acts)
+    got, loss2 = fq.fq_cnn_backward(net, x, tgt, acts)
+    assert torch.equal(got, want) and torch.equal(loss, loss2)
