@@ -296,12 +296,11 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                                     WIDE ? r.x0 - 1 : r.x0 - 1 + k, r.z0 - 1, g, r.n);
                 }
             }
-            if (fail) {
-                s_fail = 1;
-                for (uint32_t k = i > RING_SLOTS ? i - RING_SLOTS : 0; k < i; ++k)  // let issued copies land
-                    mbar_wait(&slot_full[k % RING_SLOTS], (k / RING_SLOTS) & 1u);
-                mbar_wait(&w_bar, 0);
-            }
+            if (fail) s_fail = 1;
+            // let issued copies land before the CTA can exit, whoever gave up
+            for (uint32_t k = i > RING_SLOTS ? i - RING_SLOTS : 0; k < i; ++k)
+                mbar_wait(&slot_full[k % RING_SLOTS], (k / RING_SLOTS) & 1u);
+            mbar_wait(&w_bar, 0);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -659,14 +658,12 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 }
                 t += fb - fa;
             }
-            if (!ok) {
-                s_fail = 1;
-                // let the copies already issued land before the CTA can exit
-                for (int k = 1; k <= kWgXSlots && jx - k >= 0; ++k)
-                    mbar_wait(&x_full[(jx - k) % kWgXSlots], (uint32_t)((jx - k) / kWgXSlots) & 1u);
-                for (int k = 1; k <= kWgDySlots && jg - k >= 0; ++k)
-                    mbar_wait(&g_full[(jg - k) % kWgDySlots], (uint32_t)((jg - k) / kWgDySlots) & 1u);
-            }
+            if (!ok) s_fail = 1;
+            // let issued copies land before the CTA can exit, whoever gave up
+            for (int k = 1; k <= kWgXSlots && jx - k >= 0; ++k)
+                mbar_wait(&x_full[(jx - k) % kWgXSlots], (uint32_t)((jx - k) / kWgXSlots) & 1u);
+            for (int k = 1; k <= kWgDySlots && jg - k >= 0; ++k)
+                mbar_wait(&g_full[(jg - k) % kWgDySlots], (uint32_t)((jg - k) / kWgDySlots) & 1u);
         }
     } else {
         const int dti = warp / 3, dzi = warp % 3;  // dt + 2, dz + 1
