@@ -21,8 +21,9 @@
 // (distance, transmit path, u) runs in float-float; the pulse itself is
 // evaluated at the small offset j - frac(u), where binary32 suffices: the
 // taps' Hann-phase cosines follow the Chebyshev recurrence
-// C_{j+1} = 2 cos(w) C_j - C_{j-1} from the first tap, and for the
-// two-cycle pulse the carrier is cos(2 theta) = 2 C^2 - 1 of the Hann phase.
+// C_{j+1} = 2 cos(w) C_j - C_{j-1} from the first tap (from the two middle
+// ones outwards in the 4-element kernel), and for the two-cycle pulse the
+// carrier is cos(2 theta) = 2 C^2 - 1 of the Hann phase.
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -40,7 +41,7 @@ constexpr int kMaxTaps = 64;  // pulse taps per (scatterer, element) pair the ke
 // up to kQuadSmemMax (below QuadShared): the more angles a CTA holds, the
 // more of the receive geometry, the scatterer loads and the bound pass it
 // shares (2D compounded workload: 5 angles per CTA 6% faster than 3; 3D
-// workload: all 9 angles, 216 KB of records at 1536 samples, 1686 ms against
+// workload: all 9 angles, 222 KB of records at 1536 samples, 1686 ms against
 // 1821 ms for groups of 5 and 4).  The CTAs that fit per SM by shared memory
 // split 32 resident warps (64 registers per thread): on the 2D workload 32
 // warps ran 9.4% faster than 16 (128 registers), 24 warps 7.8%.
@@ -62,9 +63,6 @@ struct RfParams {
     float tab_h[2][2];  // (cos, sin)(w_h * j) for j = jmin, jmin + 1
     float tab_c[2][2];  // (cos, sin)(w_c * j) for j = jmin, jmin + 1
     int two_cycle;      // n_cycles == 2: carrier = 2 C^2 - 1 of the Hann phase
-    // first-tap thresholds on frac for the fast kernels: jlo = jmin + (frac > theta),
-    // floor(frac + half_w) = floor(half_w) + (frac >= theta2)
-    float theta, theta2, jmin_f;
     float att_l2;       // -att log2(e): exp(-att path) = 2^(att_l2 path)
     // quad kernel: transmit angles per CTA (ag), angle groups (n_ag), the
     // half-width of the tap-bound window (ceil(half_w) + 1 samples) and the
@@ -1618,14 +1616,14 @@ fq_status dispatch_rf(const RfParams &p, int F, const float *pos, const float *a
     }
 }
 
-// The quad kernel's pulse taps come from a binary32 Chebyshev recurrence
-// started at the first tap; its rounded constants (the recurrence factor
-// 2 cos w, the table entries e^{i w j}) give every echo the same small error
-// pattern, whose sum over the taps (the echo's DC content) does not average
-// out: ~-2.3e-7 of the echo amplitude for the two-cycle pulse at ~4 samples
-// per carrier period.  rf2iq passes DC to baseband at -f0 with about half
-// gain, and delay-and-sum adds that component coherently over every
-// (transmit, element) term of a voxel while the echoes themselves add with
+// The quad kernel's pulse taps come from two binary32 polynomials at the middle
+// taps and a Chebyshev recurrence outwards from them; the rounded constants (the
+// recurrence factor 2 cos w, the polynomials' coefficients) give every echo the
+// same small error pattern, whose sum over the taps (the echo's DC content) does
+// not average out: -2.6e-7 of the echo amplitude for the two-cycle pulse at
+// 4.006 samples per carrier period, -2.1e-7 at 4.  rf2iq passes DC to baseband at
+// -f0 with about half gain, and delay-and-sum adds that component coherently over
+// every (transmit, element) term of a voxel while the echoes themselves add with
 // random phases, so it grew to ~1.2e-5 of the beamformed image of the 3D
 // workload.  This host routine runs the same binary32 operations lane by
 // lane (the kernel's f32x2 instructions round each lane like these scalar
@@ -1636,7 +1634,7 @@ fq_status dispatch_rf(const RfParams &p, int F, const float *pos, const float *a
 //
 // The delays are (i + 1/2) / N, so the pulse's samples over all of them are
 // the even grid (m + 1/2) / N of its support, whose sum has a closed form;
-// the recurrence runs on blocks of independent lanes, which the compiler
+// the operations run on blocks of independent lanes, which the compiler
 // vectorises (one double-precision pulse per tap took 0.45 ms of every call).
 constexpr int kBiasN = 4096, kBiasL = 16;
 
@@ -1719,9 +1717,6 @@ fq_status make_rf_params(const fq_probe *probe, const fq_tx *tx, int64_t S, int 
     p.w_c = (float)wc;
     p.w_h = (float)wh;
     p.jmin = (int)std::ceil(0.0 - hw);  // frac in [0, 1): jlo in {jmin, jmin + 1}
-    p.jmin_f = (float)p.jmin;
-    p.theta = (float)(p.jmin + hw);
-    p.theta2 = (float)(std::floor(hw) + 1.0 - hw);
     p.att_l2 = (float)(-(double)p.att / std::log(2.0));
     for (int q = 0; q < 2; ++q) {
         double j = p.jmin + q;
