@@ -1021,7 +1021,9 @@ fq_status launch_das(const DasParams &p, const void *ch, void *iq, cudaStream_t 
     if constexpr (sizeof(ChT) == 2) {
         constexpr int NW = kDasWarpThreads / 32, NT = kDasWarpThreads;
         const size_t smem = das_w_smem_bytes(p.pr.M, p.A, NW, p.rot_tab ? p.pr.ns : 0);
-        // 64 frames a pass when they hold the ensemble; 32-bit byte offsets when
+        // 64 frames a pass (four a lane) when they hold the ensemble, else 128: 64 x
+        // 16 x 32 voxels, matrix probe, BF16: 64 frames 8.2 ms, 65 frames 12.3 (two
+        // passes of 64 would be 16.4); 256 x 256, linear: 0.84, 1.37.  32-bit byte offsets when
         // an angle's lines (and the second row and frame group of the last
         // sample) stay below 4 GB
         const bool f64 = p.Fp <= 64;

@@ -111,10 +111,10 @@ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y
 // only blocks of the triangle are computed (F = 100: 5200 of 5050 products;
 // 32 x 32 tiles with 2 x 2 outputs per thread computed 10240 and read two
 // 8-byte operands per complex product).  2^21 pixels x 100 frames: 6.9 -> 2.8
-// ms; 65536 x 200: 0.60 -> 0.30 ms, with three CTAs per SM (two 3.1; FMA pipe
-// 51% busy, the rest issue: four loads, the panels' copies and barriers).  A panel row is two planes, columns
-// (4b, 4b + 1) and (4b + 2, 4b + 3), so that the 16-byte loads of 32
-// consecutive blocks are contiguous.
+// ms; 65536 x 200: 0.60 -> 0.29 ms, with three CTAs per SM (two 3.1; FMA pipe
+// 48% busy, the rest issue: four loads, the panels' copies and barriers).  A
+// panel row is two planes, columns (4b, 4b + 1) and (4b + 2, 4b + 3), so that the
+// 16-byte loads of 32 consecutive blocks are contiguous.
 //
 // Panels of more than 272 frames hold 8 pixels, so that three CTAs fit as well
 // (16 pixels: two, and one from 448 frames on).  There a copy comes with every 64

@@ -825,8 +825,8 @@ __global__ void cnn_pd_kernel(const float *__restrict__ y, int F, int Z, int X, 
 // ------------------------------------------------------------------- host --
 struct ParamLayout {   // offsets in floats inside the parameter block
     size_t w[4], b[4], m, v, n_train;  // master weights/biases, then Adam m and v over the same span
-    size_t wf_bytes_off, wb_bytes_off;   // 64-byte-row tap tiles (per-tap kernel)
-    size_t wfc_bytes_off, wbc_bytes_off; // 16-byte-chunk tap tiles (frame-ring kernel)
+    size_t wf_bytes_off, wb_bytes_off;   // 64-byte-row tap tiles (narrow tile)
+    size_t wfc_bytes_off, wbc_bytes_off; // 16-byte-chunk tap tiles (WIDE tile)
     size_t total_bytes;
 };
 
