@@ -1094,6 +1094,11 @@ __device__ __forceinline__ void tridiagonalise_rows(float2 *Ap, int F, float *d,
     }
 }
 
+// an element of the Gram matrix; L2: past the L1 cache, where an earlier launch's
+// may be left
+template <bool L2>
+__device__ __forceinline__ float2 load_gram(const float2 *p) { return L2 ? __ldcg(p) : *p; }
+
 // One step of subspace iteration with the matrix itself: V <- orth(G V) for the
 // k <= kRefineMaxK vectors, where lambda_j is well above the rounding of G.
 // It takes the rounding of the F reflectors out of the filter's subspace (a
@@ -1106,6 +1111,7 @@ __device__ __forceinline__ void tridiagonalise_rows(float2 *Ap, int F, float *d,
 // and below 1.1e-19, and the filter removed nothing).
 // Y: k F values of scratch.
 constexpr int kRefineMaxK = 8;
+template <bool L2>
 __device__ __forceinline__ void refine_vectors(const float2 *__restrict__ G, float ginv, int F, int k, const float *lam,
                                                float2 *Y, float2 *V, float2 *Vt, int lane, int wid, int nw)
 {
@@ -1116,7 +1122,7 @@ __device__ __forceinline__ void refine_vectors(const float2 *__restrict__ G, flo
 #pragma unroll
             for (int u = 0; u < 4; ++u) s[u] = make_float2(0, 0);
             for (int f = lane; f < F; f += 32) {
-                float2 g = G[(size_t)i * F + f];
+                float2 g = load_gram<L2>(G + (size_t)i * F + f);
                 g = make_float2(g.x * ginv, g.y * ginv);
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
@@ -1173,6 +1179,9 @@ __device__ __forceinline__ void refine_vectors(const float2 *__restrict__ G, flo
 // implicit QL with Wilkinson shifts on the real tridiagonal (after a
 // diagonal unitary scaling), eigenvalue sort and back-transformation.
 // Optional: the energy / fixed cutoff k.
+// L2: for a launch that may start before the one ahead of it in its stream has
+// ended (see batched_eig).
+template <bool L2>
 __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, float2 *__restrict__ big,
                                          float2 *__restrict__ hv, float *__restrict__ tau_g,
                                          double *__restrict__ lam_out, float2 *__restrict__ V,
@@ -1199,7 +1208,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
     float amax = 0.0f;
     for (int i = wid; i < F; i += nw)
         for (int j = lane; j <= i; j += 32) {
-            float2 g = G[(size_t)i * F + j];
+            float2 g = load_gram<L2>(G + (size_t)i * F + j);
             amax = fmaxf(amax, fmaxf(fabsf(g.x), fabsf(g.y)));
         }
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
@@ -1215,7 +1224,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
     const float gscale = s_scale, ginv = 1.0f / s_scale;
     for (int i = wid; i < F; i += nw)
         for (int j = lane; j <= i; j += 32) {
-            float2 g = G[(size_t)i * F + j];
+            float2 g = load_gram<L2>(G + (size_t)i * F + j);
             Ap[pidx(i, j)] = make_float2(g.x * ginv, g.y * ginv);
         }
     __syncthreads();
@@ -1357,7 +1366,7 @@ __device__ __forceinline__ void eig_body(const float2 *__restrict__ G, int F, fl
             else
                 back_transform(F, k, Z, zk, perm, delta, hv, tau_g, V, Vt, nullptr, 0, lane, wid, nw);
             if (k <= kRefineMaxK && k < F)
-                refine_vectors(G, ginv, F, k, lamd, big || 2 * k > F + 1 ? reinterpret_cast<float2 *>(ii_scr) : dyn, V, Vt, lane, wid, nw);
+                refine_vectors<L2>(G, ginv, F, k, lamd, big || 2 * k > F + 1 ? reinterpret_cast<float2 *>(ii_scr) : dyn, V, Vt, lane, wid, nw);
             return;
         }
     }
@@ -1498,7 +1507,7 @@ __global__ void __launch_bounds__(NT) eig_kernel(const float2 *__restrict__ G, i
                                                           int *__restrict__ k_out, int *__restrict__ status,
                                                           int topk_only, float *__restrict__ ii_scr)
 {
-    eig_body(G, F, big, hv, tau_g, lam_out, V, Vt, k_cut, thresh, k_out, status, topk_only, ii_scr, NT);
+    eig_body<false>(G, F, big, hv, tau_g, lam_out, V, Vt, k_cut, thresh, k_out, status, topk_only, ii_scr, NT);
 }
 
 // One CTA per member, each with the threads of its single call, so that its sums
@@ -1512,7 +1521,7 @@ __global__ void __launch_bounds__(NT) eig_batched_kernel(const fqb::EnsDev *__re
     char *ws = e.cws;
     double *lam = e.eigvals ? e.eigvals : (double *)(ws + e.cl_lam);
     int *kk = e.k_used ? e.k_used : (int *)(ws + e.cl_k);
-    eig_body((const float2 *)(ws + e.cl_G), e.F, eig_in_smem(e.F) ? nullptr : (float2 *)(ws + e.cl_big), (float2 *)(ws + e.cl_hv),
+    eig_body<NT == kTopThreads>((const float2 *)(ws + e.cl_G), e.F, eig_in_smem(e.F) ? nullptr : (float2 *)(ws + e.cl_big), (float2 *)(ws + e.cl_hv),
              (float *)(ws + e.cl_tau), lam, (float2 *)(ws + e.cl_V), (float2 *)(ws + e.cl_Vt), e.k_cut,
              e.energy_thresh, kk, e.status, 1, (float *)(ws + e.cl_ii), NT);
     if (NT == kTopThreads) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -2081,8 +2090,8 @@ fq_status batched_gram_reduce(const fqb::EnsDev *ens, const fqb::StageQueue &q, 
 // live in the L1 cache as far as they fit, and shared memory for the other
 // members' matrices took it from them (6 members of 240 frames 3.8 -> 2.64 ms, of
 // 400 14.4 -> 9.4).  The other members' launch starts as soon as
-// all CTAs of the first run (programmatic launch; it reads nothing of theirs) and
-// ends after them, so that the stages that follow see both (6 members of 50 to 300
+// all CTAs of the first run (programmatic launch; it reads nothing of theirs, and
+// the Gram matrices, which were complete before them, from L2) and ends after them, so that the stages that follow see both (6 members of 50 to 300
 // frames: 3.97 ms, one after the other 5.33, in one launch 5.5).
 fq_status batched_eig(const fqb::EnsDev *ens, const int *members, const int *F, int n, cudaStream_t st)
 {

@@ -463,3 +463,27 @@ def test_weight_gradients_of_an_unaligned_volume():
     want, loss = fq.fq_cnn_backward(net, aligned, tgt, acts)
     got, loss2 = fq.fq_cnn_backward(net, x, tgt, acts)
     assert torch.equal(got, want) and torch.equal(loss, loss2)
+
+
+def test_overlapping_eigen_launches_see_new_inputs():
+    """The launch that starts beside the large matrices' reads this launch's
+    Gram matrices, not what the caches hold of the last one's: a plan launched
+    again on other amplitudes gives what a fresh plan gives."""
+    ms = [w for i, F in enumerate((230, 60, 240, 200, 41))
+          for w in W.config4(seed=140 + i, n=1, s_range=(300, 800), f_range=(F, F), grids=((16, 1, 24),))]
+    b = fq.Batch(ms)
+    b.capture()
+    amps = [w.amp.copy() for w in ms]
+    rng = np.random.default_rng(2)
+    for _ in range(3):
+        for w, a, d in zip(ms, amps, b.inputs):
+            w.amp = (a * rng.uniform(0.5, 2.0, a.shape)).astype(np.float32)
+            d[3].copy_(torch.from_numpy(w.amp))
+        b.graph_launch()
+        b.status()
+        c = fq.Batch(ms)
+        c.launch()
+        c.status()
+        torch.cuda.synchronize()
+        for i in range(len(ms)):
+            assert torch.equal(b.eigvals[i], c.eigvals[i]) and torch.equal(b.pd[i], c.pd[i]), i
