@@ -364,7 +364,7 @@ __device__ __forceinline__ void gram_part(const T *__restrict__ S, int64_t P, in
                 if (on && px < n) sums(row);
             }
         }
-        // (the other panel was last read before the barrier at the end of the last round)
+        // (the other panel was last read before the barrier that ended the loop before)
         if (next > 0) stage.put(next, panel + (cur ^ 1) * psz);
         if (kRows) fqi::cp_async_commit();
         __syncthreads();
